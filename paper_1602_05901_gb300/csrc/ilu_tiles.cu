@@ -3,45 +3,50 @@
 // The forward sweep y_c = D_c^{-1} (r_c - A_{c,-z} y_{-z} - A_{c,-y} y_{-y} -
 // A_{c,-x} y_{-x}) has the i+j+k wavefront as its dependency structure
 // (Section "Restricted Additive Schwarz Method": L y = b is solved row by
-// row).  Instead of one launch per hyperplane, each warp owns a tile of
-// 8 (j) x 4 (k) pencils and walks along i.  Lane (a, b) handles cell
-// (i = s - a - b, j0 + a, k0 + b) at step s, so the cell's -y and -z
-// neighbours inside the tile were computed by lanes (a-1, b) and (a, b-1) one
-// step earlier and arrive by warp shuffle; the -x neighbour is the lane's own
-// previous result.
+// row); the backward sweep z_c = y_c - D_c^{-1} (A_{c,+x} z_{+x} + A_{c,+y} z_{+y} +
+// A_{c,+z} z_{+z}) is its mirror image.  What bounds a sweep is the chain of
+// nx+ny+nz-2 dependent steps, then (on large grids) HBM, then (FP64) the FP64 pipe: one
+// warp-wide DFMA occupies a quarter of an SM for 63 cycles (76 with all four busy).
 //
-// Everything else a step needs arrives through shared-memory rings filled by
-// TMA bulk copies (cp.async.bulk + mbarrier):
-//   * the factor row of each lane (three off-diagonal blocks and D^{-1}, 36
-//     values, packed at setup in exactly the order the warp reads them) and
-//     the input vector, gathered into the same tile order before the sweep.
-//     These come in groups of GS steps (one mbarrier, two copies per group)
-//     through a ring of NG groups, so a copy is issued NG - 1 groups ahead;
-//   * the values of neighbouring tiles' edge cells, ELA steps ahead.  A tile
-//     publishes the results of its last j-row and last k-layer into small
-//     per-tile edge buffers indexed by the step at which the neighbour will
-//     need them.  The buffers hold a signalling-NaN sentinel until written
-//     (arithmetic never produces one), so a consumer that finds the sentinel
-//     in its staged copy re-reads the value from global memory until it
-//     appears (bounded by a time limit that ends the sweep with
-//     RSV_ETIMEOUT).
+// The factor is packed as C_q = -D_c^{-1} A_{c,q}: three 3x3 blocks per cell and sweep.
+// A step is then y_c = v_c + C_x y_x + C_y y_y + C_z y_z with v = D^{-1} r formed for the
+// whole vector before the sweep (off the chain), and z_c = y_c + C_x z_x + C_y z_y + C_z z_z:
+// 27 multiply-adds on the chain instead of 36 and 6 additions, and 27 + 27 + 9 values per cell
+// and application instead of 36 + 36.
 //
-// A step is written for few instructions on its dependency chain: GS steps are
-// unrolled so every ring offset is a constant, the lead lane's edge copies are
-// predicated instead of branched around (a divergent branch cost waiting tiles
-// more than it saved), the sentinel test is one warp vote, and results leave in
-// 16-byte stores.
+// Instead of one launch per hyperplane, a tile of 8 (j) x 4 (k) pencils walks along x.  Lane
+// (a, b) holds pencil (a, b) counted from the corner the sweep starts at, and visits its
+// cell i at step s = i + a + b (backward: x is counted from the far end too, so both sweeps
+// are the same code on mirrored coordinates).  Its y and z neighbours are the results that lanes
+// (a-1, b) and (a, b-1) left one step earlier in a shared-memory array with a halo; the
+// halo of the tile's low faces comes from the neighbouring tiles through small edge buffers in
+// global memory, indexed by the step at which they are needed.  The buffers hold a
+// signalling-NaN sentinel until written (arithmetic never produces one), so a reader that
+// finds the sentinel re-reads until the value appears; the wait is bounded by a time limit
+// that ends the sweep with RSV_ETIMEOUT.  A published value travels as itself (relaxed stores and
+// loads of words that are checked one by one), so no fence is needed.
 //
-// The backward sweep z_c = y_c - D_c^{-1} (A_{c,+x} z_{+x} + A_{c,+y} z_{+y} +
-// A_{c,+z} z_{+z}) is the mirror image (lane (a, b) visits
-// i = nx-1 - (s - (7-a) - (3-b))).  The forward sweep writes y straight into
-// the tile order the backward sweep reads (at forward step s every lane's
-// cell is visited at backward step S-1-s), so y never exists in natural
-// order; the backward sweep writes z in natural order.
+// A tile is one CTA: compute warps that do nothing but the recurrence, an edge warp that
+// collects the halo values a window of steps at a time, and a data warp that keeps the factor rows and the input
+// vector in a shared-memory ring ahead of them (TMA bulk copies); the two announce their progress by counters.
+//   FP32: one compute warp, all three components of a cell per lane.  A step issues about 60 instructions.
+//   FP64: three, warp e computing component e of all 32 cells, so a step's products occupy
+//   three quarters of an SM for 10 x 63 cycles instead of one for 30 x 63; they exchange results
+//   through the array with one barrier per step.
+// Measured (one apply = gather + two sweeps; one warp per tile with 36 values per cell and every edge read and
+// wait in that warp -> this form):
+//   256x8x4 (a lone tile) FP32 155 -> 78 us; 100x100x50 FP32 363 -> 183 us; 256x256x128 FP32 1034 -> 905 us;
+//   75x61x37 FP64 865 -> 255 us; 128x128x64 FP64 1580 -> 516 us.
+// What is left of an FP32 apply on 100x100x50: 248 steps of 0.13 us and 24 hand-offs of about 1 us (store,
+// L2, poll) per sweep.  Independent FP32 tiles, 4 per SM, stream at 0.83 of the measured HBM rate.  Also measured:
+// factor rows by register loads several steps ahead instead of the ring (a lone tile's step 0.36 us instead
+// of 0.13: loads in flight share six scoreboards, and a wait on one waits for younger loads); one service warp for
+// edges and data (hand-off 3 us); edge windows of 8 and 16 steps (100x100x50: 181 and 219 us against 176) and of 2
+// (229 us); L2 prefetches ahead of the ring (no change).
 //
-// Tiles are processed in order of J+K (backward: reverse order); all warps
-// are co-resident (cooperative launch), and a warp only ever waits for tiles
-// earlier in its order, so the waits cannot form a cycle.
+// Tiles are processed in order of J+K (backward: reverse order); all of a launch's CTAs are
+// co-resident (cooperative launch), and a tile only ever waits for tiles earlier in
+// its order, so the waits cannot form a cycle.
 #include <algorithm>
 
 #include "common.cuh"
@@ -50,68 +55,75 @@ namespace rsv {
 namespace {
 
 constexpr int TJ = 8, TK = 4;
-// Edge ring: NSE stages, neighbour values copied ELA steps ahead.  Each step of
-// look-ahead is a step of lag per tile hand-off on the sweep's critical path, so
-// the copies run one step ahead (measured on 100x100x50, FP32 apply: 379 us with
-// one step, 406 us with two, 462 us with three; per-lane relaxed register loads
-// instead of TMA: 595 us).  The stage a step refills (NSE stages: 4 for FP32, 3 for
-// FP64) was last read NSE - 1 steps earlier, and its values fed that step's
-// results, so those reads are complete and the refill needs no proxy fence (a
-// fence there waits for the warp's outstanding stores: 5% slower with it).
-constexpr int ELA = 1;
-// Steps per data group, GS (Bits<T>).  A tile's step count is padded to a multiple
-// of GS (the padded steps hold no valid cell), so every group is full and, GS
-// being a multiple of NSE, every edge stage is a constant of the unrolled step.
-// FP64 takes three steps per group: 64.5 KB per tile, 3 tiles per SM instead of 2
-// (FP64 CPR solve on 256x256x128: 8.71 s against 9.58 s).  FP32 keeps four: three
-// would fit 7 tiles per SM instead of 5, but the apply on 256x256x128 then took
-// 1.081 ms against 1.061 ms (the wavefront, not residency, bounds it).
+constexpr int kTailRows = 16;  // rows behind the last tile's: the edge windows read past a tile's end
 
 template <typename T> struct Bits;
 template <> struct Bits<double> {
     using U = unsigned long long;
     static constexpr U SENT = 0xFFF4C0DE5A17E7A1ull;  // signalling NaN
-    static constexpr int NQP = 38;                    // padded factor row: conflict-free 16-byte reads
-    static constexpr int NG = 2;                      // data ring groups (copies one group ahead)
-    static constexpr int GS = 3, NSE = 3;             // steps per data group, edge stages
+    static constexpr int GS = 1;                      // steps per data group
+    static constexpr int WIN = 2;                     // steps per edge window
+    static constexpr int RD = 4;                      // steps of results kept (ring of halo'd arrays)
+    static constexpr int MIN_NG = 3, MAX_NG = 8;      // groups in the data ring
 };
 template <> struct Bits<float> {
     using U = unsigned int;
     static constexpr U SENT = 0x7FA5C0DEu;
-    static constexpr int NQP = 36;
-    static constexpr int NG = 2;
-    static constexpr int GS = 4, NSE = 4;
+    static constexpr int GS = 2;
+    static constexpr int WIN = 4;
+    static constexpr int RD = 16;
+    static constexpr int MIN_NG = 3, MAX_NG = 8;
 };
 
-// Data stage of one step: factor [32][NQP] and vector [32][4]; a data group holds
-// the factor of its GS steps, then their vectors (two contiguous copies).
-// Edge stage: edge j [TK][4] | edge k [TJ][4].
-template <typename T> struct Stage {
-    static constexpr int F = 32 * Bits<T>::NQP;
+// Packed arrays, per step row of a tile:
+//   FP32  factor [7][32] float4 (lane's 27 values and a zero), input [32] float4 (value x 3, pad),
+//         edges [TK] and [TJ] float4;
+//   FP64  factor [3 components][4][32] double2 | [32] double (component e's 9 values), input
+//         [4][32] (three components, pad), edges [3][TK] and [3][TJ];
+//   both  D^{-1} [9][32] for the transform of the input.
+// The pad carries CPR-PF's pressure correction from the input to the output.
+template <typename T> struct Row {
+    static constexpr int F = sizeof(T) == 4 ? 7 * 32 * 4 : 27 * 32;
     static constexpr int V = 32 * 4;
-    static constexpr int EJ = TK * 4;
-    static constexpr int EK = TJ * 4;
-    static constexpr int GS = Bits<T>::GS, NSE = Bits<T>::NSE;
-    static_assert(GS % NSE == 0 && ELA >= 1 && ELA < NSE, "edge stages are fixed per unrolled step");
-    static constexpr int GSIZE = GS * (F + V);
-    static constexpr int ESIZE = EJ + EK;
-    static constexpr unsigned FB = F * sizeof(T), VB = V * sizeof(T), EJB = EJ * sizeof(T), EKB = EK * sizeof(T);
+    static constexpr int EJ = sizeof(T) == 4 ? TK * 4 : TK * 3;
+    static constexpr int EK = sizeof(T) == 4 ? TJ * 4 : TJ * 3;
+    static constexpr int D = 9 * 32;
 };
 
-template <typename T> constexpr size_t sweep_smem() {
-    return (size_t)(Bits<T>::NG * Stage<T>::GSIZE + Bits<T>::NSE * Stage<T>::ESIZE) * sizeof(T) +
-           (Bits<T>::NG + Bits<T>::NSE) * sizeof(uint64_t);
+// Results of one step with their halo: position (b + 1) kHaloW + a + 1; FP32 float4 entries, FP64
+// one plane per component.
+constexpr int kHaloW = TJ + 1;
+constexpr int kHalo = kHaloW * (TK + 1);
+template <typename T> constexpr int kSlot = (sizeof(T) == 4 ? 4 : 3) * kHalo;  // values per step
+
+struct Control {      // shared between the warps of a CTA
+    int ready;        // steps whose halo is complete
+    int loaded;       // steps whose data have landed (one more than the tile's steps once all have)
+    int steps;        // steps the compute warps have finished
+    int abort;
+};
+
+// Shared memory: data ring [NG][GS][F | V ... as factor of GS steps, then their inputs] | result ring | control | barriers
+template <typename T> constexpr size_t group_bytes() { return (size_t)Bits<T>::GS * (Row<T>::F + Row<T>::V) * sizeof(T); }
+template <typename T> constexpr size_t fixed_bytes() {
+    return (size_t)Bits<T>::RD * kSlot<T> * sizeof(T) + sizeof(Control) + Bits<T>::MAX_NG * sizeof(uint64_t);
 }
+template <typename T> constexpr size_t sweep_smem(int ng) { return ng * group_bytes<T>() + fixed_bytes<T>(); }
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+__device__ __forceinline__ uint64_t global_timer() {
+    uint64_t t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
 }
-__device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect(uint64_t *bar, unsigned bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+__device__ __forceinline__ bool mbar_test(uint64_t *bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 __device__ __forceinline__ void tma_load_1d(void *dst, const void *src, unsigned bytes, uint64_t *bar) {
     asm volatile(
@@ -119,460 +131,684 @@ __device__ __forceinline__ void tma_load_1d(void *dst, const void *src, unsigned
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
         : "memory");
 }
-// Edge rows of one step into an edge stage, by the lanes whose `go` is set (the
-// lead lane): the byte count, then the j row and/or the k row.  Predicated, so
-// the warp takes no branch around it.
-__device__ __forceinline__ void edge_issue(unsigned go, unsigned goj, unsigned gok, uint64_t *bar, unsigned bytes,
-                                           void *dj, const void *sj, unsigned bj, void *dk, const void *sk,
-                                           unsigned bk) {
-    asm volatile(
-        "{\n .reg .pred p, pj, pk;\n"
-        " setp.ne.u32 p, %0, 0;\n setp.ne.u32 pj, %1, 0;\n setp.ne.u32 pk, %2, 0;\n"
-        " @p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%3], %4;\n"
-        " @pj cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%5], [%6], %7, [%3];\n"
-        " @pk cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%8], [%9], %10, [%3];\n}" ::"r"(go),
-        "r"(goj), "r"(gok), "r"(smem_u32(bar)), "r"(bytes), "r"(smem_u32(dj)), "l"(sj), "r"(bj), "r"(smem_u32(dk)),
-        "l"(sk), "r"(bk)
-        : "memory");
+// Control words: the writer's earlier shared-memory accesses are done when a reader sees the new value.
+__device__ __forceinline__ int ld_acquire(const int *p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, unsigned parity) {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
+__device__ __forceinline__ void st_release(int *p, int v) {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
-__device__ __forceinline__ uint64_t global_timer() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
+__device__ __forceinline__ int ld_volatile(const int *p) { return *(volatile const int *)p; }
+__device__ __forceinline__ void st_volatile(int *p, int v) { *(volatile int *)p = v; }
+// Shared-memory accesses that stay in program order (volatile): the results of a step travel between the
+// lanes of one warp as a store followed by loads, and the look-ahead loads have their place behind them.
+__device__ __forceinline__ float4 lds4(unsigned p) {
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(p));
+    return v;
+}
+__device__ __forceinline__ double2 lds2d(unsigned p) {
+    double2 v;
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(p));
+    return v;
+}
+__device__ __forceinline__ double ldsd(unsigned p) {
+    double v;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(p));
+    return v;
+}
+__device__ __forceinline__ void sts4(unsigned p, float x, float y, float z) {
+    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p), "f"(x), "f"(y), "f"(z), "f"(0.f));
+}
+__device__ __forceinline__ void stsd(unsigned p, double x) { asm volatile("st.shared.f64 [%0], %1;" ::"r"(p), "d"(x)); }
+// Predicated stores: a branch around a store costs the step more than the store.
+__device__ __forceinline__ void st_if(bool on, float4 *p, float x, float y, float z, float w) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n @q st.global.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"l"(p),
+                 "f"(x), "f"(y), "f"(z), "f"(w), "r"((unsigned)on));
+}
+__device__ __forceinline__ void st_if(bool on, float *p, float x) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.global.f32 [%0], %1;\n}" ::"l"(p), "f"(x), "r"((unsigned)on));
+}
+__device__ __forceinline__ void st_if(bool on, double *p, double x) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.global.f64 [%0], %1;\n}" ::"l"(p), "d"(x), "r"((unsigned)on));
+}
+__device__ __forceinline__ void st_relaxed_if(bool on, float4 *p, float x, float y, float z) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %5, 0;\n @q st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};\n}" ::"l"(p),
+                 "f"(x), "f"(y), "f"(z), "f"(0.f), "r"((unsigned)on));
+}
+__device__ __forceinline__ void st_relaxed_if(bool on, double *p, double x) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.relaxed.gpu.global.f64 [%0], %1;\n}" ::"l"(p), "d"(x), "r"((unsigned)on));
+}
+// Two FMAs in one instruction: (a.x b.x + c.x, a.y b.y + c.y).
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n .reg .b64 a, b, c, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mov.b64 c, {%6, %7};\n"
+        " fma.rn.f32x2 d, a, b, c;\n mov.b64 {%0, %1}, d;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n .reg .b64 a, b, d;\n mov.b64 a, {%2, %3};\n mov.b64 b, {%4, %5};\n mul.rn.f32x2 d, a, b;\n"
+        " mov.b64 {%0, %1}, d;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 lo(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi(const float4 &v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float4 ld_relaxed(const float4 *p) {
+    float4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_relaxed(const double *p) {
+    double v;
+    asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ bool is_sent(double v) {
+    return (unsigned long long)__double_as_longlong(v) == Bits<double>::SENT;
+}
+__device__ __forceinline__ bool is_sent(const float4 &v) {
+    return __float_as_uint(v.x) == Bits<float>::SENT || __float_as_uint(v.y) == Bits<float>::SENT ||
+           __float_as_uint(v.z) == Bits<float>::SENT;
 }
 
-__device__ __forceinline__ unsigned long long ld_relaxed(const double *p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ unsigned ld_relaxed(const float *p) {
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-// A cell's three results (and a zero pad) as one 16-byte edge-buffer entry.
-__device__ __forceinline__ void st_relaxed3(float *p, const float v[3]) {
-    asm volatile("st.relaxed.gpu.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
-                 "f"(0.f)
-                 : "memory");
-}
-__device__ __forceinline__ void st_relaxed3(double *p, const double v[3]) {
-    asm volatile("st.relaxed.gpu.global.v2.f64 [%0], {%1, %2};" ::"l"(p), "d"(v[0]), "d"(v[1]) : "memory");
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p + 2), "l"(__double_as_longlong(v[2])) : "memory");
-}
-__device__ __forceinline__ unsigned long long bits_of(double v) { return (unsigned long long)__double_as_longlong(v); }
-__device__ __forceinline__ unsigned bits_of(float v) { return __float_as_uint(v); }
-__device__ __forceinline__ double value_of(unsigned long long v) { return __longlong_as_double((long long)v); }
-__device__ __forceinline__ float value_of(unsigned v) { return __uint_as_float(v); }
-template <typename T> __device__ __forceinline__ bool is_sent3(const T v[3]) {
-    return bits_of(v[0]) == Bits<T>::SENT || bits_of(v[1]) == Bits<T>::SENT || bits_of(v[2]) == Bits<T>::SENT;
-}
-// Three values of a 16-byte-aligned shared-memory entry.
-__device__ __forceinline__ void lds3(const float *p, float v[3]) {
-    const float4 q = *reinterpret_cast<const float4 *>(p);
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = q.z;
-}
-__device__ __forceinline__ void lds3(const double *p, double v[3]) {
-    const double2 q = *reinterpret_cast<const double2 *>(p);
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = p[2];
-}
-// A tile-order vector entry: three values and the pad slot.
-__device__ __forceinline__ void lds4(const float *p, float v[3], float &pad) {
-    const float4 q = *reinterpret_cast<const float4 *>(p);
-    v[0] = q.x;
-    v[1] = q.y;
-    v[2] = q.z;
-    pad = q.w;
-}
-__device__ __forceinline__ void lds4(const double *p, double v[3], double &pad) {
-    const double2 q0 = reinterpret_cast<const double2 *>(p)[0], q1 = reinterpret_cast<const double2 *>(p)[1];
-    v[0] = q0.x;
-    v[1] = q0.y;
-    v[2] = q1.x;
-    pad = q1.y;
-}
-// y entry of the backward sweep's tile order (value, value, value, pad).
-__device__ __forceinline__ void st3pad(float *p, const float v[3], float pad) {
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], pad);
-}
-__device__ __forceinline__ void st3pad(double *p, const double v[3], double pad) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], pad);
-}
+// One halo entry (a cell's three values) on its way from an edge buffer to the result ring.
+template <typename T> struct Entry;
+template <> struct Entry<float> {
+    float4 v;
+    __device__ __forceinline__ void load(const float *g, int) { v = ld_relaxed(reinterpret_cast<const float4 *>(g)); }
+    __device__ __forceinline__ bool missing() const { return is_sent(v); }
+    __device__ __forceinline__ void put_if(bool on, float *slot, int pos) const {
+        asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %4, 0;\n @q st.shared.v4.f32 [%0], {%1, %2, %3, %3};\n}" ::"r"(
+                         smem_u32(slot) + pos * 16),
+                     "f"(v.x), "f"(v.y), "f"(v.z), "r"((unsigned)on));
+    }
+};
+template <> struct Entry<double> {
+    double v[3];
+    __device__ __forceinline__ void load(const double *g, int plane) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] = ld_relaxed(g + c * plane);
+    }
+    __device__ __forceinline__ bool missing() const { return is_sent(v[0]) || is_sent(v[1]) || is_sent(v[2]); }
+    __device__ __forceinline__ void put_if(bool on, double *slot, int pos) const {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.shared.f64 [%0], %1;\n}" ::"r"(
+                             smem_u32(slot) + (c * kHalo + pos) * 8),
+                         "d"(v[c]), "r"((unsigned)on));
+    }
+};
 
 template <typename T>
 struct SweepArgs {
-    int nT;                    // tiles of all grids
+    int nT, NG;                // tiles of all grids; groups in the data ring
     const TileSys *tsys;       // per grid
     const int *tile_sys;       // position -> grid
     const int64_t *tile_row0;  // position -> first step row of the tile in the packed arrays
     const int2 *order;         // position -> tile (J, K) inside its grid
     const int *pos_of;         // grid's poff + J * nTK + K -> position
-    const T *F;          // factor rows [nT][Sp][32][NQP]
-    const T *V;          // input vector in tile order [nT][Sp][32][4]
-    T *Vnext;            // forward: y in backward tile order [nT][Sp][32][4]; backward: null
+    const T *F;          // factor rows
+    const T *V;          // input vector in tile order
+    T *Vnext;            // forward: y in the backward sweep's tile order; backward: null
     T *z;                // backward: output in natural order; forward: null
-    T *EJ, *EK;          // edge buffers this sweep publishes [nT][Sp][TK][4], [nT][Sp][TJ][4]
-    T *EJnext, *EKnext;  // forward: the backward sweep's edge buffers (reset to the sentinel)
+    T *EJ, *EK;          // edge buffers this sweep publishes and reads
+    int has_add;         // the pads hold a correction
     const int *done;
     int *status;
     unsigned long long timeout_ns;
 };
 
+// A tile of a sweep, seen from the corner the sweep starts at.
+struct Tile {
+    int nx, Sp, S;
+    int pj, pk;          // positions of the tiles before this one in j and k (-1: none)
+    int64_t row0, rowj, rowk;
+    int64_t cell;        // this lane's pencil: its first cell visited is at cell, the next at cell +- 1
+    bool jk_ok;          // the pencil exists
+};
 template <typename T, bool FWD>
-__global__ void __launch_bounds__(32) ilu_sweep_tiles(SweepArgs<T> P) {
-    using St = Stage<T>;
-    using U = typename Bits<T>::U;
-    constexpr int NQP = Bits<T>::NQP;
-    constexpr int NG = Bits<T>::NG;
-    constexpr int GS = Bits<T>::GS, NSE = Bits<T>::NSE;
-    // (No pdl_trigger here: letting the next kernel's CTAs be scheduled beside the sweep slowed the
-    // FP32 apply on 256x256x128 from 1.034 to 1.069 ms.)
-    if (P.done && *(volatile const int *)P.done) return;
-    extern __shared__ __align__(128) unsigned char smem[];
-    T *ring = reinterpret_cast<T *>(smem);                                   // NG data groups
-    T *ering = ring + NG * St::GSIZE;                                        // NSE edge stages
-    uint64_t *bars = reinterpret_cast<uint64_t *>(ering + NSE * St::ESIZE);  // NG data + NSE edge barriers
-    uint64_t *ebars = bars + NG;
-    const int lane = threadIdx.x;
-    const int a = lane & 7, b = lane >> 3;
-    const unsigned lead = lane == 0;
-    if (lead) {
-        for (int q = 0; q < NG + NSE; ++q) mbar_init(&bars[q], 1);
-        fence_barrier_init();
-    }
-    __syncwarp();
-    unsigned phase = 0, pending = 0;  // bit q: data group stage q; bit NG + q: edge stage q
-    const uint64_t deadline = global_timer() + P.timeout_ns;
+__device__ __forceinline__ Tile tile_of(const SweepArgs<T> &P, int t, int a, int b) {
+    const int tt = FWD ? t : (P.nT - 1 - t);
+    const TileSys G = P.tsys[P.tile_sys[tt]];
+    const int2 JK = P.order[tt];
+    Tile r;
+    r.nx = G.nx;
+    r.S = G.S;
+    r.Sp = G.Sp;
+    const int dj = FWD ? -1 : 1;
+    const int J = JK.x + dj, K = JK.y + dj;
+    r.pj = J >= 0 && J < G.nTJ ? P.pos_of[G.poff + J * G.nTK + JK.y] : -1;
+    r.pk = K >= 0 && K < G.nTK ? P.pos_of[G.poff + JK.x * G.nTK + K] : -1;
+    r.row0 = P.tile_row0[tt];
+    r.rowj = r.pj >= 0 ? P.tile_row0[r.pj] : 0;
+    r.rowk = r.pk >= 0 ? P.tile_row0[r.pk] : 0;
+    const int j = JK.x * TJ + (FWD ? a : TJ - 1 - a), k = JK.y * TK + (FWD ? b : TK - 1 - b);
+    r.jk_ok = j < G.ny && k < G.nz;
+    r.cell = G.cell0 + ((int64_t)k * G.ny + j) * G.nx + (FWD ? 0 : G.nx - 1);
+    return r;
+}
+
+// The data warp of a tile (one lane): keeps the ring of data groups full and announces the steps that have
+// landed.  group0: groups the ring has carried before this tile.  When a wait runs out, or another
+// warp gave up, it raises ctl->abort; it returns with no copy in flight.
+template <typename T>
+__device__ void feed_tile(const SweepArgs<T> &P, const Tile &tl, T *ring, Control *ctl, uint64_t *full, int group0,
+                          uint64_t deadline) {
+    using R = Row<T>;
+    using B = Bits<T>;
+    constexpr int GSIZE = B::GS * (R::F + R::V);
+    const int ngr = tl.Sp / B::GS;
+    const T *Fp = P.F + tl.row0 * R::F, *Vp = P.V + tl.row0 * R::V;
+    int issued = 0, landed = 0;
+    int si = group0 % P.NG, sl = si;  // ring stages of the next group to issue and to land
+    unsigned parity = (group0 / P.NG) & 1, spins = 0;
+    uint64_t limit = deadline;
     bool failed = false;
-
-    auto wait_bar = [&](uint64_t *bar, int bit) {
-        unsigned spins = 0;
-        while (!mbar_try_wait(bar, (phase >> bit) & 1u)) {
-            if ((++spins & 1023u) == 0 && global_timer() > deadline) {
+    while (landed < (failed ? issued : ngr)) {
+        if (!failed && issued < ngr && (issued - P.NG + 1) * B::GS <= ld_acquire(&ctl->steps)) {
+            T *dst = ring + (size_t)si * GSIZE;
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&full[si])),
+                         "r"((unsigned)(GSIZE * sizeof(T)))
+                         : "memory");
+            tma_load_1d(dst, Fp, B::GS * R::F * sizeof(T), &full[si]);
+            tma_load_1d(dst + B::GS * R::F, Vp, B::GS * R::V * sizeof(T), &full[si]);
+            Fp += B::GS * R::F;
+            Vp += B::GS * R::V;
+            if (++si == P.NG) si = 0;
+            ++issued;
+            spins = 0;
+        }
+        if (landed < issued && mbar_test(&full[sl], parity)) {
+            if (++sl == P.NG) {
+                sl = 0;
+                parity ^= 1u;
+            }
+            ++landed;
+            st_release(&ctl->loaded, landed == ngr ? tl.Sp + 1 : landed * B::GS);
+            spins = 0;
+        } else if ((++spins & 63u) == 0) {
+            if (failed) {
+                if (global_timer() > limit) break;
+            } else if (ld_acquire(&ctl->abort) || global_timer() > deadline) {
                 failed = true;
-                return;
+                st_release(&ctl->abort, 1);
+                limit = global_timer() + 1000000000ull;  // copies in flight land first (bounded)
             }
         }
-        phase ^= 1u << bit;
-        pending &= ~(1u << bit);
-    };
-
-    for (int t = blockIdx.x; t < P.nT && !failed; t += gridDim.x) {
-        const int tt = FWD ? t : (P.nT - 1 - t);
-        const TileSys G = P.tsys[P.tile_sys[tt]];
-        const int nx = G.nx, ny = G.ny, nz = G.nz, S = G.S, Sp = G.Sp, nTJ = G.nTJ, nTK = G.nTK;
-        const int ngr = Sp / GS;
-        const int2 JK = P.order[tt];
-        // producers of this tile's edge inputs (same grid)
-        const int pj = FWD ? (JK.x > 0 ? P.pos_of[G.poff + (JK.x - 1) * nTK + JK.y] : -1)
-                           : (JK.x + 1 < nTJ ? P.pos_of[G.poff + (JK.x + 1) * nTK + JK.y] : -1);
-        const int pk = FWD ? (JK.y > 0 ? P.pos_of[G.poff + JK.x * nTK + JK.y - 1] : -1)
-                           : (JK.y + 1 < nTK ? P.pos_of[G.poff + JK.x * nTK + JK.y + 1] : -1);
-        const int j = JK.x * TJ + a, k = JK.y * TK + b;
-        const bool jk_ok = (j < ny) && (k < nz);
-        // Lanes on the tile's lower j (k) face take that neighbour from the edge stage,
-        // which holds zeros where the tile has no producer; inner lanes take it from the
-        // adjacent lane, whose previous result is zero where it held no cell.
-        const bool edge_j = FWD ? (a == 0) : (a == TJ - 1);
-        const bool edge_k = FWD ? (b == 0) : (b == TK - 1);
-        const bool pub_j = FWD ? (a == TJ - 1) : (a == 0);  // this lane's results feed the next tile in j
-        const bool pub_k = FWD ? (b == TK - 1) : (b == 0);
-        const int lane_j = (FWD ? lane - 1 : lane + 1) & 31;
-        const int lane_k = (FWD ? lane - 8 : lane + 8) & 31;
-        const int off = FWD ? (a + b) : ((TJ - 1 - a) + (TK - 1 - b));
-        const int64_t base = G.cell0 + (int64_t)k * nx * ny + (int64_t)j * nx;
-        const size_t tile0 = (size_t)P.tile_row0[tt];
-        const size_t rowj = pj >= 0 ? (size_t)P.tile_row0[pj] : 0, rowk = pk >= 0 ? (size_t)P.tile_row0[pk] : 0;
-        const T *Ft = P.F + tile0 * St::F;
-        const T *Vt = P.V + tile0 * St::V;
-        const bool edges = pj >= 0 || pk >= 0;
-        const unsigned edge_bytes = (pj >= 0 ? St::EJB : 0u) + (pk >= 0 ? St::EKB : 0u);
-        __syncwarp();  // the previous tile's reads of the rings are done
-        if (FWD) {
-            // this tile's backward-sweep edge buffers start at the sentinel
-            U *ej = reinterpret_cast<U *>(P.EJnext + tile0 * St::EJ);
-            U *ek = reinterpret_cast<U *>(P.EKnext + tile0 * St::EK);
-            for (int q = lane; q < Sp * St::EJ; q += 32) ej[q] = Bits<T>::SENT;
-            for (int q = lane; q < Sp * St::EK; q += 32) ek[q] = Bits<T>::SENT;
-        }
-        // faces without a producer read zeros from the edge stages (no copy writes them)
-        if (pj < 0)
-            for (int q = lane; q < NSE * St::EJ; q += 32) ering[(q / St::EJ) * St::ESIZE + q % St::EJ] = T(0);
-        if (pk < 0)
-            for (int q = lane; q < NSE * St::EK; q += 32) ering[(q / St::EK) * St::ESIZE + St::EJ + q % St::EK] = T(0);
-        __syncwarp();
-        if (lead) {
-            fence_proxy_async();
-            for (int q = 0; q < NG - 1 && q < ngr; ++q) {
-                T *dst = ring + q * St::GSIZE;
-                mbar_expect(&bars[q], GS * (St::FB + St::VB));
-                tma_load_1d(dst, Ft + (size_t)q * GS * St::F, GS * St::FB, &bars[q]);
-                tma_load_1d(dst + GS * St::F, Vt + (size_t)q * GS * St::V, GS * St::VB, &bars[q]);
-                pending |= 1u << q;
-            }
-            if (edges)
-                for (int q = 0; q < ELA && q < Sp; ++q) {
-                    T *dst = ering + q * St::ESIZE;
-                    mbar_expect(&ebars[q], edge_bytes);
-                    if (pj >= 0) tma_load_1d(dst, P.EJ + (rowj + q) * St::EJ, St::EJB, &ebars[q]);
-                    if (pk >= 0) tma_load_1d(dst + St::EJ, P.EK + (rowk + q) * St::EK, St::EKB, &ebars[q]);
-                    pending |= 1u << (NG + q);
-                }
-        }
-        T prev[3] = {T(0), T(0), T(0)};
-        int i = FWD ? -off : (nx - 1 + off);  // this lane's cell along x at the current step
-        // Per-group running addresses; a step adds a constant offset to each.
-        T *yout = FWD ? P.Vnext + ((tile0 + (S - 1)) * 32 + lane) * 4 : P.z + 3 * (base + i);
-        constexpr ptrdiff_t ystep = FWD ? -(ptrdiff_t)(32 * 4) : -3;
-        T *pubj = P.EJ + ((ptrdiff_t)tile0 - (TJ - 1)) * St::EJ + b * 4;  // row of step s - (TJ - 1)
-        T *pubk = P.EK + ((ptrdiff_t)tile0 - (TK - 1)) * St::EK + a * 4;
-        const T *pollj = P.EJ + rowj * St::EJ + b * 4;  // the j producer's row of step s
-        const T *pollk = P.EK + rowk * St::EK + a * 4;
-        const T *ejsrc = P.EJ + (rowj + ELA) * St::EJ;  // edge rows of step s + ELA
-        const T *eksrc = P.EK + (rowk + ELA) * St::EK;
-        const unsigned goj = lead && pj >= 0, gok = lead && pk >= 0, go = goj | gok;
-        int gst = 0;  // data group stage of the current group
-
-        for (int g = 0; g < ngr; ++g) {
-            // refill the stage the previous group used (every lane is past it) with group g + NG - 1
-            __syncwarp();
-            if (lead && g + NG - 1 < ngr) {
-                const int q = gst == 0 ? NG - 1 : gst - 1;
-                T *dst = ring + q * St::GSIZE;
-                fence_proxy_async();
-                mbar_expect(&bars[q], GS * (St::FB + St::VB));
-                tma_load_1d(dst, Ft + (size_t)(g + NG - 1) * GS * St::F, GS * St::FB, &bars[q]);
-                tma_load_1d(dst + GS * St::F, Vt + (size_t)(g + NG - 1) * GS * St::V, GS * St::VB, &bars[q]);
-                pending |= 1u << q;
-            }
-            wait_bar(&bars[gst], gst);
-            const T *grp = ring + gst * St::GSIZE;
-            gst = gst + 1 == NG ? 0 : gst + 1;
-            const bool last = g + 1 == ngr;
-#pragma unroll
-            for (int u = 0; u < GS; ++u) {
-                // refill the edge stage of step s + ELA - NSE (done) with the edge rows of step s + ELA.
-                // (The warp barrier also reconverges the lanes after the sentinel poll: without it
-                // the FP32 apply on 256x256x128 took 1.20 ms against 1.06 ms.)
-                __syncwarp();
-                const int eq = (u + ELA) % NSE;
-                const unsigned more = (u + ELA < GS || !last) && edges;
-                edge_issue(go & more, goj & more, gok & more, &ebars[eq], edge_bytes, ering + eq * St::ESIZE,
-                           ejsrc + u * St::EJ, St::EJB, ering + eq * St::ESIZE + St::EJ, eksrc + u * St::EK, St::EKB);
-                if (lead && more) pending |= 1u << (NG + eq);
-                const bool valid = jk_ok && (unsigned)i < (unsigned)nx;
-                // in-tile neighbours: previous step's results of the adjacent lanes
-                T nj[3], nk[3];
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    nj[e] = __shfl_sync(0xffffffffu, prev[e], lane_j);
-                    nk[e] = __shfl_sync(0xffffffffu, prev[e], lane_k);
-                }
-                // factor row and input of this lane
-                T f[NQP];
-                {
-                    const T *row = grp + u * St::F + lane * NQP;
-                    if (sizeof(T) == 4) {
-#pragma unroll
-                        for (int q = 0; q < 9; ++q) {
-                            const float4 v4 = reinterpret_cast<const float4 *>(row)[q];
-                            f[4 * q] = v4.x;
-                            f[4 * q + 1] = v4.y;
-                            f[4 * q + 2] = v4.z;
-                            f[4 * q + 3] = v4.w;
-                        }
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < 18; ++q) {
-                            const double2 v2 = reinterpret_cast<const double2 *>(row)[q];
-                            f[2 * q] = v2.x;
-                            f[2 * q + 1] = v2.y;
-                        }
-                    }
-                }
-                T vin[3], vpad;  // vpad: the pad slot, carried from the forward input to the output
-                lds4(grp + GS * St::F + u * St::V + lane * 4, vin, vpad);
-                // neighbours from other tiles
-                T ej[3] = {T(0), T(0), T(0)}, ek[3] = {T(0), T(0), T(0)};
-                if (edges) {
-                    wait_bar(&ebars[u % NSE], NG + u % NSE);
-                    const T *estg = ering + (u % NSE) * St::ESIZE;
-                    lds3(estg + b * 4, ej);
-                    lds3(estg + St::EJ + a * 4, ek);
-                    const bool bad = valid && ((edge_j && is_sent3(ej)) || (edge_k && is_sent3(ek)));
-                    if (__any_sync(0xffffffffu, bad) && bad) {
-                        // not yet published when the copy ran: re-read until it appears
-                        const T *gj = pollj + u * St::EJ, *gk = pollk + u * St::EK;
-                        unsigned spins = 0;
-                        for (;;) {
-                            const bool mj = edge_j && is_sent3(ej), mk = edge_k && is_sent3(ek);
-                            if (!mj && !mk) break;
-                            if (mj)
-                                for (int e = 0; e < 3; ++e) ej[e] = value_of(ld_relaxed(gj + e));
-                            if (mk)
-                                for (int e = 0; e < 3; ++e) ek[e] = value_of(ld_relaxed(gk + e));
-                            if ((++spins & 63u) == 0 && global_timer() > deadline) {
-                                failed = true;
-                                break;
-                            }
-                        }
-                    }
-                }
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    nj[e] = edge_j ? ej[e] : nj[e];
-                    nk[e] = edge_k ? ek[e] : nk[e];
-                }
-                // slots: forward [0] -z [1] -y [2] -x ; backward [0] +x [1] +y [2] +z
-                const T *x0 = FWD ? nk : prev;
-                const T *x2 = FWD ? prev : nk;
-                T acc[3];
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    T p0 = f[3 * e] * x0[0];
-                    T p1 = f[9 + 3 * e] * nj[0];
-                    T p2 = f[18 + 3 * e] * x2[0];
-                    p0 = fma(f[3 * e + 1], x0[1], p0);
-                    p1 = fma(f[9 + 3 * e + 1], nj[1], p1);
-                    p2 = fma(f[18 + 3 * e + 1], x2[1], p2);
-                    p0 = fma(f[3 * e + 2], x0[2], p0);
-                    p1 = fma(f[9 + 3 * e + 2], nj[2], p1);
-                    p2 = fma(f[18 + 3 * e + 2], x2[2], p2);
-                    const T sum = (p0 + p1) + p2;
-                    acc[e] = FWD ? (vin[e] - sum) : sum;
-                }
-                T res[3];
-#pragma unroll
-                for (int e = 0; e < 3; ++e) {
-                    const T d = fma(f[27 + 3 * e + 2], acc[2], fma(f[27 + 3 * e + 1], acc[1], f[27 + 3 * e] * acc[0]));
-                    res[e] = FWD ? d : (vin[e] - d);
-                }
-                if (valid) {
-                    if (FWD) {
-                        st3pad(yout + u * ystep, res, vpad);
-                    } else {
-                        T *zo = yout + u * ystep;
-                        zo[0] = res[0] + vpad;
-                        zo[1] = res[1];
-                        zo[2] = res[2];
-                    }
-                    if (pub_j) st_relaxed3(pubj + u * St::EJ, res);
-                    if (pub_k) st_relaxed3(pubk + u * St::EK, res);
-                }
-                i += FWD ? 1 : -1;
-#pragma unroll
-                for (int e = 0; e < 3; ++e) prev[e] = valid ? res[e] : T(0);
-            }
-            yout += GS * ystep;
-            pubj += GS * St::EJ;
-            pubk += GS * St::EK;
-            pollj += GS * St::EJ;
-            pollk += GS * St::EK;
-            ejsrc += GS * St::EJ;
-            eksrc += GS * St::EK;
-            if (__any_sync(0xffffffffu, failed)) {
-                failed = true;
-                break;
-            }
-        }
-    }
-    if (failed) {
-        if (lead) {
-            atomicCAS(P.status, 0, (int)RSV_ETIMEOUT);
-            // let copies still in flight land before the CTA exits (bounded)
-            const uint64_t limit = global_timer() + 1000000000ull;
-            for (int q = 0; q < NG + NSE; ++q)
-                if (pending & (1u << q))
-                    while (!mbar_try_wait(&bars[q], (phase >> q) & 1u) && global_timer() < limit) {
-                    }
-        }
-        __syncwarp();
     }
 }
 
-// Factor rows in warp-step order.  One thread per (tile, step, lane).  Block
-// values come from `v` (FP64, or the FP32 copy for mixed precision); D^{-1}
-// from the FP64 factor; both are stored as T.
+// The edge warp of a tile: collects the halo of a window of steps from the edge buffers, hands over those that
+// have arrived and announces them.
+template <typename T>
+__device__ void fetch_edges(const SweepArgs<T> &P, const Tile &tl, T *results, Control *ctl, uint64_t deadline) {
+    using R = Row<T>;
+    using B = Bits<T>;
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    // lanes 0..TK-1 collect the j halo, lanes 8..8+TJ-1 the k halo
+    const bool jl = lane < TK, kl = lane >= 8 && lane < 8 + TJ;
+    const int off = jl ? lane : lane - 8;  // the consuming lane's a + b
+    const bool exists = __shfl_sync(ALL, (int)tl.jk_ok, jl ? lane * 8 : (lane - 8) & 31) != 0;
+    const bool on = exists && ((jl && tl.pj >= 0) || (kl && tl.pk >= 0));
+    constexpr int E = sizeof(T) == 4 ? 4 : 1;  // values per entry in a buffer row
+    const T *g = jl ? P.EJ + tl.rowj * R::EJ + off * E : P.EK + tl.rowk * R::EK + off * E;
+    const int rstep = jl ? R::EJ : R::EK, plane = jl ? TK : TJ;
+    const int hp = jl ? (off + 1) * kHaloW : off + 1;  // halo position
+    int q0 = 0;
+    unsigned spins = 0;
+    while (q0 < tl.Sp) {
+        const int room = ld_volatile(&ctl->steps) + B::RD;  // the halo of step q goes to the slot of step q - 1, last read at step q - RD
+        Entry<T> en[B::WIN];
+#pragma unroll
+        for (int w = 0; w < B::WIN; ++w)
+            if (on) en[w].load(g + w * rstep, plane);
+        // leading steps of the window that are complete in every lane (branch-free: this loop's length is most of
+        // what a hand-off costs)
+        int n = 0;
+        bool more = true;
+#pragma unroll
+        for (int w = 0; w < B::WIN; ++w) {
+            more = more && !(on && (unsigned)(q0 + w - off) < (unsigned)tl.nx && en[w].missing());
+            n += more;
+        }
+        n = min(min(__reduce_min_sync(ALL, n), room - q0), tl.Sp - q0);
+#pragma unroll
+        for (int w = 0; w < B::WIN; ++w)
+            en[w].put_if(w < n && on && (unsigned)(q0 + w - off) < (unsigned)tl.nx,
+                         results + ((q0 + w - 1) & (B::RD - 1)) * kSlot<T>, hp);
+        if (n > 0) {
+            __syncwarp();
+            q0 += n;
+            g += n * rstep;
+            if (lane == 0) st_release(&ctl->ready, q0);
+            spins = 0;
+        } else if ((++spins & 7u) == 0 && __any_sync(ALL, ld_acquire(&ctl->abort) != 0 || global_timer() > deadline)) {
+            if (lane == 0) st_release(&ctl->abort, 1);
+            break;
+        }
+    }
+}
+
+// A compute warp's wait for the halo of step s and the data of the step behind it: returns the number of steps
+// that may run, or 0 when the time is up or another warp gave up (the same for the whole warp).
+__device__ __forceinline__ int wait_step(Control *ctl, int s, uint64_t deadline) {
+    unsigned spins = 0;
+    for (;;) {
+        const int n = min(ld_acquire(&ctl->ready), ld_acquire(&ctl->loaded) - 1);
+        if (s < n) return n;
+        if ((++spins & 63u) == 0 && __any_sync(0xffffffffu, ld_acquire(&ctl->abort) != 0 || global_timer() > deadline))
+            return 0;
+    }
+}
+
+// Shared memory of a CTA.
+template <typename T> struct Smem {
+    T *ring, *results;
+    Control *ctl;
+    uint64_t *full;
+    __device__ __forceinline__ Smem(unsigned char *raw, int ng) {
+        ring = reinterpret_cast<T *>(raw);
+        results = ring + (size_t)ng * Bits<T>::GS * (Row<T>::F + Row<T>::V);
+        full = reinterpret_cast<uint64_t *>(results + Bits<T>::RD * kSlot<T>);
+        ctl = reinterpret_cast<Control *>(full + Bits<T>::MAX_NG);
+    }
+    // Once per CTA.
+    __device__ __forceinline__ void init(int ng) const {
+        if (threadIdx.x) return;
+        for (int q = 0; q < ng; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[q])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        ctl->abort = 0;
+    }
+    // Before each tile, by the whole CTA; false when a warp gave up.  Faces without a producer read zeros.
+    __device__ __forceinline__ bool begin(const Tile &tl) const {
+        __syncthreads();  // every warp is done with the previous tile
+        if (ld_volatile(&ctl->abort)) return false;
+        for (int q = threadIdx.x; q < Bits<T>::RD * kSlot<T>; q += blockDim.x) results[q] = T(0);
+        if (threadIdx.x == 0) {
+            ctl->ready = tl.pj < 0 && tl.pk < 0 ? tl.Sp : 0;
+            ctl->loaded = ctl->steps = 0;
+        }
+        __syncthreads();
+        return true;
+    }
+};
+
+// FP32: warp 0 computes, warp 1 fetches the edges, warp 2 the data.
+//
+// The products of a cell's components 0 and 1 of each neighbour are packed FMAs (fma.rn.f32x2): a step takes 9
+// of them and 9 scalar ones.  The factor row is stored in the order the packed operands need (put_row).
+template <bool FWD>
+__global__ void __launch_bounds__(96, 5) ilu_sweep_f32(SweepArgs<float> P) {
+    using R = Row<float>;
+    using B = Bits<float>;
+    constexpr int GSIZE = B::GS * (R::F + R::V);
+    static_assert(B::GS == 2, "the two steps of a group alternate the look-ahead registers");
+    if (P.done && *(volatile const int *)P.done) return;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const Smem<float> sm(smem, P.NG);
+    Control *ctl = sm.ctl;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int a = lane & 7, b = lane >> 3;
+    const uint64_t deadline = global_timer() + P.timeout_ns;
+    sm.init(P.NG);
+    int group0 = 0;  // data groups of the tiles before this one
+    for (int t = blockIdx.x; t < P.nT; t += gridDim.x) {
+        const Tile tl = tile_of<float, FWD>(P, t, a, b);
+        if (!sm.begin(tl)) break;
+        const int ngr = tl.Sp / B::GS;
+        if (warp == 1) {
+            if (tl.pj >= 0 || tl.pk >= 0) fetch_edges<float>(P, tl, sm.results, ctl, deadline);
+        } else if (warp == 2) {
+            if (lane == 0) feed_tile<float>(P, tl, sm.ring, ctl, sm.full, group0, deadline);
+        } else {
+            const unsigned res = smem_u32(sm.results) + ((b + 1) * kHaloW + a + 1) * 16;
+            // this tile's edge entries: a result of step s is needed TJ - 1 (TK - 1) steps earlier in the next tile's count
+            float4 *pubj = reinterpret_cast<float4 *>(P.EJ + (tl.row0 - (TJ - 1)) * R::EJ) + b;
+            float4 *pubk = reinterpret_cast<float4 *>(P.EK + (tl.row0 - (TK - 1)) * R::EK) + a;
+            // forward: y goes to row S - 1 - s of the backward order, where this lane's pencil is lane 31 - lane
+            float4 *yout = FWD ? reinterpret_cast<float4 *>(P.Vnext + (tl.row0 + tl.S - 1) * R::V) + (31 - lane) : nullptr;
+            float *zout = FWD ? nullptr : P.z + 3 * (tl.cell + (a + b));  // cell of step 0 (before the pencil's start)
+            const unsigned nx = tl.jk_ok ? tl.nx : 0;
+            const bool pj = a == TJ - 1, pk = b == TK - 1;
+            int i = -(a + b);  // cells visited so far; in the grid when 0 <= i < nx
+            float2 p01 = make_float2(0.f, 0.f);  // the lane's previous result
+            float p2 = 0.f;
+            float4 f[2][7], v[2];
+            const unsigned ring0 = smem_u32(sm.ring) + lane * 16, ring1 = ring0 + P.NG * GSIZE * 4;
+            unsigned stage = ring0 + (group0 % P.NG) * (GSIZE * 4);
+            auto fetch = [&](float4(&fo)[7], float4 &vo, int u) {
+#pragma unroll
+                for (int q = 0; q < 7; ++q) fo[q] = lds4(stage + (u * 7 + q) * 512);
+                vo = lds4(stage + (B::GS * 7 + u) * 512);
+            };
+            // One step from the results at `in` to those at `out`, its data in f, v.
+            auto step = [&](const float4(&f)[7], const float4 &v, const float4 &J, const float4 &K, unsigned out, int u) {
+                const bool valid = (unsigned)i < nx;
+                const float2 J01 = make_float2(J.x, J.y), K01 = make_float2(K.x, K.y);
+                float2 s0 = mul2(lo(f[0]), p01), s1 = mul2(hi(f[1]), p01), s2 = mul2(lo(f[3]), p01);
+                float r0 = f[4].z * p2, r1 = f[5].y * p2, r2 = f[6].x * p2;
+                s0 = fma2(hi(f[0]), J01, s0);
+                s1 = fma2(lo(f[2]), J01, s1);
+                s2 = fma2(hi(f[3]), J01, s2);
+                r0 = fmaf(f[4].w, J.z, r0);
+                r1 = fmaf(f[5].z, J.z, r1);
+                r2 = fmaf(f[6].y, J.z, r2);
+                s0 = fma2(lo(f[1]), K01, s0);
+                s1 = fma2(hi(f[2]), K01, s1);
+                s2 = fma2(lo(f[4]), K01, s2);
+                r0 = fmaf(f[5].x, K.z, r0);
+                r1 = fmaf(f[5].w, K.z, r1);
+                r2 = fmaf(f[6].z, K.z, r2);
+                // v last: starting the sums from it costs a rounding at its magnitude per product (error of
+                // an apply against 64 bits 9e-8 instead of 6e-8)
+                r0 = v.x + ((r0 + s0.x) + s0.y);
+                r1 = v.y + ((r1 + s1.x) + s1.y);
+                r2 = v.z + ((r2 + s2.x) + s2.y);
+                p01 = make_float2(valid ? r0 : 0.f, valid ? r1 : 0.f);
+                p2 = valid ? r2 : 0.f;
+                sts4(out, p01.x, p01.y, p2);
+                __syncwarp();
+                st_relaxed_if(valid && pj, pubj + u * TK, r0, r1, r2);
+                st_relaxed_if(valid && pk, pubk + u * TJ, r0, r1, r2);
+                if (FWD) {
+                    st_if(valid, yout - u * 32, r0, r1, r2, v.w);
+                } else {
+                    st_if(valid, zout - 3 * u, r0 + v.w);
+                    st_if(valid, zout - 3 * u + 1, r1);
+                    st_if(valid, zout - 3 * u + 2, r2);
+                }
+                ++i;
+            };
+            int n = wait_step(ctl, 0, deadline);
+            if (n) fetch(f[0], v[0], 0);
+            unsigned prev = res + (B::RD - 1) * kHalo * 16;  // results of the step before
+            for (int s = 0; n && s < tl.Sp; s += 2) {
+                const unsigned out = res + (s & (B::RD - 1)) * (kHalo * 16);
+                if (s >= n && !(n = wait_step(ctl, s, deadline))) break;
+                {
+                    const float4 J = lds4(prev - 16), K = lds4(prev - kHaloW * 16);
+                    fetch(f[1], v[1], 1);
+                    step(f[0], v[0], J, K, out, 0);
+                }
+                if (s + 1 >= n && !(n = wait_step(ctl, s + 1, deadline))) break;
+                {
+                    const float4 J = lds4(out - 16), K = lds4(out - kHaloW * 16);
+                    stage += GSIZE * 4;
+                    if (stage == ring1) stage = ring0;
+                    fetch(f[0], v[0], 0);  // behind the tile's last group: a stale stage, unused
+                    prev = out + kHalo * 16;
+                    step(f[1], v[1], J, K, prev, 1);
+                }
+                if (lane == 0) st_volatile(&ctl->steps, s + 2);  // the group's values are in registers and used
+                pubj += 2 * TK;
+                pubk += 2 * TJ;
+                if (FWD)
+                    yout -= 2 * 32;
+                else
+                    zout -= 6;
+            }
+            if (!n && lane == 0) st_release(&ctl->abort, 1);
+        }
+        group0 += ngr;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && ld_volatile(&ctl->abort)) atomicCAS(P.status, 0, (int)RSV_ETIMEOUT);
+}
+
+// FP64: three compute warps, one per component; the edge warp on the fourth quarter of the SM; the data warp.
+template <bool FWD>
+__global__ void __launch_bounds__(160) ilu_sweep_f64(SweepArgs<double> P) {
+    using R = Row<double>;
+    using B = Bits<double>;
+    constexpr int GSIZE = R::F + R::V;
+    static_assert(B::GS == 1, "a data group is one step");
+    if (P.done && *(volatile const int *)P.done) return;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const Smem<double> sm(smem, P.NG);
+    Control *ctl = sm.ctl;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // component (3: edges, 4: data); which quarter of the SM has none differs between CTAs that share an SM
+    const int e = warp < 4 ? (warp + blockIdx.x / 152) & 3 : 4;
+    const int a = lane & 7, b = lane >> 3;
+    const uint64_t deadline = global_timer() + P.timeout_ns;
+    sm.init(P.NG);
+    int group0 = 0;
+    for (int t = blockIdx.x; t < P.nT; t += gridDim.x) {
+        const Tile tl = tile_of<double, FWD>(P, t, a, b);
+        if (!sm.begin(tl)) break;
+        if (e == 3) {
+            if (tl.pj >= 0 || tl.pk >= 0) fetch_edges<double>(P, tl, sm.results, ctl, deadline);
+        } else if (e == 4) {
+            if (lane == 0) feed_tile<double>(P, tl, sm.ring, ctl, sm.full, group0, deadline);
+        } else {
+            const unsigned res = smem_u32(sm.results) + ((b + 1) * kHaloW + a + 1) * 8;
+            double *pubj = P.EJ + (tl.row0 - (TJ - 1)) * R::EJ + e * TK + b;
+            double *pubk = P.EK + (tl.row0 - (TK - 1)) * R::EK + e * TJ + a;
+            double *yout = FWD ? P.Vnext + (tl.row0 + tl.S - 1) * R::V + (31 - lane) : nullptr;
+            double *zout = FWD ? nullptr : P.z + 3 * (tl.cell + (a + b)) + e;
+            const unsigned nx = tl.jk_ok ? tl.nx : 0;
+            const bool pj = a == TJ - 1, pk = b == TK - 1;
+            const bool pads = P.has_add && e == 0;  // warp 0 carries the pads
+            int i = -(a + b);
+            double2 f[2][4];
+            double f8[2], v[2], pad[2] = {0.0, 0.0};
+            double zlate = 0.0;  // backward, warp 0 with pads: the step before's z_c[0] + p_c, stored one step late
+            bool late = false;
+            const unsigned ring0 = smem_u32(sm.ring), ring1 = ring0 + P.NG * GSIZE * 8;
+            unsigned stage = ring0 + (group0 % P.NG) * (GSIZE * 8);
+            auto fetch = [&](int u) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) f[u][q] = lds2d(stage + e * 2304 + q * 512 + lane * 16);
+                f8[u] = ldsd(stage + e * 2304 + 2048 + lane * 8);
+                v[u] = ldsd(stage + R::F * 8 + e * 256 + lane * 8);
+                if (pads) pad[u] = ldsd(stage + R::F * 8 + 768 + lane * 8);
+            };
+            int n = wait_step(ctl, 0, deadline);
+            bool ok = n > 0, stop = false;
+            fetch(0);
+            unsigned prev = res + (B::RD - 1) * kSlot<double> * 8;
+            for (int s0 = 0; !stop && s0 < tl.Sp; s0 += 2) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int s = s0 + u;
+                    if (s >= n && ok) {
+                        n = wait_step(ctl, s, deadline);
+                        ok = n > 0;
+                    }
+                    const unsigned out = res + (s & (B::RD - 1)) * (kSlot<double> * 8);
+                    // the other two components' own results, then the neighbours'
+                    double x[9];
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) x[c] = ldsd(prev + c * (kHalo * 8));
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) x[3 + c] = ldsd(prev + c * (kHalo * 8) - 8);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) x[6 + c] = ldsd(prev + c * (kHalo * 8) - kHaloW * 8);
+                    stage += GSIZE * 8;
+                    if (stage == ring1) stage = ring0;
+                    fetch(u ^ 1);
+                    const bool valid = (unsigned)i < nx;
+                    double r = f[u][0].x * x[0];
+                    r = fma(f[u][0].y, x[1], r);
+                    r = fma(f[u][1].x, x[2], r);
+                    r = fma(f[u][1].y, x[3], r);
+                    r = fma(f[u][2].x, x[4], r);
+                    r = fma(f[u][2].y, x[5], r);
+                    r = fma(f[u][3].x, x[6], r);
+                    r = fma(f[u][3].y, x[7], r);
+                    r = v[u] + fma(f8[u], x[8], r);  // v last: as in FP32
+                    if (!FWD) st_if(late, zout + 3, zlate);
+                    stsd(out + e * (kHalo * 8), valid ? r : 0.0);
+                    st_relaxed_if(valid && pj, pubj, r);
+                    st_relaxed_if(valid && pk, pubk, r);
+                    if (u == 0) {
+                        asm volatile("barrier.cta.sync 1, 96;" ::: "memory");
+                    } else {
+                        // also: did any warp's wait run out in these two steps
+                        unsigned any;
+                        asm volatile(
+                            "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, 96, p;\n"
+                            " selp.u32 %0, 1, 0, q;\n}"
+                            : "=r"(any)
+                            : "r"((unsigned)!ok)
+                            : "memory");
+                        stop = any != 0;
+                    }
+                    if (e == 0 && lane == 0) st_volatile(&ctl->steps, s + 1);  // every warp is past the step
+                    if (FWD) {
+                        st_if(valid, yout + e * 32, r);
+                        if (pads) st_if(valid, yout + 96, pad[u]);
+                        yout -= R::V;
+                    } else {
+                        st_if(valid && !pads, zout, r);
+                        if (pads) {
+                            late = valid;
+                            zlate = r + pad[u];
+                        }
+                        zout -= 3;
+                    }
+                    ++i;
+                    pubj += R::EJ;
+                    pubk += R::EK;
+                    prev = out;
+                }
+            }
+            if (!FWD) st_if(late && !stop, zout + 3, zlate);
+            if (stop && lane == 0) st_release(&ctl->abort, 1);
+        }
+        group0 += tl.Sp;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && ld_volatile(&ctl->abort)) atomicCAS(P.status, 0, (int)RSV_ETIMEOUT);
+}
+
+// Storage of a cell's factor row: value n = 9 e + 3 q + f is C_q[e][f], q = 0 (x), 1 (y), 2 (z).  FP32: the
+// pairs f = 0, 1 of (e, q) = (0, 0), (0, 1), ..., (2, 2), then f = 2 of the same.
+__device__ __forceinline__ void put_row(float *F, int64_t row, int lane, const double c[27]) {
+    float w[28];
+#pragma unroll
+    for (int n = 0; n < 9; ++n) {
+        w[2 * n] = (float)c[3 * n];
+        w[2 * n + 1] = (float)c[3 * n + 1];
+        w[18 + n] = (float)c[3 * n + 2];
+    }
+    w[27] = 0.f;
+    float4 *o = reinterpret_cast<float4 *>(F + row * Row<float>::F) + lane;
+#pragma unroll
+    for (int q = 0; q < 7; ++q) o[q * 32] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+}
+__device__ __forceinline__ void put_row(double *F, int64_t row, int lane, const double c[27]) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        double *o = F + row * Row<double>::F + e * 288;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            reinterpret_cast<double2 *>(o)[q * 32 + lane] = make_double2(c[9 * e + 2 * q], c[9 * e + 2 * q + 1]);
+        o[256 + lane] = c[9 * e + 8];
+    }
+}
+
+// The packed factor of both sweeps and D^{-1} in tile order.  One thread per (tile, step, lane) of the
+// forward order; its cell sits at step S - 1 - s, lane 31 - lane of the backward order.  Block values come
+// from `v` (FP64, or the FP32 copy for mixed precision), D^{-1} from the FP64 factor; the products are FP64
+// and rounded once.  Entries without a cell are never read as values.
 template <typename T, typename Tv>
-__global__ void pack_tiles(const TileSys *__restrict__ tsys, const int *__restrict__ tile_sys,
+__global__ void __launch_bounds__(256) pack_tiles(const TileSys *__restrict__ tsys, const int *__restrict__ tile_sys,
                            const int64_t *__restrict__ tile_row0, const int2 *__restrict__ order,
                            const int32_t *__restrict__ rp, const Tv *__restrict__ v,
-                           const double *__restrict__ dinv, T *__restrict__ Ff, T *__restrict__ Fb) {
-    constexpr int NQP = Bits<T>::NQP;
+                           const double *__restrict__ dinv, T *__restrict__ Ff, T *__restrict__ Fb, T *__restrict__ D) {
     const int t = blockIdx.y;
     const TileSys G = tsys[tile_sys[t]];
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (gid >= (int64_t)G.Sp * 32) return;
     const int lane = (int)(gid & 31);
     const int s = (int)(gid >> 5);
     const int a = lane & 7, b = lane >> 3;
     const int2 JK = order[t];
-    const int j = JK.x * TJ + a, k = JK.y * TK + b;
+    const int i = s - a - b, j = JK.x * TJ + a, k = JK.y * TK + b;
+    if (j >= ny || k >= nz || i < 0 || i >= nx) return;
+    const int64_t c = G.cell0 + (int64_t)k * nx * ny + (int64_t)j * nx + i;
+    const int64_t row = tile_row0[t] + s, rowb = tile_row0[t] + (G.S - 1 - s);
+    double d[9];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) d[e] = dinv[9 * c + e];
+#pragma unroll
+    for (int e = 0; e < 9; ++e) D[row * Row<T>::D + e * 32 + lane] = (T)d[e];
+    // blocks of the row: -z, -y, -x, self, +x, +y, +z (absent faces skipped)
+    const bool has[6] = {i > 0, j > 0, k > 0, i < nx - 1, j < ny - 1, k < nz - 1};
+    const int before[6] = {has[2] + has[1], has[2], 0, 1, 1 + has[3], 1 + has[3] + has[4]};
+    const Tv *lo = v + 9 * (int64_t)rp[c], *hi = lo + 9 * (has[0] + has[1] + has[2]);
+#pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
-        const bool fwd = dir == 0;
-        const int i = fwd ? (s - a - b) : (nx - 1 - (s - (TJ - 1 - a) - (TK - 1 - b)));
-        T *out = (fwd ? Ff : Fb) + (((size_t)tile_row0[t] + s) * 32 + lane) * NQP;
-        const bool valid = j < ny && k < nz && i >= 0 && i < nx;
-        for (int q = 0; q < NQP; ++q) out[q] = T(0);
-        if (!valid) continue;
-        const int64_t c = G.cell0 + (int64_t)k * nx * ny + (int64_t)j * nx + i;
-        // slots of the row: -z, -y, -x, self, +x, +y, +z (absent faces skipped)
-        int q = 0, mz = -1, my = -1, mx = -1, px = -1, py = -1, pz = -1;
-        if (k > 0) mz = q++;
-        if (j > 0) my = q++;
-        if (i > 0) mx = q++;
-        q++;
-        if (i < nx - 1) px = q++;
-        if (j < ny - 1) py = q++;
-        if (k < nz - 1) pz = q++;
-        const int sl[3] = {fwd ? mz : px, fwd ? my : py, fwd ? mx : pz};
-        for (int blk = 0; blk < 3; ++blk)
-            if (sl[blk] >= 0)
-                for (int e = 0; e < 9; ++e) out[blk * 9 + e] = (T)v[9 * ((int64_t)rp[c] + sl[blk]) + e];
-        for (int e = 0; e < 9; ++e) out[27 + e] = (T)dinv[9 * c + e];
+        double o[27];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const int n = 3 * dir + q;
+            double A[9];
+            const Tv *blk = (dir == 0 ? lo : hi) + 9 * before[n];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) A[e] = has[n] ? (double)blk[e] : 0.0;
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+#pragma unroll
+                for (int f = 0; f < 3; ++f)
+                    o[9 * e + 3 * q + f] = -(d[3 * e] * A[f] + d[3 * e + 1] * A[3 + f] + d[3 * e + 2] * A[6 + f]);
+        }
+        if (dir == 0)
+            put_row(Ff, row, lane, o);
+        else
+            put_row(Fb, rowb, 31 - lane, o);
     }
 }
 
-// A tile-order vector entry (three values and the pad slot) as 16-byte stores.
-__device__ __forceinline__ void st4(float *p, const float v[4]) {
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+// Tile-order entry of the sweeps' input: three values and the pad.
+__device__ __forceinline__ void put_input(float *V, int64_t row, int lane, const float v[3], float pad, bool) {
+    reinterpret_cast<float4 *>(V + row * Row<float>::V)[lane] = make_float4(v[0], v[1], v[2], pad);
 }
-__device__ __forceinline__ void st4(double *p, const double v[4]) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+__device__ __forceinline__ void put_input(double *V, int64_t row, int lane, const double v[3], double pad, bool has) {
+    double *o = V + row * Row<double>::V + lane;
+    o[0] = v[0];
+    o[32] = v[1];
+    o[64] = v[2];
+    if (has) o[96] = pad;
+}
+// `rows` rows of an edge buffer (per values each) to the sentinel, by one warp in 16-byte stores.
+template <typename T>
+__device__ __forceinline__ void reset_rows(T *E, int64_t row, int rows, int per, int lane) {
+    constexpr int N = 16 / sizeof(T);
+    typename Bits<T>::U w[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) w[q] = Bits<T>::SENT;
+    uint4 *o = reinterpret_cast<uint4 *>(E + row * per);
+    for (int q = lane; q < rows * per / N; q += 32) o[q] = *reinterpret_cast<const uint4 *>(w);
 }
 
-// Before a forward sweep: r into tile order, and the forward edge buffers to
+// Before a forward sweep: v = D^{-1} r in tile order, and the edge buffers of both sweeps to
 // the sentinel.  One thread per (tile, lane) and kGatherSteps consecutive steps:
 // its cells are consecutive along x, and all their loads are issued before the
-// stores (one load per thread left the gather latency-bound).  The entry's pad
-// slot takes add[c] (or 0): the forward sweep carries it into y's entry and the
-// backward sweep adds it to the cell's first output component.
+// stores (one load per thread left the gather latency-bound).  The pad
+// takes add[c] (or 0).
 constexpr int kGatherSteps = 4;
 template <typename T>
-__global__ void gather_tiles(const TileSys *__restrict__ tsys, const int *__restrict__ tile_sys,
+__global__ void __launch_bounds__(256) gather_tiles(const TileSys *__restrict__ tsys, const int *__restrict__ tile_sys,
                              const int64_t *__restrict__ tile_row0, const int2 *__restrict__ order,
-                             const T *__restrict__ r, const T *__restrict__ add, T *__restrict__ Vt,
-                             T *__restrict__ EJ, T *__restrict__ EK) {
+                             const T *__restrict__ r, const T *__restrict__ add, const T *__restrict__ D,
+                             T *__restrict__ Vt, T *__restrict__ EJf, T *__restrict__ EKf, T *__restrict__ EJb,
+                             T *__restrict__ EKb) {
     pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
     pdl_trigger();
-    using U = typename Bits<T>::U;
+    using R = Row<T>;
     const int t = blockIdx.y;
     const TileSys G = tsys[tile_sys[t]];
     const int nx = G.nx, ny = G.ny, nz = G.nz;
@@ -585,36 +821,52 @@ __global__ void gather_tiles(const TileSys *__restrict__ tsys, const int *__rest
     const int j = JK.x * TJ + a, k = JK.y * TK + b;
     const bool jk_ok = j < ny && k < nz;
     const int64_t pencil = G.cell0 + (int64_t)k * nx * ny + (int64_t)j * nx;
-    T v[kGatherSteps][4];
+    const int64_t row = tile_row0[t] + s0;
+    T x[kGatherSteps][4], d[kGatherSteps][9];
+    bool ok[kGatherSteps];
 #pragma unroll
     for (int u = 0; u < kGatherSteps; ++u) {
         const int i = s0 + u - a - b;
-        v[u][0] = v[u][1] = v[u][2] = v[u][3] = T(0);
-        if (jk_ok && s0 + u < G.Sp && i >= 0 && i < nx) {
+        ok[u] = jk_ok && i >= 0 && i < nx;
+        if (ok[u]) {
             const int64_t c = pencil + i;
-            v[u][0] = r[3 * c];
-            v[u][1] = r[3 * c + 1];
-            v[u][2] = r[3 * c + 2];
-            if (add) v[u][3] = add[c];
+            x[u][0] = r[3 * c];
+            x[u][1] = r[3 * c + 1];
+            x[u][2] = r[3 * c + 2];
+            x[u][3] = add ? add[c] : T(0);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) d[u][e] = D[(row + u) * R::D + e * 32 + lane];
         }
     }
+    const int rows = min(kGatherSteps, G.Sp - s0);
+    reset_rows(EJf, row, rows, R::EJ, lane);
+    reset_rows(EKf, row, rows, R::EK, lane);
+    reset_rows(EJb, row, rows, R::EJ, lane);
+    reset_rows(EKb, row, rows, R::EK, lane);
 #pragma unroll
-    for (int u = 0; u < kGatherSteps; ++u) {
-        if (s0 + u >= G.Sp) break;
-        const size_t row = (size_t)tile_row0[t] + s0 + u;
-        st4(Vt + (row * 32 + lane) * 4, v[u]);
-        // edge buffers [row][TK][4] and [row][TJ][4]: the 32 threads of a (t, s) row
-        // cover its 16 + 32 entries
-        if (lane < TK * 4) reinterpret_cast<U *>(EJ)[row * TK * 4 + lane] = Bits<T>::SENT;
-        reinterpret_cast<U *>(EK)[row * TJ * 4 + lane] = Bits<T>::SENT;
-    }
+    for (int u = 0; u < kGatherSteps; ++u)
+        if (ok[u]) {
+            T v[3];
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+                v[e] = fma(d[u][3 * e + 2], x[u][2], fma(d[u][3 * e + 1], x[u][1], d[u][3 * e] * x[u][0]));
+            put_input(Vt, row + u, lane, v, x[u][3], add != nullptr);
+        }
 }
+
+template <typename T> constexpr const void *sweep_kernel(bool fwd) {
+    if constexpr (sizeof(T) == 4)
+        return fwd ? (const void *)ilu_sweep_f32<true> : (const void *)ilu_sweep_f32<false>;
+    else
+        return fwd ? (const void *)ilu_sweep_f64<true> : (const void *)ilu_sweep_f64<false>;
+}
+template <typename T> constexpr int kSweepThreads = sizeof(T) == 4 ? 96 : 160;
 
 }  // namespace
 
 template <typename T>
 cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
-    using St = Stage<T>;
+    using R = Row<T>;
     cudaError_t e = cudaSuccess;
     if (!Tl->Ff || Tl->elem != (int)sizeof(T)) {
         free_tiles(Tl);
@@ -634,7 +886,7 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
             ts.nTJ = (sg.ny + TJ - 1) / TJ;
             ts.nTK = (sg.nz + TK - 1) / TK;
             ts.S = sg.nx + TJ + TK - 2;
-            ts.Sp = (ts.S + Bits<T>::GS - 1) / Bits<T>::GS * Bits<T>::GS;
+            ts.Sp = (ts.S + 1) / 2 * 2;  // the steps are unrolled by two
             ts.cell0 = sg.cell0;
             ts.poff = (int)order.size();
             maxS = std::max(maxS, ts.Sp);
@@ -657,17 +909,19 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
         Tl->maxS = maxS;
         Tl->rows = rows;
         Tl->elem = (int)sizeof(T);
+        const size_t all = (size_t)(rows + kTailRows) * sizeof(T);
         auto alloc = [&](void **p, size_t bytes) {
             if (e == cudaSuccess) e = cudaMalloc(p, std::max<size_t>(bytes, 16));
         };
-        alloc(&Tl->Ff, rows * St::FB);
-        alloc(&Tl->Fb, rows * St::FB);
-        alloc(&Tl->Vf, rows * St::VB);
-        alloc(&Tl->Vb, rows * St::VB);
-        alloc(&Tl->EJf, rows * St::EJB);
-        alloc(&Tl->EKf, rows * St::EKB);
-        alloc(&Tl->EJb, rows * St::EJB);
-        alloc(&Tl->EKb, rows * St::EKB);
+        alloc(&Tl->Ff, all * R::F);
+        alloc(&Tl->Fb, all * R::F);
+        alloc(&Tl->D, all * R::D);
+        alloc(&Tl->Vf, all * R::V);
+        alloc(&Tl->Vb, all * R::V);
+        alloc(&Tl->EJf, all * R::EJ);
+        alloc(&Tl->EKf, all * R::EK);
+        alloc(&Tl->EJb, all * R::EJ);
+        alloc(&Tl->EKb, all * R::EK);
         alloc((void **)&Tl->order, sizeof(int2) * nT);
         alloc((void **)&Tl->pos_of, sizeof(int) * nT);
         alloc((void **)&Tl->tile_sys, sizeof(int) * nT);
@@ -686,40 +940,42 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
                                  A->stream)) != cudaSuccess ||
             (e = cudaStreamSynchronize(A->stream)) != cudaSuccess)
             return e;
-        int dev = 0, sms = 0, per_f = 0, per_b = 0;
+        int dev = 0, sms = 0, most = 0, per_f = 0, per_b = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const size_t smem = sweep_smem<T>();
-        if ((e = cudaFuncSetAttribute((const void *)ilu_sweep_tiles<T, true>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute((const void *)ilu_sweep_tiles<T, false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute((const void *)ilu_sweep_tiles<T, true>,
-                                      cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute((const void *)ilu_sweep_tiles<T, false>,
-                                      cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess)
-            return e;
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_f, ilu_sweep_tiles<T, true>, 32, smem)) !=
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+        // Groups in the data ring: as many as leave room for every tile to be resident, at most MAX_NG (a
+        // deeper ring hides more of the memory latency from a lone tile), at least MIN_NG.
+        const int want = std::max(1, (nT + sms - 1) / sms);  // tiles per SM
+        const int64_t room = (int64_t)most / want - 1024 - (int64_t)fixed_bytes<T>();
+        Tl->ng = (int)std::max<int64_t>(Bits<T>::MIN_NG, std::min<int64_t>(Bits<T>::MAX_NG, room / (int64_t)group_bytes<T>()));
+        const size_t smem = Tl->smem = sweep_smem<T>(Tl->ng);
+        for (bool fwd : {true, false})
+            if ((e = cudaFuncSetAttribute(sweep_kernel<T>(fwd), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)sweep_smem<T>(Bits<T>::MAX_NG))) != cudaSuccess ||
+                (e = cudaFuncSetAttribute(sweep_kernel<T>(fwd), cudaFuncAttributePreferredSharedMemoryCarveout,
+                                          100)) != cudaSuccess)
+                return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_f, sweep_kernel<T>(true), kSweepThreads<T>, smem)) !=
                 cudaSuccess ||
-            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_b, ilu_sweep_tiles<T, false>, 32, smem)) !=
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_b, sweep_kernel<T>(false), kSweepThreads<T>, smem)) !=
                 cudaSuccess)
             return e;
         Tl->grid = std::max(1, std::min(nT, sms * std::min(per_f, per_b)));
-        Tl->smem = smem;
     }
     const dim3 g((unsigned)((Tl->maxS * 32 + 255) / 256), (unsigned)Tl->nT);
     rsv::count_launches(1);
     if (sizeof(T) == 8)
         pack_tiles<T, double><<<g, 256, 0, A->stream>>>(Tl->tsys, Tl->tile_sys, Tl->tile_row0, Tl->order, A->d_rp,
-                                                        A->d_v, dinv, (T *)Tl->Ff, (T *)Tl->Fb);
+                                                        A->d_v, dinv, (T *)Tl->Ff, (T *)Tl->Fb, (T *)Tl->D);
     else
         pack_tiles<T, float><<<g, 256, 0, A->stream>>>(Tl->tsys, Tl->tile_sys, Tl->tile_row0, Tl->order, A->d_rp,
-                                                       A->d_v32, dinv, (T *)Tl->Ff, (T *)Tl->Fb);
+                                                       A->d_v32, dinv, (T *)Tl->Ff, (T *)Tl->Fb, (T *)Tl->D);
     return cudaGetLastError();
 }
 
 void free_tiles(IluTiles *Tl) {
-    for (void *p : {Tl->Ff, Tl->Fb, Tl->Vf, Tl->Vb, Tl->EJf, Tl->EKf, Tl->EJb, Tl->EKb, (void *)Tl->order,
+    for (void *p : {Tl->Ff, Tl->Fb, Tl->D, Tl->Vf, Tl->Vb, Tl->EJf, Tl->EKf, Tl->EJb, Tl->EKb, (void *)Tl->order,
                     (void *)Tl->pos_of, (void *)Tl->tile_sys, (void *)Tl->tile_row0, (void *)Tl->tsys})
         if (p) cudaFree(p);
     *Tl = IluTiles();
@@ -732,20 +988,20 @@ cudaError_t launch_ilu_apply_tiles(const rsv_mat *A, const IluTiles &Tl, const T
     const int groups = (Tl.maxS + kGatherSteps - 1) / kGatherSteps;
     const dim3 g((unsigned)((groups * 32 + 255) / 256), (unsigned)Tl.nT);
     cudaError_t e = launch_pdl(gather_tiles<T>, g, dim3(256), 0, A->stream, Tl.tsys, Tl.tile_sys, Tl.tile_row0,
-                               Tl.order, r, add0, (T *)Tl.Vf, (T *)Tl.EJf, (T *)Tl.EKf);
+                               Tl.order, r, add0, (const T *)Tl.D, (T *)Tl.Vf, (T *)Tl.EJf, (T *)Tl.EKf, (T *)Tl.EJb,
+                               (T *)Tl.EKb);
     if (e != cudaSuccess) return e;
-    SweepArgs<T> f{Tl.nT, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Ff,
-                   (const T *)Tl.Vf, (T *)Tl.Vb, nullptr, (T *)Tl.EJf, (T *)Tl.EKf, (T *)Tl.EJb, (T *)Tl.EKb,
-                   done, status, timeout_ns};
-    SweepArgs<T> bw{Tl.nT, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Fb,
-                    (const T *)Tl.Vb, nullptr, z, (T *)Tl.EJb, (T *)Tl.EKb, nullptr, nullptr,
-                    done, status, timeout_ns};
+    const int has_add = add0 != nullptr;
+    SweepArgs<T> f{Tl.nT, Tl.ng, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Ff,
+                   (const T *)Tl.Vf, (T *)Tl.Vb, nullptr, (T *)Tl.EJf, (T *)Tl.EKf, has_add, done, status, timeout_ns};
+    SweepArgs<T> bw{Tl.nT, Tl.ng, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Fb,
+                    (const T *)Tl.Vb, nullptr, z, (T *)Tl.EJb, (T *)Tl.EKb, has_add, done, status, timeout_ns};
     void *fa[] = {&f};
     void *ba[] = {&bw};
-    e = cudaLaunchCooperativeKernel((const void *)ilu_sweep_tiles<T, true>, dim3(Tl.grid), dim3(32), fa, Tl.smem,
+    e = cudaLaunchCooperativeKernel(sweep_kernel<T>(true), dim3(Tl.grid), dim3(kSweepThreads<T>), fa, Tl.smem,
                                     A->stream);
     if (e != cudaSuccess) return e;
-    return cudaLaunchCooperativeKernel((const void *)ilu_sweep_tiles<T, false>, dim3(Tl.grid), dim3(32), ba, Tl.smem,
+    return cudaLaunchCooperativeKernel(sweep_kernel<T>(false), dim3(Tl.grid), dim3(kSweepThreads<T>), ba, Tl.smem,
                                        A->stream);
 }
 
