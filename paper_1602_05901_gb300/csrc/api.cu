@@ -224,9 +224,13 @@ rsv_status rsv_mat_get_pattern(const rsv_mat *A, const int32_t **row_ptr, const 
 rsv_status rsv_mat_set_values(rsv_mat *A, const double *vals, int on_device) {
     if (!A || !vals) return RSV_EINVAL;
     const size_t bytes = sizeof(double) * 9 * (size_t)A->nnzb;
-    RSV_CUDA_TRY(cudaMemcpyAsync(A->d_v, vals, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                                 A->stream));
-    if (A->d_v32) RSV_CUDA_TRY(launch_cast_f64_f32(A->stream, 9 * A->nnzb, A->d_v, A->d_v32));
+    if (on_device && A->d_v32) {
+        RSV_CUDA_TRY(launch_copy_cast(A->stream, 9 * A->nnzb, vals, A->d_v, A->d_v32));
+    } else {
+        RSV_CUDA_TRY(cudaMemcpyAsync(A->d_v, vals, bytes,
+                                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, A->stream));
+        if (A->d_v32) RSV_CUDA_TRY(launch_cast_f64_f32(A->stream, 9 * A->nnzb, A->d_v, A->d_v32));
+    }
     RSV_CUDA_TRY(spmv_autotune(A));  // first values only: time the SpMV tile candidates on this pattern
     if (!on_device) RSV_CUDA_TRY(cudaStreamSynchronize(A->stream));
     A->version++;

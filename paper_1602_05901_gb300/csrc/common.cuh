@@ -64,6 +64,25 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     return cudaLaunchKernelEx(&cfg, kern, ((KArgs)args)...);
 }
 
+// float -> double and double -> float (round to nearest even) in integer arithmetic: the conversion instructions
+// run at the FP64 pipe's rate on GB300 (76 cycles per warp; these take about 10).  Zero, subnormal,
+// overflowing, infinite and NaN values take the instruction.
+__device__ __forceinline__ double exact_double(float x) {
+    const unsigned u = __float_as_uint(x);
+    if (((u >> 23) & 255u) - 1u >= 254u) return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double exact_double(double x) { return x; }
+__device__ __forceinline__ float round_float(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    // exponents -125 .. 126: the rounded value is a normal float whichever way it rounds
+    if (((hi >> 20) & 2047u) - 898u >= 252u) return (float)x;
+    const unsigned m = ((hi & 0x7fffffffu) - 0x38000000u) << 3 | lo >> 29;  // truncated float bits
+    const unsigned rest = lo << 3;                                            // dropped bits, left-aligned
+    const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (m & 1u));
+    return __uint_as_float((hi & 0x80000000u) | (m + up));
+}
+
 constexpr int kMaxRestart = 64;
 constexpr int kRedBlocks = 304;   // 2 x 152 SMs: grid of every reduction kernel
 constexpr int kRedThreads = 256;
@@ -137,8 +156,8 @@ struct Cpr {  // CPR pressure stage: quasi-IMPES weights and the GMG hierarchy (
     void *x[kMaxLevels] = {}, *b[kMaxLevels] = {};  // per-level solution and right-hand side (T)
     double *w64 = nullptr;        // quasi-IMPES weights [nb][3], FP64
     void *w = nullptr;            // weights in T
-    double *dense = nullptr, *minv = nullptr, *work = nullptr;  // coarsest LU / inverse / scratch
-    int *piv = nullptr;
+    double *dense = nullptr, *minv = nullptr, *work = nullptr;  // coarsest matrix / inverse / scratch
+    int *piv = nullptr;           // coarsest inverse: row permutations
     void *r = nullptr, *z = nullptr, *xp = nullptr;  // full-stage residual and ILU correction (T)
     void *apc = nullptr;          // pressure column of every block [nnzb][3] (T): CPR-PF's stage-two residual
     void *amg = nullptr;          // algebraic hierarchy (amg.cu) when the pressure stage coarsens algebraically
@@ -203,6 +222,8 @@ cudaError_t launch_spmv_f64(const rsv_mat *A, double alpha, const double *x, dou
 cudaError_t launch_spmv_f32(const rsv_mat *A, float alpha, const float *x, float beta, float *y,
                             const int *done, int *status = nullptr, unsigned long long timeout_ns = 2000000000ull);
 cudaError_t launch_cast_f64_f32(cudaStream_t st, int64_t n, const double *a, float *b);
+// c = a and b = (float)a, one read of a.
+cudaError_t launch_copy_cast(cudaStream_t st, int64_t n, const double *a, double *c, float *b);
 // Time the SpMV's block-rows-per-CTA candidates (32, 64, 128) on A's pattern and keep the
 // fastest per precision; once per matrix (later calls return at once).
 cudaError_t spmv_autotune(rsv_mat *A);

@@ -15,7 +15,7 @@
 //   * smoothing is red-black Gauss-Seidel, colour (i+j+k) mod 2, red then
 //     black before the recursion and black then red after it;
 //   * the coarsest level (at most gmg_max_coarse cells) is solved with its
-//     explicit inverse, computed at setup from a partial-pivoting LU.
+//     explicit inverse, computed at setup by Gauss-Jordan elimination with partial pivoting.
 // Full stage (CPR-PF, two-stage multiplicative): x = Pi_p p; r = f - A x;
 // x = x + ILU0^{-1} r, with Pi_p p = (p_c, 0, 0)_c.
 //
@@ -75,7 +75,7 @@ __global__ void qi_setup_kernel(G3 g, const int32_t *__restrict__ rp, const Tv *
     if (decoupling == 2)  // true-IMPES: the cell's accumulation block instead of A's diagonal block
         for (int q = 0; q < 9; ++q) d[q] = acc[9 * c + q];
     else
-        for (int q = 0; q < 9; ++q) d[q] = (double)dv[q];
+        for (int q = 0; q < 9; ++q) d[q] = exact_double(dv[q]);
     double w0, w1, w2;
     if (decoupling == 1 || decoupling == 2) {
         // ABF / true-IMPES: the first row of D^{-1} = adj(D) / det(D), from the cofactors of D's first column
@@ -105,7 +105,7 @@ __global__ void qi_setup_kernel(G3 g, const int32_t *__restrict__ rp, const Tv *
         double val = 0.0;
         if (has[s]) {
             const Tv *blk = v + 9 * ((int64_t)rp[c] + slot_pos[s]);
-            val = w0 * (double)blk[0] + w1 * (double)blk[3] + w2 * (double)blk[6];
+            val = w0 * exact_double(blk[0]) + w1 * exact_double(blk[3]) + w2 * exact_double(blk[6]);
         }
         a7[(int64_t)s * n + c] = val;
     }
@@ -138,104 +138,212 @@ __global__ void gmg_coarsen_kernel(G3 f, const double *__restrict__ af, G3 cg, d
 
 __global__ void cast_stencil(int64_t n, const double *__restrict__ a, float *__restrict__ b) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        b[i] = (float)a[i];
+        b[i] = round_float(a[i]);
 }
 
-// Dense matrix of the coarsest stencil, row-major n x n.
+// Dense matrix of the coarsest stencil, row-major n x n; M is cleared before.
 __global__ void coarse_dense_kernel(G3 g, const double *__restrict__ a7, double *__restrict__ M) {
     const int64_t n = g.n();
     const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (c >= n) return;
-    for (int64_t q = 0; q < n; ++q) M[c * n + q] = 0.0;
     int i, j, k;
     ijk(c, g, i, j, k);
     for (int s = 0; s < 7; ++s) {
         const int ii = i + kDI[s], jj = j + kDJ[s], kk = k + kDK[s];
         if (ii < 0 || jj < 0 || kk < 0 || ii >= g.nx || jj >= g.ny || kk >= g.nz) continue;
-        M[c * n + (int64_t)kk * g.nx * g.ny + (int64_t)jj * g.nx + ii] += a7[(int64_t)s * n + c];
+        M[c * n + (int64_t)kk * g.nx * g.ny + (int64_t)jj * g.nx + ii] = a7[(int64_t)s * n + c];
     }
 }
 
-// In-place LU with partial pivoting of the n x n matrix M (one CTA), then its
-// inverse into Minv by solving for the unit vectors.  |pivot| <= 1e-300
-// reports RSV_ESINGULAR.
-__global__ void __launch_bounds__(1024) coarse_lu_kernel(int n, double *M, int *piv, int *status) {
-    __shared__ double sval[32];
-    __shared__ int sidx[32];
-    __shared__ int spiv;
-    for (int k = 0; k < n; ++k) {
-        // pivot search in column k (max |M[i][k]|, smallest i on ties)
-        double best = -1.0;
-        int bi = k;
-        for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-            const double a = fabs(M[(int64_t)i * n + k]);
-            if (a > best) { best = a; bi = i; }
+// The coarsest level's inverse by Gauss-Jordan elimination with partial pivoting, kGjB columns (a panel) at a time.
+// FP64 arithmetic bounds it: one SM adds and multiplies 1.7 values per clock, so only the panel's own n x kGjB
+// values stay in one CTA (gj_panel) and the other columns are updated by the whole chip (gj_update).
+// 8x8x4 cells (n = 256): LU and triangular solves by single CTAs took 4.06 + 0.28 ms, this form 0.5 ms.
+constexpr int kGjB = 8;
+constexpr int kGjRows = 1024;  // rows that one thread each of the panel CTA holds in registers
+
+// The largest key of the warp and the smallest row that has it (keys: bits of |value|, which order like the
+// values; integer reductions keep the search off the FP64 pipe).
+__device__ __forceinline__ void warp_largest(unsigned long long &key, int &at) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+    const unsigned long long best = (unsigned long long)hi << 32 | lo;
+    at = (int)__reduce_min_sync(0xffffffffu, key == best ? (unsigned)at : 0x7fffffffu);
+    key = best;
+}
+__device__ __forceinline__ unsigned long long abs_bits(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+}
+
+// One panel: Gauss-Jordan steps k0 .. k0 + kGjB - 1 on its own columns of the n x n matrix A.  Thread i
+// holds row i of the panel in registers.  Q [n][kGjB]: the panel afterwards (rows of the pivot block: its inverse P; other rows:
+// -A_iK P).  perm[i]: the row of A that the panel's pivoting moved to position i.  Largest |pivot| first, the
+// smallest row on ties; |pivot| <= 1e-300 reports RSV_ESINGULAR.
+__global__ void __launch_bounds__(kGjRows) gj_panel(int n, int k0, const double *__restrict__ A, double *__restrict__ Q,
+                                                       int *__restrict__ perm, int *status) {
+    pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
+    pdl_trigger();
+    __shared__ unsigned long long wmax[32];
+    __shared__ double prow[kGjB], krow[kGjB];
+    __shared__ int widx[32], sidx[2];
+    const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = (int)(blockDim.x >> 5);
+    const int nk = min(kGjB, n - k0);
+    double a[kGjB];
+#pragma unroll
+    for (int c = 0; c < kGjB; ++c) a[c] = i < n && c < nk ? A[(int64_t)i * n + k0 + c] : 0.0;
+    int src = i;
+#pragma unroll
+    for (int t = 0; t < kGjB; ++t) {
+        if (t >= nk) break;
+        const int k = k0 + t;
+        const bool in = i >= k && i < n;
+        unsigned long long key = in ? abs_bits(a[t]) : 0ull;
+        int at = in ? i : n;  // n: no candidate, behind every row of the same key
+        warp_largest(key, at);
+        if (lane == 0) {
+            wmax[warp] = key;
+            widx[warp] = at;
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const double ob = __shfl_down_sync(0xffffffffu, best, o);
-            const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-            if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-        }
-        if ((threadIdx.x & 31) == 0) { sval[threadIdx.x >> 5] = best; sidx[threadIdx.x >> 5] = bi; }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = -1.0;
-            int p = k;
-            for (int q = 0; q < (int)(blockDim.x >> 5); ++q)
-                if (sval[q] > b || (sval[q] == b && sidx[q] < p)) { b = sval[q]; p = sidx[q]; }
-            spiv = p;
-            piv[k] = p;
-            if (!(b > 1e-300)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
+        key = lane < nw ? wmax[lane] : 0ull;
+        at = lane < nw ? widx[lane] : n;
+        warp_largest(key, at);
+        const int p = at;
+        if (i == k) {
+#pragma unroll
+            for (int c = 0; c < kGjB; ++c) krow[c] = a[c];
+            sidx[0] = src;
+            if (!(__longlong_as_double((long long)key) > 1e-300)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
+        }
+        if (i == p) {
+            const double ip = 1.0 / a[t];
+#pragma unroll
+            for (int c = 0; c < kGjB; ++c) prow[c] = c == t ? ip : a[c] * ip;
+            sidx[1] = src;
         }
         __syncthreads();
-        const int p = spiv;
-        if (p != k)
-            for (int q = threadIdx.x; q < n; q += blockDim.x) {
-                const double t = M[(int64_t)k * n + q];
-                M[(int64_t)k * n + q] = M[(int64_t)p * n + q];
-                M[(int64_t)p * n + q] = t;
+        if (i == p && p != k) {
+#pragma unroll
+            for (int c = 0; c < kGjB; ++c) a[c] = krow[c];
+            src = sidx[0];
+        }
+        if (i == k) {
+#pragma unroll
+            for (int c = 0; c < kGjB; ++c) a[c] = prow[c];
+            src = sidx[1];
+        } else {
+            const double m = -a[t];
+#pragma unroll
+            for (int c = 0; c < kGjB; ++c) a[c] = c == t ? m * prow[c] : fma(m, prow[c], a[c]);
+        }
+    }
+    if (i < n) {
+#pragma unroll
+        for (int c = 0; c < kGjB; ++c) Q[i * kGjB + c] = a[c];
+        perm[i] = src;
+    }
+}
+
+// The same for more rows than a CTA has threads (few levels on a large grid): the panel lives in Q, the row
+// order in perm.
+__global__ void __launch_bounds__(kGjRows) gj_panel_large(int n, int k0, const double *__restrict__ A, double *Q, int *perm,
+                                                          int *status) {
+    pdl_wait();
+    pdl_trigger();
+    __shared__ unsigned long long wmax[32];
+    __shared__ double prow[kGjB];
+    __shared__ int widx[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nk = min(kGjB, n - k0);
+    for (int i = threadIdx.x; i < n; i += kGjRows) {
+        for (int c = 0; c < kGjB; ++c) Q[(int64_t)i * kGjB + c] = c < nk ? A[(int64_t)i * n + k0 + c] : 0.0;
+        perm[i] = i;
+    }
+    __syncthreads();
+    for (int t = 0; t < nk; ++t) {
+        const int k = k0 + t;
+        unsigned long long key = 0ull;
+        int at = n;
+        for (int i = k + threadIdx.x; i < n; i += kGjRows) {
+            const unsigned long long v = abs_bits(Q[(int64_t)i * kGjB + t]);
+            if (at == n || v > key) {
+                key = v;
+                at = i;
             }
+        }
+        warp_largest(key, at);
+        if (lane == 0) {
+            wmax[warp] = key;
+            widx[warp] = at;
+        }
         __syncthreads();
-        const double pk = M[(int64_t)k * n + k];
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) M[(int64_t)i * n + k] /= pk;
+        key = wmax[lane];
+        at = widx[lane];
+        warp_largest(key, at);
+        const int p = at;
+        if (threadIdx.x == 0 && !(__longlong_as_double((long long)key) > 1e-300)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
+        if (threadIdx.x < kGjB) {  // the pivot row, scaled; its place takes row k
+            const int c = threadIdx.x;
+            const double ip = 1.0 / Q[(int64_t)p * kGjB + t], v = Q[(int64_t)p * kGjB + c];
+            __syncwarp((1u << kGjB) - 1u);
+            if (p != k) Q[(int64_t)p * kGjB + c] = Q[(int64_t)k * kGjB + c];
+            prow[c] = c == t ? ip : v * ip;
+            if (c == 0 && p != k) {
+                const int sp = perm[p];
+                perm[p] = perm[k];
+                perm[k] = sp;
+            }
+        }
         __syncthreads();
-        const int m = n - k - 1;
-        for (int64_t t = threadIdx.x; t < (int64_t)m * m; t += blockDim.x) {
-            const int i = k + 1 + (int)(t / m), q = k + 1 + (int)(t % m);
-            M[(int64_t)i * n + q] -= M[(int64_t)i * n + k] * M[(int64_t)k * n + q];
+        for (int i = threadIdx.x; i < n; i += kGjRows) {
+            double *q = Q + (int64_t)i * kGjB;
+            const double m = -q[t];
+            for (int c = 0; c < kGjB; ++c) q[c] = i == k ? prow[c] : c == t ? m * prow[c] : fma(m, prow[c], q[c]);
         }
         __syncthreads();
     }
 }
 
-// Column j of the inverse: solve (LU) x = P e_j.  One CTA per column.
-__global__ void coarse_inverse_kernel(int n, const double *__restrict__ LU, const int *__restrict__ piv,
-                                      double *__restrict__ Minv, double *__restrict__ work) {
-    const int j = blockIdx.x;
-    double *x = work + (int64_t)j * n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = (i == j) ? 1.0 : 0.0;
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < n; ++k)
-            if (piv[k] != k) {
-                const double t = x[k];
-                x[k] = x[piv[k]];
-                x[piv[k]] = t;
-            }
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {  // unit lower triangle
-        const double xk = x[k];
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) x[i] -= LU[(int64_t)i * n + k] * xk;
-        __syncthreads();
+// The panel's effect on the matrix: B = the panel's columns from Q, every other column j
+// B_ij = (i in the pivot block ? 0 : A_perm(i)j) + sum_t Q_it A_perm(k0 + t)j.  Tracks the row order
+// (order_out = order_in through perm).  The last panel writes column j of B to column order_out(j) of
+// the result: the inverse of the row-permuted matrix, its columns put back.
+__global__ void __launch_bounds__(256) gj_update(int n, int k0, const double *__restrict__ A, const double *__restrict__ Q,
+                                                 const int *__restrict__ perm, const int *__restrict__ order_in,
+                                                 int *__restrict__ order_out, double *__restrict__ B) {
+    pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
+    pdl_trigger();
+    const int j = blockIdx.x * 32 + (threadIdx.x & 31), i = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (i >= n || j >= n) return;
+    const int nk = min(kGjB, n - k0);
+    if (j == 0) order_out[i] = order_in ? order_in[perm[i]] : perm[i];
+    double r;
+    if (j >= k0 && j < k0 + nk) {
+        r = Q[(int64_t)i * kGjB + (j - k0)];
+    } else {
+        r = i >= k0 && i < k0 + nk ? 0.0 : A[(int64_t)perm[i] * n + j];
+#pragma unroll
+        for (int t = 0; t < kGjB; ++t)
+            if (t < nk) r = fma(Q[(int64_t)i * kGjB + t], A[(int64_t)perm[k0 + t] * n + j], r);
     }
-    for (int k = n - 1; k >= 0; --k) {  // upper triangle
-        if (threadIdx.x == 0) x[k] /= LU[(int64_t)k * n + k];
-        __syncthreads();
-        const double xk = x[k];
-        for (int i = threadIdx.x; i < k; i += blockDim.x) x[i] -= LU[(int64_t)i * n + k] * xk;
-        __syncthreads();
+    const bool last = k0 + nk >= n;
+    const int to = !last ? j : order_in ? order_in[perm[j]] : perm[j];
+    B[(int64_t)i * n + to] = r;
+}
+
+// Minv = inverse of the n x n matrix in `dense` (overwritten).  work: n (n + kGjB) doubles; index: 3 n ints.
+cudaError_t coarse_inverse(cudaStream_t st, int n, double *dense, double *work, int *index, double *Minv, int *status) {
+    double *X[2] = {dense, work}, *Q = work + (int64_t)n * n;
+    int *perm = index, *order[2] = {index + n, index + 2 * n};
+    cudaError_t e = cudaSuccess;
+    for (int k0 = 0, q = 0; k0 < n && e == cudaSuccess; k0 += kGjB, q ^= 1) {
+        count_launches(2);
+        e = n <= kGjRows ? launch_pdl(gj_panel, dim3(1), dim3((n + 31) / 32 * 32), 0, st, n, k0, X[q], Q, perm, status)
+                         : launch_pdl(gj_panel_large, dim3(1), dim3(kGjRows), 0, st, n, k0, X[q], Q, perm, status);
+        if (e == cudaSuccess)
+            e = launch_pdl(gj_update, dim3((n + 31) / 32, (n + 7) / 8), dim3(256), 0, st, n, k0, X[q], Q, perm,
+                           k0 ? order[q] : nullptr, order[q ^ 1], k0 + kGjB >= n ? Minv : X[q ^ 1]);
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) Minv[(int64_t)i * n + j] = x[i];
+    return e;
 }
 
 // x = Minv b (one warp per row), b and x in T, arithmetic in FP64.
@@ -572,8 +680,8 @@ cudaError_t cpr_setup(const rsv_mat *A, bool mixed, int max_levels, int max_coar
     const int64_t ncd = coarsening == 1 ? 1 : nc;  // the algebraic hierarchy keeps its own coarsest inverse
     alloc((void **)&P->dense, sizeof(double) * ncd * ncd);
     alloc((void **)&P->minv, sizeof(double) * ncd * ncd);
-    alloc((void **)&P->work, sizeof(double) * ncd * ncd);
-    alloc((void **)&P->piv, sizeof(int) * ncd);
+    alloc((void **)&P->work, sizeof(double) * ncd * (ncd + kGjB));
+    alloc((void **)&P->piv, sizeof(int) * 3 * ncd);
     alloc(&P->r, es * 3 * nb);
     alloc(&P->z, es * 3 * nb);
     alloc(&P->xp, es * 3 * nb);
@@ -594,10 +702,10 @@ cudaError_t cpr_setup(const rsv_mat *A, bool mixed, int max_levels, int max_coar
     }
     if (coarsening != 1) {
         G3 gc{P->dims[nl - 1][0], P->dims[nl - 1][1], P->dims[nl - 1][2]};
-        count_launches(3);
-        coarse_dense_kernel<<<blocks(nc), 256, 0, st>>>(gc, P->a7[nl - 1], P->dense);
-        coarse_lu_kernel<<<1, 1024, 0, st>>>(nc, P->dense, P->piv, status);
-        coarse_inverse_kernel<<<nc, 128, 0, st>>>(nc, P->dense, P->piv, P->minv, P->work);
+        count_launches(1);
+        if ((e = cudaMemsetAsync(P->dense, 0, sizeof(double) * nc * nc, st)) != cudaSuccess) return e;
+        coarse_dense_kernel<<<blocks(nc, 64), 64, 0, st>>>(gc, P->a7[nl - 1], P->dense);
+        if ((e = coarse_inverse(st, nc, P->dense, P->work, P->piv, P->minv, status)) != cudaSuccess) return e;
     }
     const unsigned pcb = (unsigned)std::min<int64_t>(blocks(A->nnzb), 152 * 32);
     count_launches(1);

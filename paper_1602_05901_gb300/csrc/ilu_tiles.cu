@@ -512,9 +512,9 @@ __global__ void __launch_bounds__(96, 5) ilu_sweep_f32(SweepArgs<float> P) {
                 r2 = fmaf(f[6].z, K.z, r2);
                 // v last: starting the sums from it costs a rounding at its magnitude per product (error of
                 // an apply against 64 bits 9e-8 instead of 6e-8)
-                r0 = v.x + ((r0 + s0.x) + s0.y);
-                r1 = v.y + ((r1 + s1.x) + s1.y);
-                r2 = v.z + ((r2 + s2.x) + s2.y);
+                r0 = v.x + ((r0 + s0.y) + s0.x);
+                r1 = v.y + ((r1 + s1.y) + s1.x);
+                r2 = v.z + ((r2 + s2.y) + s2.x);
                 p01 = make_float2(valid ? r0 : 0.f, valid ? r1 : 0.f);
                 p2 = valid ? r2 : 0.f;
                 sts4(out, p01.x, p01.y, p2);
@@ -695,13 +695,13 @@ __global__ void __launch_bounds__(160) ilu_sweep_f64(SweepArgs<double> P) {
 
 // Storage of a cell's factor row: value n = 9 e + 3 q + f is C_q[e][f], q = 0 (x), 1 (y), 2 (z).  FP32: the
 // pairs f = 0, 1 of (e, q) = (0, 0), (0, 1), ..., (2, 2), then f = 2 of the same.
-__device__ __forceinline__ void put_row(float *F, int64_t row, int lane, const double c[27]) {
+__device__ __forceinline__ void put_row(float *F, int64_t row, int lane, const float c[27]) {
     float w[28];
 #pragma unroll
     for (int n = 0; n < 9; ++n) {
-        w[2 * n] = (float)c[3 * n];
-        w[2 * n + 1] = (float)c[3 * n + 1];
-        w[18 + n] = (float)c[3 * n + 2];
+        w[2 * n] = c[3 * n];
+        w[2 * n + 1] = c[3 * n + 1];
+        w[18 + n] = c[3 * n + 2];
     }
     w[27] = 0.f;
     float4 *o = reinterpret_cast<float4 *>(F + row * Row<float>::F) + lane;
@@ -719,14 +719,51 @@ __device__ __forceinline__ void put_row(double *F, int64_t row, int lane, const 
     }
 }
 
+// One entry -sum_m d[m] A[m] of a packed block.  FP64, or rounded to FP32 from a double-float sum: d as two
+// floats (48 bits), exact products and two-sums, about 44 bits before the one rounding; in FP64 the products and
+// conversions are what bounded the packing (128x128x64: 799 us with 36 unmultiplied values, 589 us with
+// FP64 products, 152 us now).
+template <typename T> struct Row3;  // three entries of a row of D^{-1}
+template <> struct Row3<double> {
+    double d[3];
+    __device__ __forceinline__ explicit Row3(const double *p) : d{p[0], p[1], p[2]} {}
+    __device__ __forceinline__ double times(const double *A) const {
+        return -(d[0] * A[0] + d[1] * A[3] + d[2] * A[6]);
+    }
+    __device__ __forceinline__ double at(int m) const { return d[m]; }
+};
+template <> struct Row3<float> {
+    float h[3], l[3];
+    __device__ __forceinline__ explicit Row3(const double *p) {
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            h[m] = round_float(p[m]);
+            l[m] = round_float(p[m] - exact_double(h[m]));
+        }
+    }
+    __device__ __forceinline__ float times(const float *A) const {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+            const float p = __fmul_rn(h[m], A[3 * m]);
+            const float e = __fmaf_rn(l[m], A[3 * m], __fmaf_rn(h[m], A[3 * m], -p));  // h A = p + its rounding; + l A
+            const float s = __fadd_rn(hi, p), bp = __fsub_rn(s, hi);
+            lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(p, bp))));
+            hi = s;
+        }
+        return -__fadd_rn(hi, lo);
+    }
+    __device__ __forceinline__ float at(int m) const { return h[m]; }
+};
+
 // The packed factor of both sweeps and D^{-1} in tile order.  One thread per (tile, step, lane) of the
 // forward order; its cell sits at step S - 1 - s, lane 31 - lane of the backward order.  Block values come
-// from `v` (FP64, or the FP32 copy for mixed precision), D^{-1} from the FP64 factor; the products are FP64
-// and rounded once.  Entries without a cell are never read as values.
-template <typename T, typename Tv>
+// from `v` (FP64, or the FP32 copy for mixed precision), D^{-1} from the FP64 factor.  Entries without a cell
+// are never read as values.
+template <typename T>
 __global__ void __launch_bounds__(256) pack_tiles(const TileSys *__restrict__ tsys, const int *__restrict__ tile_sys,
                            const int64_t *__restrict__ tile_row0, const int2 *__restrict__ order,
-                           const int32_t *__restrict__ rp, const Tv *__restrict__ v,
+                           const int32_t *__restrict__ rp, const T *__restrict__ v,
                            const double *__restrict__ dinv, T *__restrict__ Ff, T *__restrict__ Fb, T *__restrict__ D) {
     const int t = blockIdx.y;
     const TileSys G = tsys[tile_sys[t]];
@@ -740,30 +777,27 @@ __global__ void __launch_bounds__(256) pack_tiles(const TileSys *__restrict__ ts
     if (j >= ny || k >= nz || i < 0 || i >= nx) return;
     const int64_t c = G.cell0 + (int64_t)k * nx * ny + (int64_t)j * nx + i;
     const int64_t row = tile_row0[t] + s, rowb = tile_row0[t] + (G.S - 1 - s);
-    double d[9];
+    const Row3<T> d[3] = {Row3<T>(dinv + 9 * c), Row3<T>(dinv + 9 * c + 3), Row3<T>(dinv + 9 * c + 6)};
 #pragma unroll
-    for (int e = 0; e < 9; ++e) d[e] = dinv[9 * c + e];
-#pragma unroll
-    for (int e = 0; e < 9; ++e) D[row * Row<T>::D + e * 32 + lane] = (T)d[e];
+    for (int e = 0; e < 9; ++e) D[row * Row<T>::D + e * 32 + lane] = d[e / 3].at(e % 3);
     // blocks of the row: -z, -y, -x, self, +x, +y, +z (absent faces skipped)
     const bool has[6] = {i > 0, j > 0, k > 0, i < nx - 1, j < ny - 1, k < nz - 1};
     const int before[6] = {has[2] + has[1], has[2], 0, 1, 1 + has[3], 1 + has[3] + has[4]};
-    const Tv *lo = v + 9 * (int64_t)rp[c], *hi = lo + 9 * (has[0] + has[1] + has[2]);
+    const T *lo = v + 9 * (int64_t)rp[c], *hi = lo + 9 * (has[0] + has[1] + has[2]);
 #pragma unroll
     for (int dir = 0; dir < 2; ++dir) {
-        double o[27];
+        T o[27];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const int n = 3 * dir + q;
-            double A[9];
-            const Tv *blk = (dir == 0 ? lo : hi) + 9 * before[n];
+            T A[9];
+            const T *blk = (dir == 0 ? lo : hi) + 9 * before[n];
 #pragma unroll
-            for (int e = 0; e < 9; ++e) A[e] = has[n] ? (double)blk[e] : 0.0;
+            for (int e = 0; e < 9; ++e) A[e] = has[n] ? blk[e] : T(0);
 #pragma unroll
             for (int e = 0; e < 3; ++e)
 #pragma unroll
-                for (int f = 0; f < 3; ++f)
-                    o[9 * e + 3 * q + f] = -(d[3 * e] * A[f] + d[3 * e + 1] * A[3 + f] + d[3 * e + 2] * A[6 + f]);
+                for (int f = 0; f < 3; ++f) o[9 * e + 3 * q + f] = d[e].times(A + f);
         }
         if (dir == 0)
             put_row(Ff, row, lane, o);
@@ -965,12 +999,9 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
     }
     const dim3 g((unsigned)((Tl->maxS * 32 + 255) / 256), (unsigned)Tl->nT);
     rsv::count_launches(1);
-    if (sizeof(T) == 8)
-        pack_tiles<T, double><<<g, 256, 0, A->stream>>>(Tl->tsys, Tl->tile_sys, Tl->tile_row0, Tl->order, A->d_rp,
-                                                        A->d_v, dinv, (T *)Tl->Ff, (T *)Tl->Fb, (T *)Tl->D);
-    else
-        pack_tiles<T, float><<<g, 256, 0, A->stream>>>(Tl->tsys, Tl->tile_sys, Tl->tile_row0, Tl->order, A->d_rp,
-                                                       A->d_v32, dinv, (T *)Tl->Ff, (T *)Tl->Fb, (T *)Tl->D);
+    const T *v = sizeof(T) == 8 ? (const T *)A->d_v : (const T *)A->d_v32;
+    pack_tiles<T><<<g, 256, 0, A->stream>>>(Tl->tsys, Tl->tile_sys, Tl->tile_row0, Tl->order, A->d_rp, v, dinv,
+                                            (T *)Tl->Ff, (T *)Tl->Fb, (T *)Tl->D);
     return cudaGetLastError();
 }
 

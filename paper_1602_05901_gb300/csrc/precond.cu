@@ -42,14 +42,6 @@ __device__ __forceinline__ bool inv3(const double *a, double *o) {
     return true;
 }
 
-__device__ __forceinline__ void mm3(const double *a, const double *b, double *c) {
-#pragma unroll
-    for (int e = 0; e < 3; ++e)
-#pragma unroll
-        for (int f = 0; f < 3; ++f) c[3 * e + f] = a[3 * e] * b[f] + a[3 * e + 1] * b[3 + f] + a[3 * e + 2] * b[6 + f];
-}
-
-
 // Position of the blocks of row c inside the BSR row (columns ascending:
 // -z, -y, -x, self, +x, +y, +z, absent faces skipped).
 struct RowSlots {
@@ -73,7 +65,7 @@ __device__ __forceinline__ RowSlots row_slots(int c, Dims g) {
 template <typename Tv>
 __device__ __forceinline__ void load9(const Tv *p, double *o) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) o[q] = (double)p[q];
+    for (int q = 0; q < 9; ++q) o[q] = exact_double(p[q]);
 }
 
 // dinv_c = A_cc^{-1} in FP64 from the FP64 values or their FP32 copy; dinv32
@@ -118,41 +110,73 @@ __global__ void bj_apply_kernel(int64_t nb, const T *__restrict__ dinv, const T 
 
 // D_c = A_cc - sum_{l lower} (A_cl D_l^{-1}) A_lc, lower neighbours in
 // ascending column order (-z, -y, -x).
+//
+// One lane per entry of D_c: nine lanes per cell, three cells per warp.  A plane's time is one cell's chain
+// of FP64 operations, each of which occupies an SM quarter for 63 cycles: 34 of them with one entry per lane
+// against 200 with one cell per thread (128x128x64, 318 planes: 17.3 -> 6.2 us per plane).  What does
+// not depend on the plane before (indices, matrix blocks) is loaded before pdl_wait, while that plane runs.
+// Products and sums keep the order of a row-by-column 3x3 product.
+constexpr unsigned kCellLanes = 0x07ffffffu;  // 27 lanes of a warp
+__device__ __forceinline__ double shfl9(double v, int src) { return __shfl_sync(kCellLanes, v, src); }
 template <typename Tv>
-__global__ void ilu_factor_plane(const SysGrid *__restrict__ sys, const int32_t *__restrict__ sys_of_cell,
+__global__ void __launch_bounds__(128) ilu_factor_plane(const SysGrid *__restrict__ sys, const int32_t *__restrict__ sys_of_cell,
                                  const int32_t *__restrict__ rp, const Tv *__restrict__ v,
                                  const int32_t *__restrict__ cells, int p0, int p1, double *dinv, int *status) {
-    pdl_wait();  // launched with launch_pdl: the previous plane may still be running
-    pdl_trigger();
-    const int t = p0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= p1) return;
-    const int c = cells[t];
+    const int lane = threadIdx.x & 31;
+    const int t = p0 + (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 3 + lane / 9;
+    if (lane >= 27) return;
+    const int n = lane % 9, e = n / 3, f = n % 3, first = lane - n, row = first + 3 * e;
+    const bool on = t < p1;
+    const int c = cells[on ? t : p0];
     int local;
     const Dims g = grid_of(c, sys, sys_of_cell, local);
     const RowSlots s = row_slots(local, g);
     const int64_t base = rp[c];
-    double D[9];
-    load9(v + 9 * (base + s.d), D);
     const int lower[3] = {s.mz, s.my, s.mx};
     const int loff[3] = {g.nx * g.ny, g.nx, 1};
+    double D = exact_double(v[9 * (base + s.d) + n]);
+    double acl[3][3], alc[3][3];  // row e of A_cl and column f of A_lc
+#pragma unroll
     for (int q = 0; q < 3; ++q) {
         if (lower[q] < 0) continue;
         const int l = c - loff[q];
         const RowSlots sl = row_slots(local - loff[q], g);
         const int up = (q == 0) ? sl.pz : (q == 1) ? sl.py : sl.px;  // block of row l in column c
-        double Acl[9], Dl[9], Alc[9], T[9], U[9];
-        load9(v + 9 * (base + lower[q]), Acl);
-        load9(dinv + 9 * (int64_t)l, Dl);
-        load9(v + 9 * ((int64_t)rp[l] + up), Alc);
-        mm3(Acl, Dl, T);
-        mm3(T, Alc, U);
+        const Tv *pa = v + 9 * (base + lower[q]) + 3 * e, *pb = v + 9 * ((int64_t)rp[l] + up) + f;
 #pragma unroll
-        for (int e = 0; e < 9; ++e) D[e] -= U[e];
+        for (int m = 0; m < 3; ++m) {
+            acl[q][m] = exact_double(pa[m]);
+            alc[q][m] = exact_double(pb[3 * m]);
+        }
     }
-    if (!inv3(D, dinv + 9 * (int64_t)c)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
+    pdl_wait();  // launched with launch_pdl: the previous plane may still be running
+    pdl_trigger();
+    double dl[3][3];  // column f of D_l^{-1}
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int m = 0; m < 3; ++m) dl[q][m] = lower[q] < 0 ? 0.0 : dinv[9 * (int64_t)(c - loff[q]) + 3 * m + f];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        double T = 0.0;
+        if (lower[q] >= 0) T = fma(acl[q][2], dl[q][2], fma(acl[q][1], dl[q][1], acl[q][0] * dl[q][0]));
+        const double t0 = shfl9(T, row), t1 = shfl9(T, row + 1), t2 = shfl9(T, row + 2);
+        if (lower[q] >= 0) D -= fma(t2, alc[q][2], fma(t1, alc[q][1], t0 * alc[q][0]));
+    }
+    // inverse by cofactors: entry n is (D[i0] D[i1] - D[i2] D[i3]) / det, the i's one hex digit per entry
+    const int i0 = (int)(0x13205124ull >> (4 * n)) & 15, i1 = (int)(0x467386578ull >> (4 * n)) & 15;
+    const int i2 = (int)(0x104023215ull >> (4 * n)) & 15, i3 = (int)(0x376568487ull >> (4 * n)) & 15;
+    const double cof = shfl9(D, first + i0) * shfl9(D, first + i1) - shfl9(D, first + i2) * shfl9(D, first + i3);
+    const double det = shfl9(D, first) * shfl9(cof, first) + shfl9(D, first + 1) * shfl9(cof, first + 3) +
+                       shfl9(D, first + 2) * shfl9(cof, first + 6);
+    if (!on) return;
+    if (fabs(det) > 1e-300)
+        dinv[9 * (int64_t)c + n] = cof * (1.0 / det);
+    else if (n == 0)
+        atomicCAS(status, 0, (int)RSV_ESINGULAR);
 }
 
-constexpr int kPlaneThreads = 128;
+constexpr int kPlaneCells = 12;  // cells of a factor CTA: four warps of three
 
 }  // namespace
 
@@ -211,18 +235,29 @@ template cudaError_t launch_bj_apply<double>(cudaStream_t, int64_t, const double
 template cudaError_t launch_bj_apply<float>(cudaStream_t, int64_t, const float *, const float *, float *,
                                             const int *);
 
-// One launch per hyperplane, each a programmatic dependent of the one before (its launch
-// overlaps the previous plane; it waits for it on the device before reading its factors).
+// One launch per hyperplane.  Each but the first is a programmatic dependent of the one before: it loads
+// the matrix while the previous plane runs and waits for it on the device before reading its factors.  The
+// first is launched the ordinary way, so all of them find the matrix values written.
 cudaError_t launch_ilu_setup(const rsv_mat *A, const Schedule &sch, bool from_f32, double *dinv, int *status) {
     for (int h = 0; h < sch.nplanes; ++h) {
         const int p0 = sch.plane_ptr[h], p1 = sch.plane_ptr[h + 1];
-        const dim3 grid((p1 - p0 + kPlaneThreads - 1) / kPlaneThreads), block(kPlaneThreads);
+        const dim3 grid((p1 - p0 + kPlaneCells - 1) / kPlaneCells), block(128);
         rsv::count_launches(1);
-        const cudaError_t e =
-            from_f32 ? launch_pdl(ilu_factor_plane<float>, grid, block, 0, A->stream, A->d_sys, A->d_sys_of_cell,
-                                  A->d_rp, A->d_v32, sch.cells, p0, p1, dinv, status)
-                     : launch_pdl(ilu_factor_plane<double>, grid, block, 0, A->stream, A->d_sys, A->d_sys_of_cell,
-                                  A->d_rp, A->d_v, sch.cells, p0, p1, dinv, status);
+        cudaError_t e = cudaSuccess;
+        if (h == 0) {
+            if (from_f32)
+                ilu_factor_plane<float><<<grid, block, 0, A->stream>>>(A->d_sys, A->d_sys_of_cell, A->d_rp, A->d_v32,
+                                                                       sch.cells, p0, p1, dinv, status);
+            else
+                ilu_factor_plane<double><<<grid, block, 0, A->stream>>>(A->d_sys, A->d_sys_of_cell, A->d_rp, A->d_v,
+                                                                        sch.cells, p0, p1, dinv, status);
+            e = cudaGetLastError();
+        } else {
+            e = from_f32 ? launch_pdl(ilu_factor_plane<float>, grid, block, 0, A->stream, A->d_sys, A->d_sys_of_cell,
+                                      A->d_rp, A->d_v32, sch.cells, p0, p1, dinv, status)
+                         : launch_pdl(ilu_factor_plane<double>, grid, block, 0, A->stream, A->d_sys, A->d_sys_of_cell,
+                                      A->d_rp, A->d_v, sch.cells, p0, p1, dinv, status);
+        }
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
