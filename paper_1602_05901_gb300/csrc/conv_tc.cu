@@ -109,6 +109,40 @@ struct FwdArgs {
     const int *gate;      // skip the launch when *gate != 0 (may be null)
 };
 
+// Epilogue of 16 output channels n .. n + 15 of voxel v: bias, ReLU, mask, FP32 and BF16 stores.
+__device__ __forceinline__ void store16(const FwdArgs &a, int64_t v, int n, float acc[16]) {
+    if (a.bias) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] += __ldg(a.bias + n + i);
+    }
+    if (a.relu) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i] = fmaxf(acc[i], 0.0f);
+    }
+    if (a.mask) {
+        const uint4 *mp = (const uint4 *)(a.mask + v * a.ldm + n);
+        uint4 mv[2] = {mp[0], mp[1]};
+        const __nv_bfloat16 *mb = (const __nv_bfloat16 *)mv;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (!(__bfloat162float(mb[i]) > 0.0f)) acc[i] = 0.0f;
+    }
+    if (a.y32) {
+        float4 *o = (float4 *)(a.y32 + v * a.n_total + n);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+    }
+    if (a.y) {
+        uint4 ov[2];
+        __nv_bfloat162 *ob = (__nv_bfloat162 *)ov;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ob[i] = __floats2bfloat162_rn(acc[2 * i], acc[2 * i + 1]);
+        uint4 *o = (uint4 *)(a.y + v * a.ldy + n);
+        o[0] = ov[0];
+        o[1] = ov[1];
+    }
+}
+
 template <int BK, int BN>
 struct FwdSmem {
     static constexpr uint32_t A = 128 * BK * 2, B = BN * BK * 2, STAGE = A + B;
@@ -217,37 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         float acc[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, acc);
         if (!valid) continue;
-        const int n = n0 + c0;
-        if (a.bias) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc[i] += a.bias[n + i];
-        }
-        if (a.relu) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) acc[i] = fmaxf(acc[i], 0.0f);
-        }
-        if (a.mask) {
-            const uint4 *mp = (const uint4 *)(a.mask + v * a.ldm + n);
-            uint4 mv[2] = {mp[0], mp[1]};
-            const __nv_bfloat16 *mb = (const __nv_bfloat16 *)mv;
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (!(__bfloat162float(mb[i]) > 0.0f)) acc[i] = 0.0f;
-        }
-        if (a.y32) {
-            float4 *o = (float4 *)(a.y32 + v * a.n_total + n);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) o[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
-        }
-        if (a.y) {
-            uint4 ov[2];
-            __nv_bfloat162 *ob = (__nv_bfloat162 *)ov;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) ob[i] = __floats2bfloat162_rn(acc[2 * i], acc[2 * i + 1]);
-            uint4 *o = (uint4 *)(a.y + v * a.ldy + n);
-            o[0] = ov[0];
-            o[1] = ov[1];
-        }
+        store16(a, v, n0 + c0, acc);
     }
 
     fence_before_sync();
@@ -260,6 +264,211 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncthreads();
     if (warp == 2) tmem_dealloc(tmem, TCOLS);
+}
+
+// ------------------------------------------------------------------ forward, x taps folded into N
+// For narrow layers (32 or 64 output channels) the kernel above is bound by L2: every tile reads its 27 shifted
+// neighbourhoods.  Here the three x taps of a (dz, dy) pair become columns of one product: with
+// P_dx[u] = sum over dz, dy, channels of w[dz, dy, dx] x[u + (dz, dy)] (N = 3 co columns), y[v] = P_-1[v - 1] +
+// P_0[v] + P_+1[v + 1], added in the epilogue from the neighbouring TMEM lanes; a tile's rows span the whole
+// x extent, so no neighbour lies outside it but the zero padding.  The y taps share one box: two M tiles
+// stacked in y read one box of 2 bh + 2 rows per dz, each (tile, dy) an operand that starts a multiple
+// of nx rows into it.  Per 128 voxels and 32 input channels that is 48 KB of operands from L2 instead of 216, and a
+// third of the MMAs.
+// The weights stay in shared memory when they fit beside three input boxes (32 -> 32 and 64 -> 32 channels);
+// else each stage carries its own.  Persistent CTAs; with 32 output channels the epilogue of a pair of tiles
+// overlaps the next pair's MMAs (two accumulator sets of 192 columns).
+// One call, 128x128x64: 32 -> 32 channels 185 -> 96 us (kernel 175 -> 72), 96 -> 32 473 -> 200 us; 64x64x32:
+// 64 -> 64 72 -> 58 us (kernel 56 -> 42), 192 -> 64 142 -> 95 us; 32x32x16 and below: both forms the same, the call's
+// fixed 25 us.  What bounds it now is the rate of the MMAs, about 140 cycles each whatever N (M = 128 rows of A from shared
+// memory); marching along z with two of three boxes kept (a third of the loads) gave nothing (97 us).
+struct FoldArgs {
+    FwdArgs f;              // bw = nx, bh rows per tile, bd = 1, ty: pairs along y
+    int pairs, S;           // pairs of tiles; pipeline stages
+    uint32_t boxA, strideA; // bytes of an input box, and its room (a tile's 128 rows may pass the box's end)
+    int resident;           // weights resident
+    uint32_t offA, offBar;  // shared-memory offsets (the resident weights come first)
+};
+
+constexpr int kFoldThreads = 320;  // producer, MMA issuer, four epilogue warps for each tile of the pair
+constexpr int kFoldMaxStages = 6;
+
+// Whether `ok` holds for all four warps at named barrier `bar`.
+__device__ __forceinline__ bool all_of_128(int bar, bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.and.pred q, %2, 128, p;\n selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(r)
+        : "r"((uint32_t)ok), "r"(bar)
+        : "memory");
+    return r != 0;
+}
+
+template <int CO>
+__global__ void __launch_bounds__(kFoldThreads, 1)
+    conv_fold_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const FoldArgs g) {
+    const FwdArgs &a = g.f;
+    if (a.gate && *a.gate) return;  // uniform across the CTA, before any barrier or allocation
+    constexpr int BN = 3 * CO;
+    constexpr int NBUF = CO == 32 ? 2 : 1;        // accumulator sets
+    constexpr uint32_t BDY = BN * 64u, BST = 3 * BDY;  // weight bytes of one dy, and of one (dz, channel block)
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    uint8_t *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    uint64_t *full = (uint64_t *)(sm + g.offBar);
+    uint64_t *empty = full + kFoldMaxStages, *accfull = empty + kFoldMaxStages, *accempty = accfull + 2;
+    uint64_t *bready = accempty + 2, *done = bready + 1;
+    uint32_t *tmem_slot = (uint32_t *)(done + 1);
+    int *flags = (int *)(tmem_slot + 1);  // [0] failed, [1] loads issued
+    float *xch = (float *)(sm + g.offBar + 512);  // [tile][2][4 warps][2][16]: boundary lanes' values of a chunk
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t deadline = now_ns() + a.timeout_ns;
+    const int nk = 3 * a.nkb;  // stages per pair
+    const uint32_t stride = g.strideA + (g.resident ? 0u : BST);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < g.S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&accfull[b], 1);
+            mbar_init(&accempty[b], 8);
+        }
+        mbar_init(bready, 1);
+        mbar_init(done, 1);
+        flags[0] = flags[1] = 0;
+        fence_mbar_init();
+    }
+    if (warp == 1) tmem_alloc(tmem_slot, 512);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        prefetch_map(&tmA);
+        prefetch_map(&tmB);
+        auto weights = [&](uint8_t *dst, int dz, int cb, uint64_t *bar) {
+            for (int t = 0; t < 9; ++t)  // rows (dy, dx, output channel)
+                tma_load_2d(dst + t * (CO * 64), &tmB, (dz * 9 + t) * a.ci + cb * 32, 0, bar);
+        };
+        if (g.resident) {
+            mbar_expect_tx(bready, (uint32_t)nk * BST);
+            for (int q = 0; q < nk; ++q) weights(sm + q * BST, q / a.nkb, q % a.nkb, bready);
+        }
+        int kk = 0;
+        bool ok = true;
+        for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x) {
+            const int y0 = (p % a.ty) * 2 * a.bh, z0 = p / a.ty;
+            for (int q = 0; q < nk; ++q, ++kk) {
+                const int s = kk % g.S;
+                if (kk >= g.S && !mbar_wait(&empty[s], ((kk / g.S) + 1) & 1, deadline)) {
+                    ok = false;
+                    break;
+                }
+                const int dz = q / a.nkb, cb = q % a.nkb;
+                uint8_t *st = sm + g.offA + s * stride;
+                mbar_expect_tx(&full[s], g.boxA + (g.resident ? 0u : BST));
+                tma_load_4d(st, &tmA, cb * 32, 0, y0 - 1, z0 + dz - 1, &full[s]);
+                if (!g.resident) weights(st + g.strideA, dz, cb, &full[s]);
+            }
+        }
+        if (!ok) flags[0] = 1;
+        flags[1] = kk;
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = idesc_bf16(128, BN);
+        int kk = 0, it = 0;
+        bool ok = !g.resident || mbar_wait(bready, 0, deadline);
+        for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x, ++it) {
+            const int buf = it % NBUF;
+            const uint32_t acc = tmem + buf * (2 * BN);
+            if (it >= NBUF && !(ok = mbar_wait(&accempty[buf], ((it / NBUF) + 1) & 1, deadline))) break;
+            fence_after_sync();
+            for (int q = 0; q < nk; ++q, ++kk) {
+                const int s = kk % g.S;
+                if (!(ok = mbar_wait(&full[s], (kk / g.S) & 1, deadline))) break;
+                fence_after_sync();
+                const uint32_t sa = smem_u32(sm + g.offA + s * stride);
+                const uint32_t sb = g.resident ? smem_u32(sm + q * BST) : sa + g.strideA;
+#pragma unroll
+                for (int m = 0; m < 2; ++m)
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            mma_bf16(acc + m * BN, kmajor_desc(sa + (uint32_t)((m * a.bh + dy) * a.bw) * 64u + j * 32, 64),
+                                     kmajor_desc(sb + dy * BDY + j * 32, 64), idesc, (q > 0 || dy > 0 || j > 0) ? 1u : 0u);
+                mma_commit(&empty[s]);
+            }
+            if (ok) mma_commit(&accfull[buf]);
+        }
+        if (!ok) flags[0] = 1;
+        mma_commit(done);
+    } else if (warp >= 2) {
+        // a warp reads the quarter of the TMEM lanes that its index allows; warps 2..5 take tile 0, 6..9 tile 1
+        const int quarter = warp & 3, row = quarter * 32 + lane, m = warp >= 6;
+        const int rx = row % a.bw, ry = row / a.bw;
+        const bool left = rx > 0, right = rx < a.bw - 1;
+        float *const mine = xch + m * 256 + quarter * 32;
+        int it = 0;
+        unsigned chunk = 0;
+        for (int p = blockIdx.x; p < g.pairs; p += gridDim.x, ++it) {
+            const int buf = it % NBUF;
+            // the four warps of a tile share barriers: they go on, or give up, together
+            if (!all_of_128(1 + m, mbar_wait(&accfull[buf], (it / NBUF) & 1, deadline))) break;
+            fence_after_sync();
+            const uint32_t acc0 = tmem + buf * (2 * BN) + m * BN + ((uint32_t)(quarter * 32) << 16);
+            const int z = p / a.ty, y = (p - z * a.ty) * 2 * a.bh + m * a.bh + ry;
+            const bool valid = ry < a.bh && y < a.ny;
+            const int64_t v = ((int64_t)z * a.ny + y) * a.nx + rx;
+#pragma unroll 1
+            for (int n = 0; n < CO; n += 16, ++chunk) {
+                uint32_t pm[16], pc[16], pp[16];
+                tmem_ld16_start(acc0 + n, pm);
+                tmem_ld16_start(acc0 + CO + n, pc);
+                tmem_ld16_start(acc0 + 2 * CO + n, pp);
+                tmem_ld_wait();
+                float *slot = mine + (chunk & 1) * 128;
+                if (lane == 31)
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4)
+                        *(uint4 *)(slot + i) = make_uint4(pm[i], pm[i + 1], pm[i + 2], pm[i + 3]);
+                if (lane == 0)
+#pragma unroll
+                    for (int i = 0; i < 16; i += 4)
+                        *(uint4 *)(slot + 16 + i) = make_uint4(pp[i], pp[i + 1], pp[i + 2], pp[i + 3]);
+                if (n + 16 >= CO) {  // the accumulators are in registers: the next pair may overwrite them
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&accempty[buf]);
+                }
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + m) : "memory");
+                float acc[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    float u = __uint_as_float(__shfl_up_sync(0xffffffffu, pm[i], 1));
+                    float d = __uint_as_float(__shfl_down_sync(0xffffffffu, pp[i], 1));
+                    if (lane == 0 && quarter > 0) u = slot[i - 32];
+                    if (lane == 31 && quarter < 3) d = slot[i + 48];
+                    acc[i] = ((left ? u : 0.0f) + __uint_as_float(pc[i])) + (right ? d : 0.0f);
+                }
+                if (valid) store16(a, v, n, acc);
+            }
+        }
+    }
+    __syncwarp();
+    const bool ok = mbar_wait(done, 0, deadline + a.timeout_ns);
+    fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0 && (flags[0] || !ok)) {
+        raise(a.err, RSV_ETIMEOUT);
+        // let copies still in flight land before the shared memory is released
+        for (int kk = max(0, flags[1] - g.S); kk < flags[1]; ++kk)
+            mbar_wait(&full[kk % g.S], (kk / g.S) & 1, now_ns() + a.timeout_ns);
+    }
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
 // ------------------------------------------------------------------ weight-gradient kernel
@@ -836,6 +1045,37 @@ WgPlan wg_plan(ConvVol v, int taps, int ci, int co) {
     return p;
 }
 
+// Shared memory of the folded kernel for this shape, or 0 where it is not the one to use: 27 taps, 32 or 64 output
+// channels, rows of nx voxels that tile a 128-voxel tile's start addresses (nx a multiple of 8, at most 128) and at
+// least half fill it, and a second tile in y.
+size_t fold_plan(ConvVol v, int taps, int ci, int co, FoldArgs *g) {
+    if (taps != 27 || (co != 32 && co != 64) || v.nx % 8 || v.nx > 128) return 0;
+    const int bh = std::min(v.ny, 128 / v.nx);
+    if (bh * v.nx < 64 || v.ny <= bh) return 0;
+    const uint32_t bst = 9u * co * 64, nk = 3 * (ci / 32);
+    g->boxA = (uint32_t)v.nx * (2 * bh + 2) * 64;
+    g->strideA = (g->boxA + (uint32_t)(128 - bh * v.nx) * 64 + 1023u) & ~1023u;
+    const uint32_t room = 227 * 1024 - 1024 - 3072;  // less alignment, barriers and the epilogue's exchange
+    g->resident = nk * bst + 3 * g->strideA <= room;
+    const uint32_t stride = g->strideA + (g->resident ? 0u : bst), base = g->resident ? nk * bst : 0u;
+    g->S = (int)std::min<uint32_t>(kFoldMaxStages, (room - base) / stride);
+    if (g->S < 2) return 0;
+    g->offA = base;
+    g->offBar = base + g->S * stride;
+    g->f.bh = bh;
+    g->f.ty = (v.ny + 2 * bh - 1) / (2 * bh);
+    g->pairs = g->f.ty * v.nz;
+    return g->offBar + 3072 + 1024;
+}
+
+template <int CO>
+cudaError_t launch_fold(cudaStream_t st, size_t smem, const CUtensorMap &ma, const CUtensorMap &mb, const FoldArgs &g) {
+    static cudaError_t attr = set_smem(conv_fold_tc<CO>, 227 * 1024);
+    if (attr != cudaSuccess) return attr;
+    conv_fold_tc<CO><<<std::min(g.pairs, 152), kFoldThreads, smem, st>>>(ma, mb, g);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 rsv_status conv_fwd(cudaStream_t st, ConvVol v, int taps, int ci, int co, const __nv_bfloat16 *x, int ldx,
@@ -875,6 +1115,27 @@ rsv_status conv_fwd(cudaStream_t st, ConvVol v, int taps, int ci, int co, const 
     a.timeout_ns = timeout_ns;
     a.gate = gate;
     CUtensorMap ma, mb;
+    FoldArgs g{};
+    if (const size_t smem = fold_plan(v, taps, ci, co, &g)) {
+        const int bh = g.f.bh, ty = g.f.ty;
+        g.f = a;
+        g.f.bw = v.nx;
+        g.f.bh = bh;
+        g.f.bd = 1;
+        g.f.ty = ty;
+        g.f.nkb = ci / 32;
+        const uint64_t dims[4] = {(uint64_t)ci, (uint64_t)v.nx, (uint64_t)v.ny, (uint64_t)v.nz};
+        const uint64_t strides[3] = {(uint64_t)ldx * 2, (uint64_t)v.nx * ldx * 2, (uint64_t)v.nx * v.ny * ldx * 2};
+        const uint32_t box[4] = {32u, (uint32_t)v.nx, (uint32_t)(2 * bh + 2), 1u};
+        RSV_TRY(make_map(&ma, x, 4, dims, strides, box, 64));
+        const uint64_t wdims[2] = {(uint64_t)taps * ci, (uint64_t)co};
+        const uint64_t wstrides[1] = {(uint64_t)taps * ci * 2};
+        const uint32_t wbox[2] = {32u, (uint32_t)co};
+        RSV_TRY(make_map(&mb, w, 2, wdims, wstrides, wbox, 64));
+        RSV_CUDA_TRY(co == 32 ? launch_fold<32>(st, smem, ma, mb, g) : launch_fold<64>(st, smem, ma, mb, g));
+        count_launches(1);
+        return RSV_OK;
+    }
     {
         const uint64_t dims[4] = {(uint64_t)ci, (uint64_t)v.nx, (uint64_t)v.ny, (uint64_t)v.nz};
         const uint64_t strides[3] = {(uint64_t)ldx * 2, (uint64_t)v.nx * ldx * 2, (uint64_t)v.nx * v.ny * ldx * 2};

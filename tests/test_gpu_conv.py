@@ -155,3 +155,31 @@ def test_conv_argument_checks(rsv):
     assert rsv.rsv_conv3d_fwd(None, 4, 4, 4, 9, 32, 32, _p(x), 32, _p(w), None, 0, None, 0, None, 0, _p(y)) == rsv.RSV_EINVAL
     assert rsv.rsv_conv3d_fwd(None, 4, 4, 4, 1, 32, 32, _p(x), 36, _p(w), None, 0, None, 0, None, 0, _p(y)) == rsv.RSV_EINVAL
     assert rsv.rsv_conv3d_wgrad(None, 6, 4, 4, 27, 32, 32, _p(x), 32, _p(x), 32, _p(y), None) == rsv.RSV_EINVAL
+
+
+# The folded form's edges: rows that do not fill a tile (24 x 5 = 120, 40 x 3), an odd count of tile rows in y, a tile
+# row of one voxel row (nx = 128), weights resident and streamed, and its neighbours that take the general kernel
+# (nx not a multiple of 8, one tile in y, more than 128 voxels in x).
+FOLD_CASES = [
+    (24, 11, 3, 32, 32), (40, 7, 2, 64, 64), (128, 3, 3, 32, 32), (128, 2, 2, 96, 32), (64, 5, 3, 64, 32),
+    (8, 33, 2, 192, 64), (64, 4, 70, 32, 32), (20, 13, 3, 32, 32), (16, 8, 3, 32, 64), (136, 3, 2, 32, 32),
+]
+
+
+@pytest.mark.parametrize("case", FOLD_CASES, ids=[f"{c[0]}x{c[1]}x{c[2]}_ci{c[3]}_co{c[4]}" for c in FOLD_CASES])
+def test_conv_narrow_layers_match_oracle(rsv, case):
+    """Same bound as above: K = 27 ci exact products summed in FP32, plus the bias."""
+    torch = pytest.importorskip("torch")
+    nx, ny, nz, ci, co = case
+    rng = np.random.default_rng(sum(case))
+    xt, xh = _bf16(torch, _vol(rng, nz, ny, nx, ci))
+    wt, wh = _bf16(torch, rng.standard_normal((co, 27, ci)) * np.sqrt(2.0 / (27 * ci)))
+    bias = rng.standard_normal(co).astype(np.float32) * 0.1
+    y32 = torch.full((nz * ny * nx, co), float("nan"), device="cuda")
+    st = rsv.rsv_conv3d_fwd(None, nx, ny, nz, 27, ci, co, _p(xt), ci, _p(wt), _p(torch.tensor(bias).cuda()), 0, None, 0,
+                            None, 0, _p(y32))
+    assert st == rsv.RSV_OK, rsv.status_string(st)
+    ref = U.conv3(xh, wh) + bias
+    absref = U.conv3(np.abs(xh), np.abs(wh)) + np.abs(bias)
+    got = y32.cpu().numpy().reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= 2 * (27 * ci + 1) * U32 * absref)
