@@ -94,63 +94,26 @@ struct StreamSwap {
     }
 };
 
-__device__ __forceinline__ int sys_of_elem(const int32_t *sys_of_cell, int64_t i) { return sys_of_cell[i / 3]; }
-
-// out1[s] = <x, y1> (or its sqrt) and, when y2, out2[s] = <x, y2>, per system s.
-template <typename T>
-__global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(const SegItem *__restrict__ items, int nitems,
-                                                              const int *__restrict__ item_begin,
-                                                              const T *__restrict__ x, const T *__restrict__ y1,
-                                                              const T *__restrict__ y2, double *out1, double *out2,
-                                                              int sqrt1, double *partial, unsigned *ticket,
-                                                              const int *done) {
-    __shared__ double sm[2][kSegThreads / 32];
-    __shared__ bool last;
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-        const SegItem w = items[it];
-        Acc<T> a1, a2;
-        if (!(done && done[w.sys])) {
-            for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) {
-                const T xv = x[i];
-                a1.add(xv, y1[i]);
-                if (y2) a2.add(xv, y2[i]);
-            }
-        }
-        double v1 = warp_sum(a1.value()), v2 = y2 ? warp_sum(a2.value()) : 0.0;
-        if ((threadIdx.x & 31) == 0) {
-            sm[0][threadIdx.x >> 5] = v1;
-            sm[1][threadIdx.x >> 5] = v2;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s1 = 0.0, s2 = 0.0;
-            for (int q = 0; q < kSegThreads / 32; ++q) {
-                s1 += sm[0][q];
-                s2 += sm[1][q];
-            }
-            partial[it] = s1;
-            partial[nitems + it] = s2;
-            __threadfence();
-            const unsigned nit = (unsigned)(item_begin[w.sys + 1] - item_begin[w.sys]);
-            last = atomicAdd(&ticket[w.sys], 1u) == nit - 1;
-        }
-        __syncthreads();
-        if (last && threadIdx.x == 0) {
-            __threadfence();
-            double s1 = 0.0, s2 = 0.0;
-            for (int q = item_begin[w.sys]; q < item_begin[w.sys + 1]; ++q) {
-                s1 += __ldcg(&partial[q]);
-                s2 += __ldcg(&partial[nitems + q]);
-            }
-            if (!(done && done[w.sys])) {
-                out1[w.sys] = sqrt1 ? sqrt(s1) : s1;
-                if (out2) out2[w.sys] = s2;
-            }
-            ticket[w.sys] = 0u;
-        }
-        __syncthreads();
-    }
+// Calls f4(i) for the 16-byte groups of a work item and f1(i) for the elements beside them, over the CTA's threads.
+// Groups start at multiples of 16 bytes of the vectors (ok: every vector's base is 16-byte aligned).
+template <typename T, typename F4, typename F1>
+__device__ __forceinline__ void over_item(const SegItem &w, bool ok, F4 f4, F1 f1) {
+    constexpr int N = Vec<T>::N;
+    const int64_t g0 = ok ? min((w.begin + N - 1) / N * N, w.end) : w.end, g1 = ok ? max(w.end / N * N, g0) : w.end;
+    const int64_t head = ok ? g0 : w.end;
+#pragma unroll 4
+    for (int64_t i = g0 + N * (int64_t)threadIdx.x; i < g1; i += N * (int64_t)blockDim.x) f4(i);
+    for (int64_t i = w.begin + threadIdx.x; i < head; i += blockDim.x) f1(i);
+    for (int64_t i = g1 + threadIdx.x; i < w.end; i += blockDim.x) f1(i);
 }
+template <typename T> __device__ __forceinline__ typename Vec<T>::V ld_vec(const T *p) {
+    return *reinterpret_cast<const typename Vec<T>::V *>(p);
+}
+template <typename T> __device__ __forceinline__ void st_vec(T *p, const typename Vec<T>::V &v) {
+    *reinterpret_cast<typename Vec<T>::V *>(p) = v;
+}
+__device__ __forceinline__ float scalar(double v, float) { return (float)v; }
+__device__ __forceinline__ double scalar(double v, double) { return v; }
 
 __device__ __forceinline__ void finish_sys(BatchDev d, int s, int code) {
     if (code && d.status[s] == 0) d.status[s] = code;
@@ -160,29 +123,24 @@ __device__ __forceinline__ void finish_sys(BatchDev d, int s, int code) {
     }
 }
 
-// BiCGSTAB scalar steps, one thread per system.
-__global__ void b_beta(BatchDev d, int nsys, double btol) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || d.done[s]) return;
+// BiCGSTAB scalar steps of system s.
+__device__ __forceinline__ void step_beta(BatchDev d, int nsys, int s, double btol) {
+    if (d.done[s]) return;
     const double rho1 = d.red[0 * nsys + s];
     if (!isfinite(rho1)) return finish_sys(d, s, RSV_ENAN);
     if (fabs(rho1) <= btol * d.rhn[s] * d.red[6 * nsys + s]) return finish_sys(d, s, RSV_EBREAKDOWN);
     d.rho1[s] = rho1;
     d.beta[s] = (rho1 / d.rho[s]) * (d.alpha[s] / d.omega[s]);
 }
-
-__global__ void b_alpha(BatchDev d, int nsys, double btol) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || d.done[s]) return;
+__device__ __forceinline__ void step_alpha(BatchDev d, int nsys, int s, double btol) {
+    if (d.done[s]) return;
     const double rv = d.red[1 * nsys + s], vn = sqrt(fmax(d.red[2 * nsys + s], 0.0));
     if (!isfinite(rv)) return finish_sys(d, s, RSV_ENAN);
     if (fabs(rv) <= btol * d.rhn[s] * vn) return finish_sys(d, s, RSV_EBREAKDOWN);
     d.alpha[s] = d.rho1[s] / rv;
 }
-
-__global__ void b_check_s(BatchDev d, int nsys) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || d.done[s]) return;
+__device__ __forceinline__ void step_check_s(BatchDev d, int nsys, int s) {
+    if (d.done[s]) return;
     d.iters[s] += 1;
     const double sn = d.red[3 * nsys + s];
     if (!isfinite(sn)) return finish_sys(d, s, RSV_ENAN);
@@ -191,10 +149,9 @@ __global__ void b_check_s(BatchDev d, int nsys) {
         finish_sys(d, s, 0);
     }
 }
-
-__global__ void b_omega(BatchDev d, int nsys, double btol) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || d.done[s]) return;
+__device__ __forceinline__ void step_omega(BatchDev d, int nsys, int s, double btol) {
+    if (d.half[s] == 1) d.half[s] = 2;  // b_half_x has run
+    if (d.done[s]) return;
     const double ts = d.red[4 * nsys + s], tt = d.red[5 * nsys + s];
     if (!isfinite(tt)) return finish_sys(d, s, RSV_ENAN);
     if (!(tt > 0.0)) return finish_sys(d, s, RSV_EBREAKDOWN);
@@ -202,14 +159,12 @@ __global__ void b_omega(BatchDev d, int nsys, double btol) {
     if (fabs(om) <= btol) return finish_sys(d, s, RSV_EBREAKDOWN);
     d.omega[s] = om;
 }
-
 // stall_limit > 0 (FP32 inner solves of refinement): a system whose residual
 // has not dropped below 0.99 of its best for stall_limit passes ends its
 // inner solve; FP32 BiCGSTAB can stagnate above the inner tolerance on an
 // ill-conditioned system, and the FP64 outer step continues from there.
-__global__ void b_finish(BatchDev d, int nsys, int maxit, int stall_limit) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsys || d.done[s]) return;
+__device__ __forceinline__ void step_finish(BatchDev d, int nsys, int s, int maxit, int stall_limit) {
+    if (d.done[s]) return;
     d.rho[s] = d.rho1[s];
     const double rn = d.red[6 * nsys + s];
     if (!isfinite(rn)) return finish_sys(d, s, RSV_ENAN);
@@ -225,52 +180,182 @@ __global__ void b_finish(BatchDev d, int nsys, int maxit, int stall_limit) {
     }
 }
 
+// The scalar step that follows a reduction, run by the thread that finishes a system's sums.
+enum class After { none, alpha, check_s, omega, finish };
+struct Scalars {
+    BatchDev d;
+    int nsys;
+    double btol;
+    int maxit, stall_limit;
+};
+
+// out1[s] = <x, y1> (or its sqrt) and, when y2, out2[s] = <x, y2>, per system s, then the scalar step `after`
+// of system s.  HBM should bound it; what did was one thread per system adding the items' partial sums one
+// after another, FP64 warp trees per item and scalar loads (24 systems, 7 M FP32 unknowns: 72 -> @T@ us).  Now a warp
+// adds the partials (each lane a fixed strided subset, then a tree: still deterministic), items are read in 16-byte
+// groups, and FP32 sums go through the warp as double-float pairs.
 template <typename T>
-__global__ void b_update_p(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const T *r, const T *v, T *p) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        if (d.done[s]) continue;
-        p[i] = r[i] + (T)d.beta[s] * (p[i] - (T)d.omega[s] * v[i]);
+__global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(const SegItem *__restrict__ items, int nitems,
+                                                              const int *__restrict__ item_begin,
+                                                              const T *__restrict__ x, const T *__restrict__ y1,
+                                                              const T *__restrict__ y2, double *out1, double *out2,
+                                                              int sqrt1, double *partial, unsigned *ticket,
+                                                              const int *done, After after, Scalars sc) {
+    __shared__ double sm[2][kSegThreads / 32];
+    __shared__ bool last;
+    const bool ok = ((((uintptr_t)x) | ((uintptr_t)y1) | ((uintptr_t)y2)) & 15) == 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+        const SegItem w = items[it];
+        Acc<T> a1, a2;
+        const bool frozen = done && done[w.sys];
+        if (!frozen)
+            over_item<T>(
+                w, ok,
+                [&](int64_t i) {
+                    const auto xv = ld_vec(x + i), yv = ld_vec(y1 + i);
+#pragma unroll
+                    for (int q = 0; q < Vec<T>::N; ++q) a1.add(Vec<T>::get(xv, q), Vec<T>::get(yv, q));
+                    if (y2) {
+                        const auto zv = ld_vec(y2 + i);
+#pragma unroll
+                        for (int q = 0; q < Vec<T>::N; ++q) a2.add(Vec<T>::get(xv, q), Vec<T>::get(zv, q));
+                    }
+                },
+                [&](int64_t i) {
+                    a1.add(x[i], y1[i]);
+                    if (y2) a2.add(x[i], y2[i]);
+                });
+        Part<T> p1 = Part<T>::of(a1), p2 = Part<T>::of(a2);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            p1.add(p1.xor_shfl(o));
+            if (y2) p2.add(p2.xor_shfl(o));
+        }
+        if (lane == 0) {
+            sm[0][warp] = p1.value();
+            sm[1][warp] = y2 ? p2.value() : 0.0;
+        }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            double s1 = 0.0;
+            for (int q = 0; q < kSegThreads / 32; ++q) s1 += sm[threadIdx.x][q];
+            partial[(size_t)threadIdx.x * nitems + it] = s1;
+        }
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            __threadfence();  // both partial sums before the ticket
+            const unsigned nit = (unsigned)(item_begin[w.sys + 1] - item_begin[w.sys]);
+            last = atomicAdd(&ticket[w.sys], 1u) == nit - 1;
+        }
+        __syncthreads();
+        if (last && warp == 0) {
+            __threadfence();
+            double s1 = 0.0, s2 = 0.0;
+            for (int q = item_begin[w.sys] + lane; q < item_begin[w.sys + 1]; q += 32) {
+                s1 += __ldcg(&partial[q]);
+                if (y2) s2 += __ldcg(&partial[nitems + q]);
+            }
+            s1 = warp_sum(s1);
+            if (y2) s2 = warp_sum(s2);
+            if (lane == 0) {
+                if (!(done && done[w.sys])) {
+                    out1[w.sys] = sqrt1 ? sqrt(s1) : s1;
+                    if (out2) out2[w.sys] = s2;
+                }
+                ticket[w.sys] = 0u;
+                switch (after) {
+                case After::none: break;
+                case After::alpha: step_alpha(sc.d, sc.nsys, w.sys, sc.btol); break;
+                case After::check_s: step_check_s(sc.d, sc.nsys, w.sys); break;
+                case After::omega: step_omega(sc.d, sc.nsys, w.sys, sc.btol); break;
+                case After::finish:  // and the next pass's beta
+                    step_finish(sc.d, sc.nsys, w.sys, sc.maxit, sc.stall_limit);
+                    step_beta(sc.d, sc.nsys, w.sys, sc.btol);
+                    break;
+                }
+            }
+        }
+        __syncthreads();
     }
 }
 
-template <typename T>
-__global__ void b_update_s(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const T *r, const T *v, T *sv) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        if (d.done[s]) continue;
-        sv[i] = r[i] - (T)d.alpha[s] * v[i];
-    }
-}
-
-template <typename T>
-__global__ void b_half_x(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const T *ph, T *x) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        if (d.half[s] != 1) continue;
-        x[i] += (T)d.alpha[s] * ph[i];
-    }
-}
-
-__global__ void b_consume_half(BatchDev d, int nsys) {
+// The first pass's beta, one thread per system.
+__global__ void b_beta(BatchDev d, int nsys, double btol) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < nsys && d.half[s] == 1) d.half[s] = 2;
+    if (s < nsys) step_beta(d, nsys, s, btol);
+}
+
+// Vector updates, one CTA per work item: a system's scalars are loaded and rounded once per item (once per element
+// bound these kernels by the FP64 pipe's conversions), and a frozen system's items return at once.
+template <typename T>
+__global__ void __launch_bounds__(kSegThreads) b_update_p(const SegItem *__restrict__ items, BatchDev d, const T *r, const T *v,
+                                                          T *p) {
+    const SegItem w = items[blockIdx.x];
+    if (d.done[w.sys]) return;
+    const T beta = scalar(d.beta[w.sys], T(0)), om = scalar(d.omega[w.sys], T(0));
+    over_item<T>(
+        w, true,
+        [&](int64_t i) {
+            const auto rv = ld_vec(r + i), vv = ld_vec(v + i);
+            auto pv = ld_vec(p + i);
+#pragma unroll
+            for (int q = 0; q < Vec<T>::N; ++q)
+                Vec<T>::set(pv, q, Vec<T>::get(rv, q) + beta * (Vec<T>::get(pv, q) - om * Vec<T>::get(vv, q)));
+            st_vec(p + i, pv);
+        },
+        [&](int64_t i) { p[i] = r[i] + beta * (p[i] - om * v[i]); });
 }
 
 template <typename T>
-__global__ void b_update_xr(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const T *ph, const T *sh,
-                            const T *sv, const T *t, T *x, T *r) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        if (d.done[s]) continue;
-        const T al = (T)d.alpha[s], om = (T)d.omega[s];
-        x[i] += al * ph[i] + om * sh[i];
-        r[i] = sv[i] - om * t[i];
-    }
+__global__ void __launch_bounds__(kSegThreads) b_update_s(const SegItem *__restrict__ items, BatchDev d, const T *r, const T *v,
+                                                          T *sv) {
+    const SegItem w = items[blockIdx.x];
+    if (d.done[w.sys]) return;
+    const T al = scalar(d.alpha[w.sys], T(0));
+    over_item<T>(
+        w, true,
+        [&](int64_t i) {
+            const auto rv = ld_vec(r + i), vv = ld_vec(v + i);
+            auto o = rv;
+#pragma unroll
+            for (int q = 0; q < Vec<T>::N; ++q) Vec<T>::set(o, q, Vec<T>::get(rv, q) - al * Vec<T>::get(vv, q));
+            st_vec(sv + i, o);
+        },
+        [&](int64_t i) { sv[i] = r[i] - al * v[i]; });
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSegThreads) b_half_x(const SegItem *__restrict__ items, BatchDev d, const T *ph, T *x) {
+    const SegItem w = items[blockIdx.x];
+    if (d.half[w.sys] != 1) return;
+    const T al = scalar(d.alpha[w.sys], T(0));
+    for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) x[i] += al * ph[i];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSegThreads) b_update_xr(const SegItem *__restrict__ items, BatchDev d, const T *ph, const T *sh,
+                                                           const T *sv, const T *t, T *x, T *r) {
+    const SegItem w = items[blockIdx.x];
+    if (d.done[w.sys]) return;
+    const T al = scalar(d.alpha[w.sys], T(0)), om = scalar(d.omega[w.sys], T(0));
+    over_item<T>(
+        w, true,
+        [&](int64_t i) {
+            const auto pv = ld_vec(ph + i), hv = ld_vec(sh + i), sw = ld_vec(sv + i), tv = ld_vec(t + i);
+            auto xv = ld_vec(x + i), rv = sw;
+#pragma unroll
+            for (int q = 0; q < Vec<T>::N; ++q) {
+                Vec<T>::set(xv, q, Vec<T>::get(xv, q) + (al * Vec<T>::get(pv, q) + om * Vec<T>::get(hv, q)));
+                Vec<T>::set(rv, q, Vec<T>::get(sw, q) - om * Vec<T>::get(tv, q));
+            }
+            st_vec(x + i, xv);
+            st_vec(r + i, rv);
+        },
+        [&](int64_t i) {
+            x[i] += al * ph[i] + om * sh[i];
+            r[i] = sv[i] - om * t[i];
+        });
 }
 
 // Start of an inner solve: per-system tolerance and scalars; systems marked
@@ -330,22 +415,22 @@ __global__ void b_outer_check(BatchDev d, int nsys, double rtol, const double *r
 }
 
 template <typename T>
-__global__ void b_scaled_copy(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const double *__restrict__ r64,
-                              const double *__restrict__ rn, T *__restrict__ out) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        out[i] = d.outer[s] ? T(0) : (T)(r64[i] / rn[s]);
-    }
+__global__ void __launch_bounds__(kSegThreads) b_scaled_copy(const SegItem *__restrict__ items, BatchDev d,
+                                                             const double *__restrict__ r64,
+                                                             const double *__restrict__ rn, T *__restrict__ out) {
+    const SegItem w = items[blockIdx.x];
+    const bool skip = d.outer[w.sys] != 0;
+    const double n = rn[w.sys];
+    for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) out[i] = skip ? T(0) : (T)(r64[i] / n);
 }
 
-__global__ void b_add_scaled(int64_t n, BatchDev d, const int32_t *__restrict__ soc, const float *__restrict__ df,
-                             const double *__restrict__ rn, double *__restrict__ x) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += stride) {
-        const int s = sys_of_elem(soc, i);
-        if (!d.outer[s]) x[i] += rn[s] * (double)df[i];
-    }
+__global__ void __launch_bounds__(kSegThreads) b_add_scaled(const SegItem *__restrict__ items, BatchDev d,
+                                                            const float *__restrict__ df, const double *__restrict__ rn,
+                                                            double *__restrict__ x) {
+    const SegItem w = items[blockIdx.x];
+    if (d.outer[w.sys]) return;
+    const double n = rn[w.sys];
+    for (int64_t i = w.begin + threadIdx.x; i < w.end; i += blockDim.x) x[i] += n * (double)df[i];
 }
 
 __global__ void b_bump_outer(BatchDev d, int nsys) {
@@ -353,16 +438,17 @@ __global__ void b_bump_outer(BatchDev d, int nsys) {
     if (s < nsys && !d.outer[s]) d.scale[s] += 1.0;  // outer steps taken (kept as a double)
 }
 
-int egrid(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 8)); }
 unsigned sgrid(int nsys) { return (unsigned)((nsys + 127) / 128); }
 
 template <typename T>
 cudaError_t seg_dot(rsv_solver *s, BatchState *B, const T *x, const T *y1, const T *y2, double *o1, double *o2,
-                    int sqrt1, int slot, const int *done) {
+                    int sqrt1, int slot, const int *done, After after = After::none) {
     count_launches(1);
-    const int grid = std::min(B->nitems, 4 * 152);
+    const int grid = std::min(B->nitems, 8 * 152);
+    const Scalars sc{B->dv, B->nsys, s->p.btol, s->p.maxit, sizeof(T) == 4 ? kStallPasses : 0};
     seg_dot_kernel<T><<<grid, kSegThreads, 0, s->st>>>(B->items, B->nitems, B->item_begin, x, y1, y2, o1, o2, sqrt1,
-                                                       B->dv.partial, B->dv.ticket + (size_t)slot * B->nsys, done);
+                                                       B->dv.partial, B->dv.ticket + (size_t)slot * B->nsys, done,
+                                                       after, sc);
     return cudaGetLastError();
 }
 
@@ -374,39 +460,36 @@ T *vecs(BatchState *B, int64_t ldv, int q) {
 // kGraphIters BiCGSTAB passes for all systems (the body that is captured).
 template <typename T>
 cudaError_t bicg_passes(rsv_solver *s, BatchState *B, T *x) {
-    const int64_t n = s->n, ldv = s->ldv;
+    const int64_t ldv = s->ldv;
     const int nsys = B->nsys;
     const BatchDev d = B->dv;
-    const int32_t *soc = s->A->d_sys_of_cell;
     T *r = vecs<T>(B, ldv, 0), *rh = vecs<T>(B, ldv, 1), *p = vecs<T>(B, ldv, 2), *v = vecs<T>(B, ldv, 3),
       *ph = vecs<T>(B, ldv, 4), *sh = vecs<T>(B, ldv, 5), *sv = vecs<T>(B, ldv, 6), *t = vecs<T>(B, ldv, 7);
-    const double btol = s->p.btol;
-    const int g = egrid(n);
+    const int g = B->nitems;
     cudaError_t e = cudaSuccess;
     for (int it = 0; it < kGraphIters && e == cudaSuccess; ++it) {
-        count_launches(14);
-        b_beta<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, btol);
-        b_update_p<T><<<g, 256, 0, s->st>>>(n, d, soc, r, v, p);
+        count_launches(4);
+        b_update_p<T><<<g, kSegThreads, 0, s->st>>>(B->items, d, r, v, p);
         if ((e = pc_apply<T>(s, p, ph, nullptr)) != cudaSuccess) break;
         if ((e = spmv<T>(s, T(1), ph, T(0), v, nullptr)) != cudaSuccess) break;
-        if ((e = seg_dot<T>(s, B, v, rh, v, d.red + 1 * nsys, d.red + 2 * nsys, 0, 1, d.done)) != cudaSuccess) break;
-        b_alpha<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, btol);
-        b_update_s<T><<<g, 256, 0, s->st>>>(n, d, soc, r, v, sv);
-        if ((e = seg_dot<T>(s, B, sv, sv, (const T *)nullptr, d.red + 3 * nsys, nullptr, 1, 2, d.done)) !=
+        if ((e = seg_dot<T>(s, B, v, rh, v, d.red + 1 * nsys, d.red + 2 * nsys, 0, 1, d.done, After::alpha)) !=
             cudaSuccess)
             break;
-        b_check_s<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys);
-        b_half_x<T><<<g, 256, 0, s->st>>>(n, d, soc, ph, x);
-        b_consume_half<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys);
+        b_update_s<T><<<g, kSegThreads, 0, s->st>>>(B->items, d, r, v, sv);
+        if ((e = seg_dot<T>(s, B, sv, sv, (const T *)nullptr, d.red + 3 * nsys, nullptr, 1, 2, d.done,
+                            After::check_s)) != cudaSuccess)
+            break;
+        b_half_x<T><<<g, kSegThreads, 0, s->st>>>(B->items, d, ph, x);
         if ((e = pc_apply<T>(s, sv, sh, nullptr)) != cudaSuccess) break;
         if ((e = spmv<T>(s, T(1), sh, T(0), t, nullptr)) != cudaSuccess) break;
-        if ((e = seg_dot<T>(s, B, t, sv, t, d.red + 4 * nsys, d.red + 5 * nsys, 0, 3, d.done)) != cudaSuccess) break;
-        b_omega<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, btol);
-        b_update_xr<T><<<g, 256, 0, s->st>>>(n, d, soc, ph, sh, sv, t, x, r);
+        if ((e = seg_dot<T>(s, B, t, sv, t, d.red + 4 * nsys, d.red + 5 * nsys, 0, 3, d.done, After::omega)) !=
+            cudaSuccess)
+            break;
+        b_update_xr<T><<<g, kSegThreads, 0, s->st>>>(B->items, d, ph, sh, sv, t, x, r);
         // ||r|| of the new residual and <rh, r> for the next pass, in one sweep
-        if ((e = seg_dot<T>(s, B, r, r, rh, d.red + 6 * nsys, d.red + 0 * nsys, 1, 0, d.done)) != cudaSuccess) break;
-        b_finish<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, s->p.maxit, sizeof(T) == 4 ? kStallPasses : 0);
-        b_count_done<<<1, 256, 0, s->st>>>(d, nsys);
+        if ((e = seg_dot<T>(s, B, r, r, rh, d.red + 6 * nsys, d.red + 0 * nsys, 1, 0, d.done, After::finish)) !=
+            cudaSuccess)
+            break;
         e = cudaGetLastError();
     }
     return e;
@@ -426,9 +509,10 @@ rsv_status bicg_inner(rsv_solver *s, BatchState *B, const T *rhs, T *x, double t
     RSV_CUDA_TRY(cudaMemsetAsync(v, 0, sizeof(T) * n, s->st));
     // ||r|| and <rh, r> of the starting residual (no system is frozen yet for this sweep)
     RSV_CUDA_TRY(seg_dot<T>(s, B, r, r, rh, d.red + 6 * nsys, d.red + 0 * nsys, 1, 0, nullptr));
-    count_launches(2);
+    count_launches(3);
     b_init<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, tol_param, mixed, s->p.rtol);
     b_count_done<<<1, 256, 0, s->st>>>(d, nsys);
+    b_beta<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys, s->p.btol);
     RSV_CUDA_TRY(cudaGetLastError());
     const int gi = sizeof(T) == 8 ? 0 : 1;
     // (re)capture the graph of kGraphIters passes when the preconditioner changed
@@ -612,11 +696,11 @@ extern "C" rsv_status rsv_solve_batched_ptr(rsv_solver *s, const double *b, doub
             RSV_CUDA_TRY(cudaStreamSynchronize(s->st));
             if (*B->h_ndone >= nsys) break;
             count_launches(2);
-            b_scaled_copy<float><<<egrid(n), 256, 0, s->st>>>(n, d, A->d_sys_of_cell, s->r64, rn, (float *)B->rin);
+            b_scaled_copy<float><<<B->nitems, kSegThreads, 0, s->st>>>(B->items, d, s->r64, rn, (float *)B->rin);
             b_bump_outer<<<sgrid(nsys), 128, 0, s->st>>>(d, nsys);
             RSV_TRY(bicg_inner<float>(s, B, (const float *)B->rin, (float *)B->xin, s->p.inner_rtol, 1));
             count_launches(1);
-            b_add_scaled<<<egrid(n), 256, 0, s->st>>>(n, d, A->d_sys_of_cell, (const float *)B->xin, rn, dx);
+            b_add_scaled<<<B->nitems, kSegThreads, 0, s->st>>>(B->items, d, (const float *)B->xin, rn, dx);
             RSV_CUDA_TRY(cudaGetLastError());
         }
     }

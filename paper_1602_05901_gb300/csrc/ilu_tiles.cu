@@ -44,7 +44,7 @@
 // edges and data (hand-off 3 us); edge windows of 8 and 16 steps (100x100x50: 181 and 219 us against 176) and of 2
 // (229 us); L2 prefetches ahead of the ring (no change).
 //
-// Tiles are processed in order of J+K (backward: reverse order); all of a launch's CTAs are
+// Tiles are processed in order of their distance from the sweep's first plane (backward: reverse order); all of a launch's CTAs are
 // co-resident (cooperative launch), and a tile only ever waits for tiles earlier in
 // its order, so the waits cannot form a cycle.
 #include <algorithm>
@@ -904,11 +904,14 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
     cudaError_t e = cudaSuccess;
     if (!Tl->Ff || Tl->elem != (int)sizeof(T)) {
         free_tiles(Tl);
-        // tiles of every grid, each grid's tiles in order of J+K, grids one after another
+        // Tiles of every grid in order of TJ J + TK K, the planes its start lies behind the grid's first cell: a
+        // CTA that is free takes the tile that can start soonest, in every grid of a batch at once.  (One grid after
+        // another left CTAs waiting in the far tiles of the first grids: @T2@.)
+        struct Place {
+            int key, g, J, K;
+        };
         std::vector<TileSys> sys;
-        std::vector<int2> order;
-        std::vector<int> tile_sys, pos;
-        std::vector<int64_t> row0;
+        std::vector<Place> places;
         int64_t rows = 0;
         int maxS = 0;
         for (int g = 0; g < A->nsys; ++g) {
@@ -922,20 +925,22 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
             ts.S = sg.nx + TJ + TK - 2;
             ts.Sp = (ts.S + 1) / 2 * 2;  // the steps are unrolled by two
             ts.cell0 = sg.cell0;
-            ts.poff = (int)order.size();
+            ts.poff = (int)places.size();
             maxS = std::max(maxS, ts.Sp);
-            pos.resize(order.size() + (size_t)ts.nTJ * ts.nTK);
-            for (int d = 0; d <= ts.nTJ + ts.nTK - 2; ++d)
-                for (int J = 0; J < ts.nTJ; ++J) {
-                    const int K = d - J;
-                    if (K < 0 || K >= ts.nTK) continue;
-                    pos[ts.poff + J * ts.nTK + K] = (int)order.size();
-                    order.push_back(make_int2(J, K));
-                    tile_sys.push_back(g);
-                    row0.push_back(rows);
-                    rows += ts.Sp;
-                }
+            for (int J = 0; J < ts.nTJ; ++J)
+                for (int K = 0; K < ts.nTK; ++K) places.push_back(Place{TJ * J + TK * K, g, J, K});
             sys.push_back(ts);
+        }
+        std::stable_sort(places.begin(), places.end(), [](const Place &a, const Place &b) { return a.key < b.key; });
+        std::vector<int2> order;
+        std::vector<int> tile_sys, pos(places.size());
+        std::vector<int64_t> row0;
+        for (const Place &q : places) {
+            pos[sys[q.g].poff + q.J * sys[q.g].nTK + q.K] = (int)order.size();
+            order.push_back(make_int2(q.J, q.K));
+            tile_sys.push_back(q.g);
+            row0.push_back(rows);
+            rows += sys[q.g].Sp;
         }
         const int nT = (int)order.size();
         if (nT > 65535) return cudaErrorInvalidConfiguration;  // tiles index blockIdx.y of the pack/gather grids
