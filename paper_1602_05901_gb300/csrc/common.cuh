@@ -216,11 +216,14 @@ namespace rsv {
 // One-time kernel attributes (large dynamic shared memory); called at matrix creation.
 cudaError_t spmv_init();
 // status (optional): receives RSV_ETIMEOUT when a CTA's staged copies do not arrive within
-// timeout_ns; the rows that CTA still owed are then written as NaN.
+// timeout_ns; the rows that CTA still owed are then written as NaN.  frozen (optional, one flag per grid of a
+// batch): a CTA whose rows all belong to flagged grids leaves them unwritten.
 cudaError_t launch_spmv_f64(const rsv_mat *A, double alpha, const double *x, double beta, double *y,
-                            const int *done, int *status = nullptr, unsigned long long timeout_ns = 2000000000ull);
+                            const int *done, int *status = nullptr, unsigned long long timeout_ns = 2000000000ull,
+                            const int *frozen = nullptr);
 cudaError_t launch_spmv_f32(const rsv_mat *A, float alpha, const float *x, float beta, float *y,
-                            const int *done, int *status = nullptr, unsigned long long timeout_ns = 2000000000ull);
+                            const int *done, int *status = nullptr, unsigned long long timeout_ns = 2000000000ull,
+                            const int *frozen = nullptr);
 cudaError_t launch_cast_f64_f32(cudaStream_t st, int64_t n, const double *a, float *b);
 // c = a and b = (float)a, one read of a.
 cudaError_t launch_copy_cast(cudaStream_t st, int64_t n, const double *a, double *c, float *b);
@@ -330,7 +333,9 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *T_);
 void free_tiles(IluTiles *T_);
 template <typename T>
 // add0 (optional): z_c[0] += add0[c] on output (carried through the sweeps in the vector's pad slot).
+// frozen (optional, one flag per grid of a batch): z of the flagged grids is not written.
 cudaError_t launch_ilu_apply_tiles(const rsv_mat *A, const IluTiles &T_, const T *r, T *z, const int *done,
-                                   int *status, unsigned long long timeout_ns, const T *add0 = nullptr);
+                                   int *status, unsigned long long timeout_ns, const T *add0 = nullptr,
+                                   const int *frozen = nullptr);
 
 }  // namespace rsv

@@ -263,8 +263,11 @@ struct SweepArgs {
     T *EJ, *EK;          // edge buffers this sweep publishes and reads
     int has_add;         // the pads hold a correction
     const int *done;
+    const int *frozen;   // per grid: its tiles are skipped (null: none)
     int *status;
     unsigned long long timeout_ns;
+    // Whether tile t of the sweep's order is skipped.
+    __device__ __forceinline__ bool skip(bool fwd, int t) const { return frozen && frozen[tile_sys[fwd ? t : nT - 1 - t]]; }
 };
 
 // A tile of a sweep, seen from the corner the sweep starts at.
@@ -464,6 +467,7 @@ __global__ void __launch_bounds__(96, 5) ilu_sweep_f32(SweepArgs<float> P) {
     sm.init(P.NG);
     int group0 = 0;  // data groups of the tiles before this one
     for (int t = blockIdx.x; t < P.nT; t += gridDim.x) {
+        if (P.skip(FWD, t)) continue;
         const Tile tl = tile_of<float, FWD>(P, t, a, b);
         if (!sm.begin(tl)) break;
         const int ngr = tl.Sp / B::GS;
@@ -585,6 +589,7 @@ __global__ void __launch_bounds__(160) ilu_sweep_f64(SweepArgs<double> P) {
     sm.init(P.NG);
     int group0 = 0;
     for (int t = blockIdx.x; t < P.nT; t += gridDim.x) {
+        if (P.skip(FWD, t)) continue;
         const Tile tl = tile_of<double, FWD>(P, t, a, b);
         if (!sm.begin(tl)) break;
         if (e == 3) {
@@ -839,11 +844,12 @@ __global__ void __launch_bounds__(256) gather_tiles(const TileSys *__restrict__ 
                              const int64_t *__restrict__ tile_row0, const int2 *__restrict__ order,
                              const T *__restrict__ r, const T *__restrict__ add, const T *__restrict__ D,
                              T *__restrict__ Vt, T *__restrict__ EJf, T *__restrict__ EKf, T *__restrict__ EJb,
-                             T *__restrict__ EKb) {
+                             T *__restrict__ EKb, const int *frozen) {
     pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
     pdl_trigger();
     using R = Row<T>;
     const int t = blockIdx.y;
+    if (frozen && frozen[tile_sys[t]]) return;
     const TileSys G = tsys[tile_sys[t]];
     const int nx = G.nx, ny = G.ny, nz = G.nz;
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1020,19 +1026,19 @@ void free_tiles(IluTiles *Tl) {
 
 template <typename T>
 cudaError_t launch_ilu_apply_tiles(const rsv_mat *A, const IluTiles &Tl, const T *r, T *z, const int *done,
-                                   int *status, unsigned long long timeout_ns, const T *add0) {
+                                   int *status, unsigned long long timeout_ns, const T *add0, const int *frozen) {
     rsv::count_launches(3);
     const int groups = (Tl.maxS + kGatherSteps - 1) / kGatherSteps;
     const dim3 g((unsigned)((groups * 32 + 255) / 256), (unsigned)Tl.nT);
     cudaError_t e = launch_pdl(gather_tiles<T>, g, dim3(256), 0, A->stream, Tl.tsys, Tl.tile_sys, Tl.tile_row0,
                                Tl.order, r, add0, (const T *)Tl.D, (T *)Tl.Vf, (T *)Tl.EJf, (T *)Tl.EKf, (T *)Tl.EJb,
-                               (T *)Tl.EKb);
+                               (T *)Tl.EKb, frozen);
     if (e != cudaSuccess) return e;
     const int has_add = add0 != nullptr;
     SweepArgs<T> f{Tl.nT, Tl.ng, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Ff,
-                   (const T *)Tl.Vf, (T *)Tl.Vb, nullptr, (T *)Tl.EJf, (T *)Tl.EKf, has_add, done, status, timeout_ns};
+                   (const T *)Tl.Vf, (T *)Tl.Vb, nullptr, (T *)Tl.EJf, (T *)Tl.EKf, has_add, done, frozen, status, timeout_ns};
     SweepArgs<T> bw{Tl.nT, Tl.ng, Tl.tsys, Tl.tile_sys, Tl.tile_row0, Tl.order, Tl.pos_of, (const T *)Tl.Fb,
-                    (const T *)Tl.Vb, nullptr, z, (T *)Tl.EJb, (T *)Tl.EKb, has_add, done, status, timeout_ns};
+                    (const T *)Tl.Vb, nullptr, z, (T *)Tl.EJb, (T *)Tl.EKb, has_add, done, frozen, status, timeout_ns};
     void *fa[] = {&f};
     void *ba[] = {&bw};
     e = cudaLaunchCooperativeKernel(sweep_kernel<T>(true), dim3(Tl.grid), dim3(kSweepThreads<T>), fa, Tl.smem,
@@ -1045,8 +1051,10 @@ cudaError_t launch_ilu_apply_tiles(const rsv_mat *A, const IluTiles &Tl, const T
 template cudaError_t tiles_setup<double>(const rsv_mat *, const double *, IluTiles *);
 template cudaError_t tiles_setup<float>(const rsv_mat *, const double *, IluTiles *);
 template cudaError_t launch_ilu_apply_tiles<double>(const rsv_mat *, const IluTiles &, const double *, double *,
-                                                    const int *, int *, unsigned long long, const double *);
+                                                    const int *, int *, unsigned long long, const double *,
+                                                    const int *);
 template cudaError_t launch_ilu_apply_tiles<float>(const rsv_mat *, const IluTiles &, const float *, float *,
-                                                   const int *, int *, unsigned long long, const float *);
+                                                   const int *, int *, unsigned long long, const float *,
+                                                   const int *);
 
 }  // namespace rsv

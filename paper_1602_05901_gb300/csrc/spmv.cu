@@ -59,14 +59,21 @@ template <typename T, int R> struct SpmvSmem {
 // bulk copies (aligned down/up to 16 bytes; the arrays carry tail padding)
 // while the others load the row pointers; then thread (row, e) forms
 // sum_p A_p[e][:] . x[3 col_p : 3 col_p + 3].
-template <typename T, int R>
+template <typename T, int R, bool LIVE>
 __global__ void __launch_bounds__(3 * R) spmv_bsr3_tma(int nb, const int32_t *__restrict__ rp,
                                                        const int32_t *__restrict__ ci, const T *__restrict__ v,
                                                        T alpha, const T *__restrict__ x, T beta, T *__restrict__ y,
-                                                       const int *done, int *status, unsigned long long timeout_ns) {
+                                                       const int *done, int *status, unsigned long long timeout_ns,
+                                                       const int *frozen, const int32_t *sys_of_cell) {
     pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
     pdl_trigger();
     if (done && *(volatile const int *)done) return;
+    if (LIVE) {  // rows of finished grids of a batch are left as they are
+        const int s1 = sys_of_cell[min(nb, (int)(blockIdx.x + 1) * R) - 1];
+        bool all = true;
+        for (int s = sys_of_cell[blockIdx.x * R]; s <= s1; ++s) all = all && frozen[s] != 0;
+        if (all) return;
+    }
     using L = SpmvSmem<T, R>;
     extern __shared__ __align__(128) unsigned char smem[];
     T *sv = reinterpret_cast<T *>(smem);
@@ -361,7 +368,10 @@ __global__ void __launch_bounds__(256) copy_cast(int64_t n4, int64_t n, const do
 
 template <typename T, int R>
 cudaError_t spmv_attr() {
-    return cudaFuncSetAttribute((const void *)spmv_bsr3_tma<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute((const void *)spmv_bsr3_tma<T, R, false>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SpmvSmem<T, R>::BYTES);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute((const void *)spmv_bsr3_tma<T, R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)SpmvSmem<T, R>::BYTES);
 }
 
@@ -370,22 +380,23 @@ cudaError_t spmv_attr() {
 // 0.383 against 0.377 ms): the SpMV keeps the staged column indices.
 template <typename T, int R>
 cudaError_t spmv_launch(const rsv_mat *A, const T *v, T alpha, const T *x, T beta, T *y, const int *done,
-                        int *status, unsigned long long timeout_ns) {
+                        int *status, unsigned long long timeout_ns, const int *frozen) {
     const int grid = (int)((A->nb + R - 1) / R);
     rsv::count_launches(1);
-    return launch_pdl(spmv_bsr3_tma<T, R>, dim3(grid), dim3(3 * R), SpmvSmem<T, R>::BYTES, A->stream, (int)A->nb,
-                      A->d_rp, A->d_ci, v, alpha, x, beta, y, done, status, timeout_ns);
+    return launch_pdl(frozen ? spmv_bsr3_tma<T, R, true> : spmv_bsr3_tma<T, R, false>, dim3(grid), dim3(3 * R),
+                      SpmvSmem<T, R>::BYTES, A->stream, (int)A->nb, A->d_rp, A->d_ci, v, alpha, x, beta, y, done, status,
+                      timeout_ns, frozen, A->d_sys_of_cell);
 }
 
 // Block rows per CTA: 32, 64 or 128, picked per matrix and precision by timing (spmv_autotune).
 template <typename T>
 cudaError_t spmv_dispatch(const rsv_mat *A, const T *v, T alpha, const T *x, T beta, T *y, const int *done,
-                          int *status, unsigned long long timeout_ns) {
+                          int *status, unsigned long long timeout_ns, const int *frozen) {
     if (A->nb == 0) return cudaSuccess;
     switch (sizeof(T) == 8 ? A->spmv_rows64 : A->spmv_rows32) {
-    case 32: return spmv_launch<T, 32>(A, v, alpha, x, beta, y, done, status, timeout_ns);
-    case 64: return spmv_launch<T, 64>(A, v, alpha, x, beta, y, done, status, timeout_ns);
-    default: return spmv_launch<T, kRows>(A, v, alpha, x, beta, y, done, status, timeout_ns);
+    case 32: return spmv_launch<T, 32>(A, v, alpha, x, beta, y, done, status, timeout_ns, frozen);
+    case 64: return spmv_launch<T, 64>(A, v, alpha, x, beta, y, done, status, timeout_ns, frozen);
+    default: return spmv_launch<T, kRows>(A, v, alpha, x, beta, y, done, status, timeout_ns, frozen);
     }
 }
 
@@ -439,13 +450,13 @@ cudaError_t spmv_init() {
 }
 
 cudaError_t launch_spmv_f64(const rsv_mat *A, double alpha, const double *x, double beta, double *y,
-                            const int *done, int *status, unsigned long long timeout_ns) {
-    return spmv_dispatch<double>(A, A->d_v, alpha, x, beta, y, done, status, timeout_ns);
+                            const int *done, int *status, unsigned long long timeout_ns, const int *frozen) {
+    return spmv_dispatch<double>(A, A->d_v, alpha, x, beta, y, done, status, timeout_ns, frozen);
 }
 
 cudaError_t launch_spmv_f32(const rsv_mat *A, float alpha, const float *x, float beta, float *y,
-                            const int *done, int *status, unsigned long long timeout_ns) {
-    return spmv_dispatch<float>(A, A->d_v32, alpha, x, beta, y, done, status, timeout_ns);
+                            const int *done, int *status, unsigned long long timeout_ns, const int *frozen) {
+    return spmv_dispatch<float>(A, A->d_v32, alpha, x, beta, y, done, status, timeout_ns, frozen);
 }
 
 cudaError_t spmv_autotune(rsv_mat *A) {
