@@ -288,12 +288,14 @@ void free_schedule(Schedule *sch);
 cudaError_t launch_bj_setup(const rsv_mat *A, bool from_f32, double *dinv, float *dinv32, int *status);
 template <typename T>
 cudaError_t launch_bj_apply(cudaStream_t st, int64_t nb, const T *dinv, const T *r, T *z, const int *done);
-cudaError_t launch_ilu_setup(const rsv_mat *A, const Schedule &sch, bool from_f32, double *dinv, int *status);
+// Hyperplanes h0 .. h1 - 1 (calls for consecutive ranges follow one another on the stream).
+cudaError_t launch_ilu_setup(const rsv_mat *A, const Schedule &sch, bool from_f32, double *dinv, int *status, int h0,
+                             int h1);
 
 // ---- implemented in cpr.cu
 // decoupling: 0 quasi-IMPES, 1 ABF, 2 true-IMPES from the accumulation blocks acc [nb][9] (rsv_pc_params).
 // coarsening: 0 geometric hierarchy, 1 algebraic (amg_setup runs afterwards, from P->a7[0]).
-cudaError_t cpr_setup(const rsv_mat *A, bool mixed, int max_levels, int max_coarse, int sweeps, int decoupling,
+cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_levels, int max_coarse, int sweeps, int decoupling,
                       const double *acc, int coarsening, Cpr *P, int *status);
 // ---- implemented in amg.cu
 rsv_status amg_setup(const rsv_mat *A, Cpr *P, int max_levels, int max_coarse, int sweeps);

@@ -632,9 +632,8 @@ void free_cpr(Cpr *P) {
     *P = Cpr();
 }
 
-cudaError_t cpr_setup(const rsv_mat *A, bool mixed, int max_levels, int max_coarse, int sweeps, int decoupling,
-                      const double *acc, int coarsening, Cpr *P, int *status) {
-    cudaStream_t st = A->stream;
+cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_levels, int max_coarse, int sweeps,
+                      int decoupling, const double *acc, int coarsening, Cpr *P, int *status) {
     const size_t es = mixed ? sizeof(float) : sizeof(double);
     amg_free(P);
     if (coarsening == 1) max_levels = 1;  // the geometric part keeps only the finest level

@@ -238,8 +238,9 @@ template cudaError_t launch_bj_apply<float>(cudaStream_t, int64_t, const float *
 // One launch per hyperplane.  Each but the first is a programmatic dependent of the one before: it loads
 // the matrix while the previous plane runs and waits for it on the device before reading its factors.  The
 // first is launched the ordinary way, so all of them find the matrix values written.
-cudaError_t launch_ilu_setup(const rsv_mat *A, const Schedule &sch, bool from_f32, double *dinv, int *status) {
-    for (int h = 0; h < sch.nplanes; ++h) {
+cudaError_t launch_ilu_setup(const rsv_mat *A, const Schedule &sch, bool from_f32, double *dinv, int *status, int h0,
+                             int h1) {
+    for (int h = h0; h < h1; ++h) {
         const int p0 = sch.plane_ptr[h], p1 = sch.plane_ptr[h + 1];
         const dim3 grid((p1 - p0 + kPlaneCells - 1) / kPlaneCells), block(128);
         rsv::count_launches(1);

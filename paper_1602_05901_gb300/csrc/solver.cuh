@@ -49,6 +49,9 @@ struct rsv_solver {
     double *acc = nullptr;       // accumulation blocks [nb][9] for true-IMPES decoupling, device
     double ms_setup = 0.0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
+    // CPR setup runs beside the block factorisation (rsv_precond_setup)
+    cudaStream_t side = nullptr;
+    cudaEvent_t fork = nullptr, joined = nullptr;
 };
 
 namespace rsv {
