@@ -17,15 +17,19 @@
 //   weight slice; four (BK = 64) or two (BK = 32) MMAs of K = 16 consume it.
 // Weight gradient:
 //   gw[co][t][ci] = sum_v gy[v, co] x[v + off_t, ci] reduces over voxels, so
-//   K = voxels.  Both operands are first copied voxel-major (one row of
-//   voxels per channel) into a flat layout padded by one zero slice in z and
-//   one zero row in y on each side, so that the dz and dy shifts of a tap are
-//   plain offsets of the flat TMA coordinate (zeros arrive at the borders).
-//   The dx shift cannot be such an offset (the innermost TMA coordinate must
-//   stay 16-byte aligned), so the input is copied three times, pre-shifted by
-//   dx = -1, 0, +1.  M = 128 rows of (tap, ci) pairs, N = output channels, K
-//   steps of 64 voxels; CTAs split the voxels and write FP32 partial sums
-//   that a second kernel adds in a fixed order.
+//   K = voxels; CTAs split the voxels and write FP32 partial sums that a
+//   second kernel adds in a fixed order.  Three forms:
+//   * 3x3x3 with rows of at most 128 voxels: whole rows of a plane, the three
+//     y taps from one box (conv_wgrad_rows).
+//   * boxes of 64 voxels read from the channels-last tensors (conv_wgrad_mn):
+//     1x1x1 layers and longer rows.
+//   * otherwise (no such box, or a leading dimension that TMA cannot take)
+//     both operands are first copied voxel-major (one row of voxels per
+//     channel) into a flat layout padded by one zero slice in z and one zero
+//     row in y on each side, so that the dz and dy shifts of a tap are plain
+//     offsets of the flat TMA coordinate.  The dx shift cannot be such an
+//     offset (the innermost TMA coordinate must stay 16-byte aligned), so the
+//     input is copied three times, pre-shifted by dx = -1, 0, +1.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -766,50 +770,189 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (warp == 2) tmem_dealloc(tmem, TCOLS);
 }
 
-// gb[c] partial sums from the channels-last gradient: CTA b sums its chunk of
-// voxels for every channel (lane l owns channels l, l + 32, ...; warps stride
-// the voxels), warps added in order.  part[b][co].
+// ------------------------------------------------------------------ weight gradient, rows of a plane shared by the y taps
+// The MN-major form above reads every tap's shifted box of the activations from L2, 2 taps of 64 channels per 24 KB,
+// and that is what bounds it (32 bytes per cycle and SM).  Here one K step is R whole rows of a plane, K = nx R voxels
+// in (y, x) order, and its column operand comes from one box of R + 2 rows: the three y taps are the same box read
+// nx shared-memory rows apart, 3 x 64 (or 32) columns of one product.  The row operand holds 128 rows: the other
+// tensor at two (of 64 channels; four of 32; one of 128) of the nine (dz, dx) shifts.  An MMA's time does
+// not depend on N up to 192, so the wider N is free.  The column operand is unshifted in x and z: a voxel pair
+// counts where both are in the grid, and boxes read zeros outside.
+// 64x64x32, 64 -> 64 channels: 74 -> 27 us; a whole call with the bias gradient 123 -> 61 us.  128x128x64, 32 -> 32: 494
+// -> 161 us; 16x16x8, 256 -> 256: 86 -> 50 us.
+struct WgRowArgs {
+    int nx, R, kcy, nchunks, cps;  // rows per K step, steps per plane, steps, steps per split
+    int cm, variants, nmb;         // channels per row block, shifts per MMA, channel blocks
+    int ca, cb;                    // channels of the row and column operand
+    int sgn;                       // +1: rows = gradient, columns = input; -1: the reverse
+    int S;                         // stages
+    uint32_t offN, stride, offBar;
+    float *partial;                // [splits][27][ca][cb]
+    int *err;
+    uint64_t timeout_ns;
+};
+
+template <int CN>
+__global__ void __launch_bounds__(kThreads, 1)
+    conv_wgrad_rows(const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmN, const WgRowArgs a) {
+    constexpr int N = 3 * CN;
+    constexpr uint32_t TCOLS = tmem_cols_for(N);
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    uint8_t *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
+    uint64_t *full = (uint64_t *)(sm + a.offBar);
+    uint64_t *empty = full + a.S;
+    uint64_t *done = empty + a.S;
+    uint32_t *tmem_slot = (uint32_t *)(done + 1);
+    int *flags = (int *)(tmem_slot + 1);  // a wait ran out; steps issued; steps consumed
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int vg = blockIdx.x / a.nmb, mb = blockIdx.x % a.nmb;
+    const int q0 = blockIdx.z * a.cps;
+    const int nk = max(0, min(a.nchunks, q0 + a.cps) - q0);
+    const int nv = min(a.variants, 9 - vg * a.variants);
+    const int colA = min(a.cm, 64), K = a.nx * a.R;
+    const uint32_t rowA = colA * 2, rowB = CN * 2, boxA = K * rowA;
+    const uint64_t deadline = now_ns() + a.timeout_ns;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < a.S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        flags[0] = flags[1] = flags[2] = 0;
+        fence_mbar_init();
+    }
+    if (warp == 2) tmem_alloc(tmem_slot, TCOLS);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        prefetch_map(&tmM);
+        prefetch_map(&tmN);
+        const int cols = a.cm / colA;
+        const uint32_t bytes = (uint32_t)(nv * cols) * boxA + (uint32_t)(a.nx * (a.R + 2)) * rowB;
+        int kk = 0, s = 0;
+        unsigned parity = 1;
+        for (; kk < nk; ++kk) {
+            if (kk >= a.S && !mbar_wait(&empty[s], parity, deadline)) {
+                flags[0] = 1;
+                break;
+            }
+            const int z = (q0 + kk) / a.kcy, y = ((q0 + kk) % a.kcy) * a.R;
+            uint8_t *st = sm + s * a.stride;
+            mbar_expect_tx(&full[s], bytes);
+            tma_load_4d(st + a.offN, &tmN, blockIdx.y * CN, 0, y - 1, z, &full[s]);
+            for (int v = 0; v < nv; ++v) {
+                const int sh = vg * a.variants + v, dz = sh / 3 - 1, dx = sh % 3 - 1;
+                for (int j = 0; j < cols; ++j)
+                    tma_load_4d(st + (v * cols + j) * boxA, &tmM, mb * a.cm + j * colA, -a.sgn * dx, y, z - a.sgn * dz,
+                                &full[s]);
+            }
+            if (++s == a.S) {
+                s = 0;
+                parity ^= 1u;
+            }
+        }
+        flags[1] = kk;
+    } else if (warp == 1 && lane == 0) {
+        constexpr uint32_t idesc = idesc_bf16(128, N, true, true);
+        const int swzA = colA == 64 ? 128 : 64, swzB = CN == 64 ? 128 : 64;
+        int kk = 0, s = 0;
+        unsigned parity = 0;
+        for (; kk < nk; ++kk) {
+            if (!mbar_wait(&full[s], parity, deadline)) {
+                flags[0] = 1;
+                break;
+            }
+            fence_after_sync();
+            const uint32_t sa = smem_u32(sm + s * a.stride), sb = sa + a.offN;
+            for (int k = 0; k < K; k += 16)
+                mma_bf16(tmem, mnmajor_desc(sa + k * rowA, swzA, boxA, 8 * rowA),
+                         mnmajor_desc(sb + k * rowB, swzB, a.nx * rowB, 8 * rowB), idesc, (kk > 0 || k > 0) ? 1u : 0u);
+            mma_commit(&empty[s]);
+            if (++s == a.S) {
+                s = 0;
+                parity ^= 1u;
+            }
+        }
+        flags[2] = kk;
+        mma_commit(done);
+    }
+    __syncwarp();
+
+    const bool ok = mbar_wait(done, 0, deadline + a.timeout_ns);
+    fence_after_sync();
+    const int row = warp * 32 + lane;
+    const int v = row / a.cm, c = row % a.cm, sh = vg * a.variants + v;
+    const bool valid = ok && v < nv && !flags[0];
+    float *out = a.partial + ((int64_t)blockIdx.z * 27 * a.ca + mb * a.cm + c) * a.cb + blockIdx.y * CN;
+#pragma unroll 1
+    for (int c0 = 0; c0 < N; c0 += 16) {
+        float acc[16];
+        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, acc);
+        if (!valid) continue;
+        if (nk == 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc[i] = 0.0f;
+        }
+        const int dy = a.sgn * (c0 / CN - 1);
+        const int tap = 9 * (sh / 3) + 3 * (dy + 1) + sh % 3;
+        float4 *o = (float4 *)(out + (int64_t)tap * a.ca * a.cb + c0 % CN);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = make_float4(acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
+    }
+
+    fence_before_sync();
+    __syncthreads();
+    if (threadIdx.x == 0 && (flags[0] || !ok)) {
+        raise(a.err, RSV_ETIMEOUT);
+        // copies still in flight land before the shared memory is given up (bounded)
+        for (int kk = flags[2]; kk < flags[1]; ++kk)
+            mbar_wait(&full[kk % a.S], (kk / a.S) & 1, now_ns() + a.timeout_ns);
+    }
+    __syncthreads();
+    if (warp == 2) tmem_dealloc(tmem, TCOLS);
+}
+
+// gb[c] partial sums from the channels-last gradient: CTA b sums its chunk of voxels, a thread eight channels (16
+// bytes) of every slots-th voxel.  part[b][co].  Bound by the loads in flight: 2-byte loads took 14.5 us on
+// 64x64x32 voxels of 64 channels, these 8.
 __global__ void __launch_bounds__(256) bias_grad_cl(const __nv_bfloat16 *__restrict__ gy, int ld, int co, int64_t V,
                                                     float *__restrict__ part) {
-    __shared__ float red[8][256];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ float red[256 * 8];
     const int64_t len = (V + gridDim.x - 1) / gridDim.x;
     const int64_t v0 = blockIdx.x * len, v1 = min(V, v0 + len);
-    const int nq = (co + 31) / 32;
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int64_t v = v0 + warp;
-    for (; v + 24 < v1; v += 32)  // four voxels in flight per warp
+    for (int c0 = 0; c0 < co; c0 += 2048) {  // channels that 256 threads cover
+        const int pieces = min(256, (co - c0) / 8), slots = 256 / pieces;
+        const int piece = threadIdx.x % pieces, slot = threadIdx.x / pieces;
+        float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (slot < slots) {
+            const __nv_bfloat16 *g = gy + c0 + piece * 8;
+#pragma unroll 4
+            for (int64_t v = v0 + slot; v < v1; v += slots) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(g + v * ld);
+                const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q < nq && lane + 32 * q < co) {
-                const int c = lane + 32 * q;
-                const float a0 = __bfloat162float(gy[v * ld + c]), a1 = __bfloat162float(gy[(v + 8) * ld + c]);
-                const float a2 = __bfloat162float(gy[(v + 16) * ld + c]), a3 = __bfloat162float(gy[(v + 24) * ld + c]);
-                acc[q] += (a0 + a1) + (a2 + a3);
+                for (int q = 0; q < 4; ++q) {
+                    acc[2 * q] += __uint_as_float(u[q] << 16);
+                    acc[2 * q + 1] += __uint_as_float(u[q] & 0xffff0000u);
+                }
             }
-    for (; v < v1; v += 8)
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            if (q < nq && lane + 32 * q < co) acc[q] += __bfloat162float(gy[v * ld + lane + 32 * q]);
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-        if (lane + 32 * q < co) red[warp][lane + 32 * q] = acc[q];
-    __syncthreads();
-    for (int c = threadIdx.x; c < co; c += 256) {
-        float t = 0.0f;
-        for (int w = 0; w < 8; ++w) t += red[w][c];
-        part[(int64_t)blockIdx.x * co + c] = t;
+            for (int q = 0; q < 8; ++q) red[slot * pieces * 8 + piece * 8 + q] = acc[q];
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < pieces * 8; c += 256) {
+            float t = 0.0f;
+            for (int q = 0; q < slots; ++q) t += red[q * pieces * 8 + c];
+            part[(int64_t)blockIdx.x * co + c0 + c] = t;
+        }
+        __syncthreads();
     }
-}
-// One warp per channel: lane l adds the blocks l, l + 32, ... in order, then a fixed shuffle tree.
-__global__ void bias_grad_cl_final(const float *__restrict__ part, int nblk, int co, float *__restrict__ gb) {
-    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (c >= co) return;
-    float t = 0.0f;
-    for (int b = lane; b < nblk; b += 32) t += part[(int64_t)b * co + c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if (lane == 0) gb[c] = t;
 }
 
 // ------------------------------------------------------------------ helper kernels
@@ -857,18 +1000,33 @@ __global__ void __launch_bounds__(256)
 }
 
 // gw[co][t][ci] = sum over splits of the partials, in split order.  The partials are
-// [s][t][ci][co] (swap = 0), or [s][t][co][ci] (swap = 1: rows were output channels).
-__global__ void wgrad_reduce(const float *__restrict__ partial, int splits, int taps, int ci, int co,
-                             float *__restrict__ gw, int swap) {
+// [s][t][ci][co] (swap = 0), or [s][t][co][ci] (swap = 1: rows were output channels).  The blocks behind the first
+// wblocks add the bias gradient's nblk partial sums (bias_grad_cl), one warp per channel: lane l the blocks l,
+// l + 32, ... in order, then a fixed shuffle tree.
+__global__ void __launch_bounds__(256) wgrad_reduce(const float *__restrict__ partial, int splits, int taps, int ci, int co,
+                                                    float *__restrict__ gw, int swap, int wblocks,
+                                                    const float *__restrict__ bpart, int nblk, float *__restrict__ gb) {
+    if ((int)blockIdx.x >= wblocks) {
+        const int c = ((int)blockIdx.x - wblocks) * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (c >= co) return;
+        float t = 0.0f;
+        for (int b = lane; b < nblk; b += 32) t += bpart[(int64_t)b * co + c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) gb[c] = t;
+        return;
+    }
     const int64_t total = (int64_t)taps * ci * co;
     const int ra = swap ? co : ci, rb = swap ? ci : co;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)wblocks * blockDim.x) {
         const int o = (int)(i / ((int64_t)taps * ci));
         const int t = (int)((i / ci) % taps);
         const int c = (int)(i % ci);
         const int row = swap ? o : c, col = swap ? c : o;
+        const float *p = partial + ((int64_t)t * ra + row) * rb + col;
         float s = 0.0f;
-        for (int q = 0; q < splits; ++q) s += partial[(((int64_t)q * taps + t) * ra + row) * rb + col];
+#pragma unroll 8
+        for (int q = 0; q < splits; ++q) s += p[q * total];
         gw[i] = s;
     }
 }
@@ -1004,7 +1162,7 @@ struct WgPlan {
     int bw, bh, bd, kcx, kcy;
 };
 
-constexpr int kBiasBlocks = 512;
+constexpr int kBiasBlocks = 304;
 
 size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -1043,6 +1201,67 @@ WgPlan wg_plan(ConvVol v, int taps, int ci, int co) {
     p.part_bytes = round256((size_t)p.splits * taps * ci * co * 4);
     p.bias_bytes = round256((size_t)kBiasBlocks * co * 4);
     return p;
+}
+
+// The form with whole rows of a plane, or S = 0 where it does not apply: 27 taps, rows of at most 128 voxels, and
+// two stages of shared memory.
+struct WgRowPlan {
+    int S, swap, R, kcy, nchunks, cps, splits, cm, cn, variants, groups, nmb, nnb;
+    uint32_t offN, stride;
+    size_t part_bytes;
+};
+
+WgRowPlan wg_row_plan(ConvVol v, int taps, int ci, int co) {
+    WgRowPlan p{};
+    if (taps != 27 || v.nx > 128 || v.nx % 8 || ci % 32 || co % 32) return p;
+    // the roles with fewer MMAs: rows a (in blocks of 128, 64 or 32 channels), columns b (of 64 or 32)
+    auto block = [](int a) { return a % 128 == 0 ? 128 : a % 64 == 0 ? 64 : 32; };
+    auto mmas = [&](int a, int b) {
+        const int cm = block(a), var = 128 / cm;
+        return (int64_t)(a / cm) * ((9 + var - 1) / var) * (b / std::min(block(b), 64));
+    };
+    p.swap = mmas(ci, co) < mmas(co, ci);  // rows = input, columns = gradient
+    const int a = p.swap ? ci : co, b = p.swap ? co : ci;
+    p.cm = block(a);
+    p.variants = 128 / p.cm;
+    p.groups = (9 + p.variants - 1) / p.variants;
+    p.nmb = a / p.cm;
+    // Rows per step: the two rows of halo cost less the more there are, up to 256 voxels with three stages.  Two rows
+    // of 120 voxels with 64 columns leave room for one stage only: 32 columns then.
+    const int even = v.nx % 16 ? 2 : 1;  // K is a multiple of 16 voxels
+    const int most = std::min((v.ny + even - 1) / even * even, std::max(256 / v.nx, even) / even * even);
+    const uint32_t room = 227 * 1024 - 1024 - 1024;  // less alignment and barriers
+    for (int cn = std::min(block(b), 64); cn >= 32 && !p.S; cn /= 2)
+        for (int least : {3, 2})
+            for (int R = most; R >= even && !p.S; R -= even) {
+                const uint32_t offN = (uint32_t)v.nx * R * 256;
+                const uint32_t stride = (offN + (uint32_t)v.nx * (R + 2) * cn * 2 + 1023u) & ~1023u;
+                const int S = (int)std::min<uint32_t>(8, room / stride);
+                if (S < least) continue;
+                p.S = S;
+                p.R = R;
+                p.cn = cn;
+                p.offN = offN;
+                p.stride = stride;
+            }
+    if (!p.S) return p;
+    p.nnb = b / p.cn;
+    p.kcy = (v.ny + p.R - 1) / p.R;
+    p.nchunks = p.kcy * v.nz;
+    const int ctas = p.groups * p.nmb * p.nnb;
+    const int splits = std::max(1, std::min(p.nchunks, 152 / ctas));  // one CTA per SM
+    p.cps = (p.nchunks + splits - 1) / splits;
+    p.splits = (p.nchunks + p.cps - 1) / p.cps;
+    p.part_bytes = round256((size_t)p.splits * 27 * ci * co * 4);
+    return p;
+}
+
+template <int CN>
+cudaError_t launch_wgrow(cudaStream_t st, dim3 grid, const CUtensorMap &mm, const CUtensorMap &mn, const WgRowArgs &a) {
+    static cudaError_t attr = set_smem(conv_wgrad_rows<CN>, 227 * 1024);
+    if (attr != cudaSuccess) return attr;
+    conv_wgrad_rows<CN><<<grid, kThreads, a.offBar + 1024 + 1024, st>>>(mm, mn, a);
+    return cudaGetLastError();
 }
 
 // Shared memory of the folded kernel for this shape, or 0 where it is not the one to use: 27 taps, 32 or 64 output
@@ -1165,7 +1384,7 @@ rsv_status conv_flip(cudaStream_t st, int ci, int co, const __nv_bfloat16 *w, __
 
 size_t conv_wgrad_scratch(ConvVol v, int taps, int ci, int co) {
     const WgPlan p = wg_plan(v, taps, ci, co);
-    return p.xt_bytes + p.gyt_bytes + p.part_bytes + p.bias_bytes;
+    return std::max(p.xt_bytes + p.gyt_bytes + p.part_bytes, wg_row_plan(v, taps, ci, co).part_bytes) + p.bias_bytes;
 }
 
 rsv_status conv_wgrad(cudaStream_t st, ConvVol v, int taps, int ci, int co, const __nv_bfloat16 *x, int ldx,
@@ -1176,8 +1395,59 @@ rsv_status conv_wgrad(cudaStream_t st, ConvVol v, int taps, int ci, int co, cons
         return RSV_EINVAL;
     const WgPlan p = wg_plan(v, taps, ci, co);
     if (!aligned16(scratch)) return RSV_EINVAL;
+    const bool aligned = aligned16(x) && aligned16(gy) && ldx % 8 == 0 && ldgy % 8 == 0;
+    if (p.mn && !aligned) return RSV_EINVAL;
+    const int64_t V = (int64_t)v.nx * v.ny * v.nz, total = (int64_t)taps * ci * co;
+    const int wblocks = (int)std::min<int64_t>((total + 255) / 256, 4096);
+    // the partial sums of both gradients, added in a fixed order
+    auto reduce = [&](const float *part, int splits, int swap, float *bpart) -> rsv_status {
+        if (gb) {
+            bias_grad_cl<<<kBiasBlocks, 256, 0, st>>>(gy, ldgy, co, V, bpart);
+            RSV_CUDA_TRY(cudaGetLastError());
+        }
+        wgrad_reduce<<<wblocks + (gb ? (co + 7) / 8 : 0), 256, 0, st>>>(part, splits, taps, ci, co, gw, swap, wblocks,
+                                                                      bpart, kBiasBlocks, gb);
+        RSV_CUDA_TRY(cudaGetLastError());
+        count_launches(gb ? 3 : 2);
+        return RSV_OK;
+    };
+    const WgRowPlan rp = aligned ? wg_row_plan(v, taps, ci, co) : WgRowPlan{};
+    if (rp.S) {
+        WgRowArgs a{};
+        a.nx = v.nx;
+        a.R = rp.R;
+        a.kcy = rp.kcy;
+        a.nchunks = rp.nchunks;
+        a.cps = rp.cps;
+        a.cm = rp.cm;
+        a.variants = rp.variants;
+        a.nmb = rp.nmb;
+        a.ca = rp.swap ? ci : co;
+        a.cb = rp.swap ? co : ci;
+        a.sgn = rp.swap ? -1 : 1;
+        a.S = rp.S;
+        a.offN = rp.offN;
+        a.stride = rp.stride;
+        a.offBar = rp.S * rp.stride;
+        a.partial = (float *)scratch;
+        a.err = err;
+        a.timeout_ns = timeout_ns;
+        CUtensorMap mm, mn;
+        auto map = [&](CUtensorMap *m, bool input, int cols, int rows) {
+            const __nv_bfloat16 *base = input ? x : gy;
+            const uint64_t ld = input ? ldx : ldgy;
+            const uint64_t dims[4] = {(uint64_t)(input ? ci : co), (uint64_t)v.nx, (uint64_t)v.ny, (uint64_t)v.nz};
+            const uint64_t strides[3] = {ld * 2, (uint64_t)v.nx * ld * 2, (uint64_t)v.nx * v.ny * ld * 2};
+            const uint32_t box[4] = {(uint32_t)cols, (uint32_t)v.nx, (uint32_t)rows, 1u};
+            return make_map(m, base, 4, dims, strides, box, cols * 2);
+        };
+        RSV_TRY(map(&mm, rp.swap, std::min(rp.cm, 64), rp.R));
+        RSV_TRY(map(&mn, !rp.swap, rp.cn, rp.R + 2));
+        const dim3 grid(rp.groups * rp.nmb, rp.nnb, rp.splits);
+        RSV_CUDA_TRY(rp.cn == 64 ? launch_wgrow<64>(st, grid, mm, mn, a) : launch_wgrow<32>(st, grid, mm, mn, a));
+        return reduce(a.partial, rp.splits, rp.swap ? 0 : 1, (float *)((char *)scratch + rp.part_bytes));
+    }
     if (p.mn) {
-        if (!aligned16(x) || !aligned16(gy) || ldx % 8 || ldgy % 8) return RSV_EINVAL;
         float *part = (float *)((char *)scratch + p.xt_bytes + p.gyt_bytes);
         float *bpart = (float *)((char *)part + p.part_bytes);
         WgMnArgs a{};
@@ -1219,20 +1489,7 @@ rsv_status conv_wgrad(cudaStream_t st, ConvVol v, int taps, int ci, int co, cons
             RSV_TRY(make_map(&mg, colp, 4, dims, strides, box, a.colB * 2));
         }
         RSV_CUDA_TRY(launch_wgmn(p.bn, st, dim3(p.mtiles, p.ntiles, p.splits), mx, mg, a));
-        const int64_t total = (int64_t)taps * ci * co;
-        wgrad_reduce<<<(int)std::min<int64_t>((total + 255) / 256, 4096), 256, 0, st>>>(part, p.splits, taps, ci, co,
-                                                                                       gw, p.swap ? 1 : 0);
-        RSV_CUDA_TRY(cudaGetLastError());
-        int n = 2;
-        if (gb) {
-            const int64_t V = (int64_t)v.nx * v.ny * v.nz;
-            bias_grad_cl<<<kBiasBlocks, 256, 0, st>>>(gy, ldgy, co, V, bpart);
-            bias_grad_cl_final<<<(co + 7) / 8, 256, 0, st>>>(bpart, kBiasBlocks, co, gb);
-            RSV_CUDA_TRY(cudaGetLastError());
-            n = 4;
-        }
-        count_launches(n);
-        return RSV_OK;
+        return reduce(part, p.splits, p.swap ? 1 : 0, bpart);
     }
     __nv_bfloat16 *xt = (__nv_bfloat16 *)scratch;
     __nv_bfloat16 *gyt = (__nv_bfloat16 *)((char *)scratch + p.xt_bytes);
@@ -1270,9 +1527,7 @@ rsv_status conv_wgrad(cudaStream_t st, ConvVol v, int taps, int ci, int co, cons
     a.err = err;
     a.timeout_ns = timeout_ns;
     RSV_CUDA_TRY(launch_wg(p.bn, st, dim3(p.mtiles, p.ntiles, p.splits), ma, mb, a));
-    const int64_t total = (int64_t)taps * ci * co;
-    wgrad_reduce<<<(int)std::min<int64_t>((total + 255) / 256, 4096), 256, 0, st>>>(part, p.splits, taps, ci, co, gw,
-                                                                                   0);
+    wgrad_reduce<<<wblocks, 256, 0, st>>>(part, p.splits, taps, ci, co, gw, 0, wblocks, nullptr, 0, nullptr);
     RSV_CUDA_TRY(cudaGetLastError());
     int n = 4;
     if (gb) {

@@ -183,3 +183,43 @@ def test_conv_narrow_layers_match_oracle(rsv, case):
     absref = U.conv3(np.abs(xh), np.abs(wh)) + np.abs(bias)
     got = y32.cpu().numpy().reshape(ref.shape)
     assert np.all(np.abs(got - ref) <= 2 * (27 * ci + 1) * U32 * absref)
+
+
+# The weight gradient by whole rows of a plane: odd and single rows, rows of 8 and 128 voxels, two shared-memory stages
+# (128 x 64 channels), every block of rows (128, 64, 32 channels) in both roles, more channels than a thread block
+# has in the bias gradient; a leading dimension that 16-byte loads cannot take; rows too long for it.
+ROW_CASES = [
+    # (nx, ny, nz, ci, co, extra ldx)
+    (8, 1, 1, 32, 32, 8),
+    (8, 5, 3, 32, 512, 0),
+    (24, 7, 5, 96, 64, 0),
+    (40, 3, 9, 64, 64, 8),
+    (120, 3, 2, 32, 64, 0),
+    (104, 3, 2, 64, 64, 0),
+    (128, 4, 2, 64, 64, 0),
+    (128, 3, 3, 32, 32, 0),
+    (64, 21, 4, 64, 128, 0),
+    (16, 6, 5, 128, 96, 0),
+    (24, 5, 3, 64, 32, 4),
+    (136, 3, 2, 32, 32, 0),
+]
+
+
+@pytest.mark.parametrize("case", ROW_CASES, ids=["{}x{}x{}_ci{}_co{}_pad{}".format(*c) for c in ROW_CASES])
+def test_conv_wgrad_rows(rsv, case):
+    torch = pytest.importorskip("torch")
+    nx, ny, nz, ci, co, pad = case
+    rng = np.random.default_rng(500 + sum(case))
+    xt, xh = _bf16(torch, _vol(rng, nz, ny, nx, ci, ci + pad))
+    gyt, gyh = _bf16(torch, _vol(rng, nz, ny, nx, co))
+    gw = torch.full((co, 27, ci), float("nan"), device="cuda")
+    gb = torch.full((co,), float("nan"), device="cuda")
+    st = rsv.rsv_conv3d_wgrad(None, nx, ny, nz, 27, ci, co, _p(xt), ci + pad, _p(gyt), co, _p(gw), _p(gb))
+    assert st == rsv.RSV_OK, rsv.status_string(st)
+    x = xh[..., :ci]
+    ref, absref = U.conv3_wgrad(gyh, x), U.conv3_wgrad(np.abs(gyh), np.abs(x))
+    nvox = nx * ny * nz
+    # one FP32 rounding per product and addition of at most nvox terms
+    assert np.all(np.abs(gw.cpu().double().numpy() - ref) <= 2 * nvox * U32 * absref + 1e-30)
+    flat = gyh.reshape(-1, co)
+    assert np.all(np.abs(gb.cpu().double().numpy() - flat.sum(0)) <= 2 * nvox * U32 * np.abs(flat).sum(0) + 1e-30)
