@@ -282,10 +282,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 // The weights stay in shared memory when they fit beside three input boxes (32 -> 32 and 64 -> 32 channels);
 // else each stage carries its own.  Persistent CTAs; with 32 output channels the epilogue of a pair of tiles
 // overlaps the next pair's MMAs (two accumulator sets of 192 columns).
-// One call, 128x128x64: 32 -> 32 channels 185 -> 96 us (kernel 175 -> 72), 96 -> 32 473 -> 200 us; 64x64x32:
-// 64 -> 64 72 -> 58 us (kernel 56 -> 42), 192 -> 64 142 -> 95 us; 32x32x16 and below: both forms the same, the call's
-// fixed 25 us.  What bounds it now is the rate of the MMAs, about 140 cycles each whatever N (M = 128 rows of A from shared
-// memory); marching along z with two of three boxes kept (a third of the loads) gave nothing (97 us).
+// One call, 128x128x64: 32 -> 32 channels 185 -> 84 us (kernel 175 -> 67), 96 -> 32 473 -> 200 us; 64x64x32:
+// 64 -> 64 72 -> 55 us (kernel 56 -> 40), 192 -> 64 142 -> 95 us; 32x32x16 and below: both forms the same, the call's
+// fixed 25 us.  What bounds it now is TMA, about three cycles per row of a box whatever its bytes.
 struct FoldArgs {
     FwdArgs f;              // bw = nx, bh rows per tile, bd = 1, ty: pairs along y
     int pairs, S;           // pairs of tiles; pipeline stages
@@ -361,49 +360,68 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
             mbar_expect_tx(bready, (uint32_t)nk * BST);
             for (int q = 0; q < nk; ++q) weights(sm + q * BST, q / a.nkb, q % a.nkb, bready);
         }
-        int kk = 0;
+        int kk = 0, s = 0;
+        unsigned parity = 1;
         bool ok = true;
         for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x) {
             const int y0 = (p % a.ty) * 2 * a.bh, z0 = p / a.ty;
+            int dz = 0, cb = 0;
             for (int q = 0; q < nk; ++q, ++kk) {
-                const int s = kk % g.S;
-                if (kk >= g.S && !mbar_wait(&empty[s], ((kk / g.S) + 1) & 1, deadline)) {
+                if (kk >= g.S && !mbar_wait(&empty[s], parity, deadline)) {
                     ok = false;
                     break;
                 }
-                const int dz = q / a.nkb, cb = q % a.nkb;
                 uint8_t *st = sm + g.offA + s * stride;
                 mbar_expect_tx(&full[s], g.boxA + (g.resident ? 0u : BST));
                 tma_load_4d(st, &tmA, cb * 32, 0, y0 - 1, z0 + dz - 1, &full[s]);
                 if (!g.resident) weights(st + g.strideA, dz, cb, &full[s]);
+                if (++cb == a.nkb) {
+                    cb = 0;
+                    ++dz;
+                }
+                if (++s == g.S) {
+                    s = 0;
+                    parity ^= 1u;
+                }
             }
         }
         if (!ok) flags[0] = 1;
         flags[1] = kk;
     } else if (warp == 1 && lane == 0) {
         constexpr uint32_t idesc = idesc_bf16(128, BN);
-        int kk = 0, it = 0;
+        const uint32_t hi = (uint32_t)(kmajor_desc(0, 64) >> 32);
+        const uint32_t lo_a = (uint32_t)kmajor_desc(smem_u32(sm + g.offA), 64), lo_b = (uint32_t)kmajor_desc(smem_u32(sm), 64);
+        uint32_t off[2][3];  // (tile, dy) in an input box
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+#pragma unroll
+            for (int dy = 0; dy < 3; ++dy) off[m][dy] = (uint32_t)((m * a.bh + dy) * a.bw) * 4u;
+        int it = 0, s = 0;
+        unsigned parity = 0;
         bool ok = !g.resident || mbar_wait(bready, 0, deadline);
         for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x, ++it) {
             const int buf = it % NBUF;
             const uint32_t acc = tmem + buf * (2 * BN);
             if (it >= NBUF && !(ok = mbar_wait(&accempty[buf], ((it / NBUF) + 1) & 1, deadline))) break;
             fence_after_sync();
-            for (int q = 0; q < nk; ++q, ++kk) {
-                const int s = kk % g.S;
-                if (!(ok = mbar_wait(&full[s], (kk / g.S) & 1, deadline))) break;
+            for (int q = 0; q < nk; ++q) {
+                if (!(ok = mbar_wait(&full[s], parity, deadline))) break;
                 fence_after_sync();
-                const uint32_t sa = smem_u32(sm + g.offA + s * stride);
-                const uint32_t sb = g.resident ? smem_u32(sm + q * BST) : sa + g.strideA;
+                const uint32_t da = lo_a + s * (stride >> 4);
+                const uint32_t db = g.resident ? lo_b + q * (BST >> 4) : da + (g.strideA >> 4);
 #pragma unroll
                 for (int m = 0; m < 2; ++m)
 #pragma unroll
                     for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
                         for (int j = 0; j < 2; ++j)
-                            mma_bf16(acc + m * BN, kmajor_desc(sa + (uint32_t)((m * a.bh + dy) * a.bw) * 64u + j * 32, 64),
-                                     kmajor_desc(sb + dy * BDY + j * 32, 64), idesc, (q > 0 || dy > 0 || j > 0) ? 1u : 0u);
+                            mma_bf16(acc + m * BN, da + off[m][dy] + 2 * j, hi, db + dy * (BDY >> 4) + 2 * j, hi, idesc,
+                                     (q > 0 || dy > 0 || j > 0) ? 1u : 0u);
                 mma_commit(&empty[s]);
+                if (++s == g.S) {
+                    s = 0;
+                    parity ^= 1u;
+                }
             }
             if (ok) mma_commit(&accfull[buf]);
         }
@@ -860,7 +878,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         flags[1] = kk;
     } else if (warp == 1 && lane == 0) {
         constexpr uint32_t idesc = idesc_bf16(128, N, true, true);
-        const int swzA = colA == 64 ? 128 : 64, swzB = CN == 64 ? 128 : 64;
+        const uint64_t a0 = mnmajor_desc(smem_u32(sm), colA == 64 ? 128 : 64, boxA, 8 * rowA);
+        const uint64_t b0 = mnmajor_desc(smem_u32(sm + a.offN), CN == 64 ? 128 : 64, a.nx * rowB, 8 * rowB);
+        const uint32_t ahi = (uint32_t)(a0 >> 32), bhi = (uint32_t)(b0 >> 32);
         int kk = 0, s = 0;
         unsigned parity = 0;
         for (; kk < nk; ++kk) {
@@ -869,10 +889,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 break;
             }
             fence_after_sync();
-            const uint32_t sa = smem_u32(sm + s * a.stride), sb = sa + a.offN;
-            for (int k = 0; k < K; k += 16)
-                mma_bf16(tmem, mnmajor_desc(sa + k * rowA, swzA, boxA, 8 * rowA),
-                         mnmajor_desc(sb + k * rowB, swzB, a.nx * rowB, 8 * rowB), idesc, (kk > 0 || k > 0) ? 1u : 0u);
+            uint32_t da = (uint32_t)a0 + s * (a.stride >> 4), db = (uint32_t)b0 + s * (a.stride >> 4);
+#pragma unroll 4
+            for (int k = 0; k < K; k += 16) {  // 16 voxels on: 16 rows of the operand's bytes
+                mma_bf16(tmem, da, ahi, db, bhi, idesc, (kk > 0 || k > 0) ? 1u : 0u);
+                da += rowA;
+                db += rowB;
+            }
             mma_commit(&empty[s]);
             if (++s == a.S) {
                 s = 0;
