@@ -113,19 +113,23 @@ struct FwdArgs {
     const int *gate;      // skip the launch when *gate != 0 (may be null)
 };
 
-// Epilogue of 16 output channels n .. n + 15 of voxel v: bias, ReLU, mask, FP32 and BF16 stores.
-__device__ __forceinline__ void store16(const FwdArgs &a, int64_t v, int n, float acc[16]) {
-    if (a.bias) {
+// Epilogue of 16 output channels n .. n + 15 of voxel v: bias (at n of a.bias), ReLU, mask (its 16 values), FP32 and BF16
+// stores.
+__device__ __forceinline__ void load_mask16(const FwdArgs &a, int64_t v, int n, uint4 mv[2]) {
+    const uint4 *mp = (const uint4 *)(a.mask + v * a.ldm + n);
+    mv[0] = mp[0];
+    mv[1] = mp[1];
+}
+__device__ __forceinline__ void store16(const FwdArgs &a, int64_t v, int n, float acc[16], const float *bias, const uint4 mv[2]) {
+    if (bias) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) acc[i] += __ldg(a.bias + n + i);
+        for (int i = 0; i < 16; ++i) acc[i] += bias[i];
     }
     if (a.relu) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) acc[i] = fmaxf(acc[i], 0.0f);
     }
     if (a.mask) {
-        const uint4 *mp = (const uint4 *)(a.mask + v * a.ldm + n);
-        uint4 mv[2] = {mp[0], mp[1]};
         const __nv_bfloat16 *mb = (const __nv_bfloat16 *)mv;
 #pragma unroll
         for (int i = 0; i < 16; ++i)
@@ -255,7 +259,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         float acc[16];
         tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, acc);
         if (!valid) continue;
-        store16(a, v, n0 + c0, acc);
+        uint4 mv[2];
+        if (a.mask) load_mask16(a, v, n0 + c0, mv);
+        store16(a, v, n0 + c0, acc, a.bias ? a.bias + n0 + c0 : nullptr, mv);
     }
 
     fence_before_sync();
@@ -279,22 +285,31 @@ __global__ void __launch_bounds__(kThreads, 1)
 // stacked in y read one box of 2 bh + 2 rows per dz, each (tile, dy) an operand that starts a multiple
 // of nx rows into it.  Per 128 voxels and 32 input channels that is 48 KB of operands from L2 instead of 216, and a
 // third of the MMAs.
-// The weights stay in shared memory when they fit beside three input boxes (32 -> 32 and 64 -> 32 channels);
-// else each stage carries its own.  Persistent CTAs; with 32 output channels the epilogue of a pair of tiles
-// overlaps the next pair's MMAs (two accumulator sets of 192 columns).
-// One call, 128x128x64: 32 -> 32 channels 185 -> 84 us (kernel 175 -> 67), 96 -> 32 473 -> 200 us; 64x64x32:
-// 64 -> 64 72 -> 55 us (kernel 56 -> 40), 192 -> 64 142 -> 95 us; 32x32x16 and below: both forms the same, the call's
-// fixed 25 us.  What bounds it now is TMA, about three cycles per row of a box whatever its bytes.
+// A CTA takes consecutive pairs along z.  With one block of channels (32, or 64 where ci is a multiple of 64) it keeps
+// the boxes of three planes, so each is loaded once instead of three times ("march").  The weights stay in shared memory
+// when they fit beside the boxes (32 -> 32 and 32 -> 64 channels); else the 3 co rows of one (dz, dy) at a time pass
+// through a ring.  With 32 output channels the epilogue of a pair of tiles overlaps the next pair's MMAs (two
+// accumulator sets of 192 columns).
+// What bounds it: with 32 output channels the issue of the MMAs, 75 cycles each where the tensor core takes 61 (N = 96),
+// and the epilogue of about the same length beside it; with 64 the MMAs (102 cycles, N = 192) and then the epilogue.
+// Kernel, 128x128x64: 32 -> 32 channels 175 us with a box per tap, 67 with three boxes per pair, descriptors by one lane
+// and eight epilogue warps, 57 now; 64x64x32: 64 -> 64 56, 40, 34.  Calls: 128x128x64, 64 -> 64 243 -> 207 us, 96 -> 32
+// 171 either way; 104x77x40, 64 -> 32 70 -> 61; 32x32x16 and below the call's fixed 30.
 struct FoldArgs {
     FwdArgs f;              // bw = nx, bh rows per tile, bd = 1, ty: pairs along y
-    int pairs, S;           // pairs of tiles; pipeline stages
+    int nz, pairs;          // planes; pairs of tiles
+    int S, SB;              // slots for input boxes; for the weights of one (dz, channel block, dy), 0: all resident
+    int march;
     uint32_t boxA, strideA; // bytes of an input box, and its room (a tile's 128 rows may pass the box's end)
-    int resident;           // weights resident
-    uint32_t offA, offBar;  // shared-memory offsets (the resident weights come first)
+    uint32_t offA, offBar;  // shared-memory offsets (the weights come first)
 };
 
-constexpr int kFoldThreads = 320;  // producer, MMA issuer, four epilogue warps for each tile of the pair
-constexpr int kFoldMaxStages = 6;
+// Producer, MMA issuer, and four epilogue warps for each half of the channels of each tile of the pair: with four for
+// all channels the epilogue, a chain of latencies, took as long as the MMAs (32 channels), or 5,400 cycles between them
+// (64).
+constexpr int kFoldThreads = 576;
+constexpr uint32_t kFoldTail = 512 + 256 + 4096;  // barriers, bias, the epilogue's exchange
+constexpr int kFoldMaxStages = 6, kFoldMaxWeights = 16;
 
 // Whether `ok` holds for all four warps at named barrier `bar`.
 __device__ __forceinline__ bool all_of_128(int bar, bool ok) {
@@ -307,43 +322,95 @@ __device__ __forceinline__ bool all_of_128(int bar, bool ok) {
     return r != 0;
 }
 
-template <int CO>
+// y taps per slot of the weights' ring.  A wait and a release per slot cost the issuing warp about as much as two MMAs:
+// the smallest weights (32 rows of 32 channels, four MMAs per y tap) take all three (96 -> 32 channels on 128x128x64:
+// 219 us a call with one each, 171 so).
+__host__ __device__ constexpr int fold_dys(int co, int bk) { return co == 32 && bk == 32 ? 3 : 1; }
+
+// A position in a ring: slot and the parity of its current phase.
+struct RingPos {
+    int s = 0;
+    unsigned parity = 0;
+    __device__ __forceinline__ void next(int S) {
+        if (++s == S) {
+            s = 0;
+            parity ^= 1u;
+        }
+    }
+};
+
+// The pairs of tiles of a CTA.  March: consecutive ones, z fastest.  Else every gridDim-th, y fastest: neighbours in y,
+// which share rows, run at the same time and find them in L2 (64 -> 32 channels on 128x128x64: 132 us a call with
+// consecutive pairs, 120 so).
+struct FoldWalk {
+    int p0, step, n, ty, nz;
+    __device__ __forceinline__ explicit FoldWalk(const FoldArgs &g) : ty(g.f.ty), nz(g.nz) {
+        if (g.march) {
+            p0 = (int)((int64_t)blockIdx.x * g.pairs / gridDim.x);
+            n = (int)((int64_t)(blockIdx.x + 1) * g.pairs / gridDim.x) - p0;
+            step = 0;
+        } else {
+            p0 = blockIdx.x;
+            step = gridDim.x;
+            n = (g.pairs - p0 + step - 1) / step;
+        }
+    }
+    __device__ __forceinline__ void at(int it, int &yp, int &z) const {
+        if (step) {
+            const int p = p0 + it * step;
+            z = p / ty;
+            yp = p - z * ty;
+        } else {
+            yp = (p0 + it) / nz;
+            z = p0 + it - yp * nz;
+        }
+    }
+};
+
+template <int CO, int BK>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     conv_fold_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const FoldArgs g) {
     const FwdArgs &a = g.f;
     if (a.gate && *a.gate) return;  // uniform across the CTA, before any barrier or allocation
-    constexpr int BN = 3 * CO;
-    constexpr int NBUF = CO == 32 ? 2 : 1;        // accumulator sets
-    constexpr uint32_t BDY = BN * 64u, BST = 3 * BDY;  // weight bytes of one dy, and of one (dz, channel block)
+    constexpr int BN = 3 * CO, SWZ = 2 * BK;       // SWZ: bytes of an operand row
+    constexpr int NBUF = CO == 32 ? 2 : 1;         // accumulator sets
+    constexpr uint32_t BDY = BN * SWZ;             // weight bytes of one (dz, channel block, dy)
+    constexpr int DYS = fold_dys(CO, BK);          // y taps in a weight slot
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     uint8_t *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
     uint64_t *full = (uint64_t *)(sm + g.offBar);
     uint64_t *empty = full + kFoldMaxStages, *accfull = empty + kFoldMaxStages, *accempty = accfull + 2;
-    uint64_t *bready = accempty + 2, *done = bready + 1;
+    uint64_t *bfull = accempty + 2, *bempty = bfull + kFoldMaxWeights, *done = bempty + kFoldMaxWeights;
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
-    int *flags = (int *)(tmem_slot + 1);  // [0] failed, [1] loads issued
-    float *xch = (float *)(sm + g.offBar + 512);  // [tile][2][4 warps][2][16]: boundary lanes' values of a chunk
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int *flags = (int *)(tmem_slot + 1);  // [0] failed, [1] boxes and [2] weight loads issued
+    float *sbias = (float *)(sm + g.offBar + 512);
+    float *xch = sbias + 64;  // [tile, half][2][4 warps][2][16]: boundary lanes' values of a chunk
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint64_t deadline = now_ns() + a.timeout_ns;
-    const int nk = 3 * a.nkb;  // stages per pair
-    const uint32_t stride = g.strideA + (g.resident ? 0u : BST);
+    const int nk = 3 * a.nkb;  // boxes (dz, channel block) that a pair reads
+    const FoldWalk walk(g);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < g.S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
+        for (int s = 0; s < max(g.SB, 1); ++s) {
+            mbar_init(&bfull[s], 1);
+            mbar_init(&bempty[s], 1);
+        }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&accfull[b], 1);
-            mbar_init(&accempty[b], 8);
+            mbar_init(&accempty[b], 16);
         }
-        mbar_init(bready, 1);
         mbar_init(done, 1);
-        flags[0] = flags[1] = 0;
+        flags[0] = flags[1] = flags[2] = 0;
         fence_mbar_init();
     }
     if (warp == 1) tmem_alloc(tmem_slot, 512);
+    if (a.bias && warp == 2)
+        for (int c = lane; c < CO; c += 32) sbias[c] = a.bias[c];
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -352,100 +419,127 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     if (warp == 0 && lane == 0) {
         prefetch_map(&tmA);
         prefetch_map(&tmB);
-        auto weights = [&](uint8_t *dst, int dz, int cb, uint64_t *bar) {
-            for (int t = 0; t < 9; ++t)  // rows (dy, dx, output channel)
-                tma_load_2d(dst + t * (CO * 64), &tmB, (dz * 9 + t) * a.ci + cb * 32, 0, bar);
-        };
-        if (g.resident) {
-            mbar_expect_tx(bready, (uint32_t)nk * BST);
-            for (int q = 0; q < nk; ++q) weights(sm + q * BST, q / a.nkb, q % a.nkb, bready);
-        }
-        int kk = 0, s = 0;
-        unsigned parity = 1;
+        int boxes = 0, loads = 0;
         bool ok = true;
-        for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x) {
-            const int y0 = (p % a.ty) * 2 * a.bh, z0 = p / a.ty;
+        if (!g.SB) {  // rows (dz, channel block, dy, dx, output channel)
+            mbar_expect_tx(&bfull[0], (uint32_t)nk * 3 * BDY);
+            for (int q = 0; q < nk; ++q)
+                for (int dy = 0; dy < 3; dy += DYS)
+                    tma_load_3d(sm + (q * 3 + dy) * BDY, &tmB, (q % a.nkb) * BK, 0, (q / a.nkb) * 9 + dy * 3, &bfull[0]);
+            loads = 1;
+        }
+        // everything in the order in which the MMAs use it
+        RingPos box, wt;
+        for (int it = 0; ok && it < walk.n; ++it) {
+            int yp, z;
+            walk.at(it, yp, z);
+            const bool start = it == 0 || z == 0;
             int dz = 0, cb = 0;
-            for (int q = 0; q < nk; ++q, ++kk) {
-                if (kk >= g.S && !mbar_wait(&empty[s], parity, deadline)) {
-                    ok = false;
-                    break;
+            for (int q = 0; ok && q < nk; ++q) {
+                if (!g.march || start || q == 2) {
+                    if (boxes >= g.S && !(ok = mbar_wait(&empty[box.s], box.parity ^ 1u, deadline))) break;
+                    mbar_expect_tx(&full[box.s], g.boxA);
+                    tma_load_4d(sm + g.offA + box.s * g.strideA, &tmA, cb * BK, 0, yp * 2 * a.bh - 1, z + dz - 1, &full[box.s]);
+                    box.next(g.S);
+                    ++boxes;
                 }
-                uint8_t *st = sm + g.offA + s * stride;
-                mbar_expect_tx(&full[s], g.boxA + (g.resident ? 0u : BST));
-                tma_load_4d(st, &tmA, cb * 32, 0, y0 - 1, z0 + dz - 1, &full[s]);
-                if (!g.resident) weights(st + g.strideA, dz, cb, &full[s]);
+                for (int dy = 0; g.SB && dy < 3; dy += DYS) {
+                    if (loads >= g.SB && !(ok = mbar_wait(&bempty[wt.s], wt.parity ^ 1u, deadline))) break;
+                    mbar_expect_tx(&bfull[wt.s], DYS * BDY);
+                    tma_load_3d(sm + wt.s * (DYS * BDY), &tmB, cb * BK, 0, dz * 9 + dy * 3, &bfull[wt.s]);
+                    wt.next(g.SB);
+                    ++loads;
+                }
                 if (++cb == a.nkb) {
                     cb = 0;
                     ++dz;
                 }
-                if (++s == g.S) {
-                    s = 0;
-                    parity ^= 1u;
-                }
             }
         }
         if (!ok) flags[0] = 1;
-        flags[1] = kk;
-    } else if (warp == 1 && lane == 0) {
+        flags[1] = boxes;
+        flags[2] = loads;
+    } else if (warp == 1) {  // in step; one lane issues
+        const uint32_t lead = elect_one();
         constexpr uint32_t idesc = idesc_bf16(128, BN);
-        const uint32_t hi = (uint32_t)(kmajor_desc(0, 64) >> 32);
-        const uint32_t lo_a = (uint32_t)kmajor_desc(smem_u32(sm + g.offA), 64), lo_b = (uint32_t)kmajor_desc(smem_u32(sm), 64);
+        const uint32_t hi = (uint32_t)(kmajor_desc(0, SWZ) >> 32);
+        const uint32_t lo_a = (uint32_t)kmajor_desc(smem_u32(sm + g.offA), SWZ), lo_b = (uint32_t)kmajor_desc(smem_u32(sm), SWZ);
         uint32_t off[2][3];  // (tile, dy) in an input box
 #pragma unroll
         for (int m = 0; m < 2; ++m)
 #pragma unroll
-            for (int dy = 0; dy < 3; ++dy) off[m][dy] = (uint32_t)((m * a.bh + dy) * a.bw) * 4u;
-        int it = 0, s = 0;
-        unsigned parity = 0;
-        bool ok = !g.resident || mbar_wait(bready, 0, deadline);
-        for (int p = blockIdx.x; ok && p < g.pairs; p += gridDim.x, ++it) {
+            for (int dy = 0; dy < 3; ++dy) off[m][dy] = (uint32_t)((m * a.bh + dy) * a.bw) * (SWZ / 16);
+        const bool march = g.march;
+        const int S = g.S;
+        RingPos box, wt;
+        bool ok = g.SB || warp_wait(&bfull[0], 0, deadline);
+        for (int it = 0; ok && it < walk.n; ++it) {
             const int buf = it % NBUF;
             const uint32_t acc = tmem + buf * (2 * BN);
-            if (it >= NBUF && !(ok = mbar_wait(&accempty[buf], ((it / NBUF) + 1) & 1, deadline))) break;
+            if (it >= NBUF && !(ok = warp_wait(&accempty[buf], ((it / NBUF) + 1) & 1, deadline))) break;
             fence_after_sync();
-            for (int q = 0; q < nk; ++q) {
-                if (!(ok = mbar_wait(&full[s], parity, deadline))) break;
-                fence_after_sync();
-                const uint32_t da = lo_a + s * (stride >> 4);
-                const uint32_t db = g.resident ? lo_b + q * (BST >> 4) : da + (g.strideA >> 4);
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-                        for (int j = 0; j < 2; ++j)
-                            mma_bf16(acc + m * BN, da + off[m][dy] + 2 * j, hi, db + dy * (BDY >> 4) + 2 * j, hi, idesc,
-                                     (q > 0 || dy > 0 || j > 0) ? 1u : 0u);
-                mma_commit(&empty[s]);
-                if (++s == g.S) {
-                    s = 0;
-                    parity ^= 1u;
+            const bool last = it + 1 == walk.n || (walk.p0 + it + 1) % walk.nz == 0;  // the next pair, if any, starts with new boxes
+            for (int q = 0; ok && q < nk; ++q) {
+                RingPos b = box;  // march: the planes z - 1, z, z + 1 lie one after another in the ring
+                if (march && (b.s += q) >= S) {
+                    b.s -= S;
+                    b.parity ^= 1u;
                 }
+                if (!(ok = warp_wait(&full[b.s], b.parity, deadline))) break;
+                const uint32_t da = lo_a + b.s * (g.strideA >> 4);
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy) {
+                    if (dy % DYS == 0) {
+                        if (g.SB && !(ok = warp_wait(&bfull[wt.s], wt.parity, deadline))) break;
+                        fence_after_sync();
+                    }
+                    const uint32_t db = lo_b + ((g.SB ? wt.s * DYS + dy % DYS : q * 3 + dy)) * (BDY >> 4);
+#pragma unroll
+                    for (int m = 0; m < 2; ++m)
+#pragma unroll
+                        for (int j = 0; j < BK / 16; ++j)
+                            mma_bf16(lead, acc + m * BN, da + off[m][dy] + 2 * j, hi, db + 2 * j, hi, idesc,
+                                     (q > 0 || dy > 0 || j > 0) ? 1u : 0u);
+                    if (g.SB && dy % DYS == DYS - 1) {
+                        mma_commit(lead, &bempty[wt.s]);
+                        wt.next(g.SB);
+                    }
+                }
+                if (!march || q == 0 || last) mma_commit(lead, &empty[b.s]);
+                if (!march) box.next(S);
             }
-            if (ok) mma_commit(&accfull[buf]);
+            if (march)
+                for (int i = 0; i < (last ? 3 : 1); ++i) box.next(S);
+            if (ok) mma_commit(lead, &accfull[buf]);
         }
-        if (!ok) flags[0] = 1;
-        mma_commit(done);
+        if (!ok && lane == 0) flags[0] = 1;
+        mma_commit(lead, done);
     } else if (warp >= 2) {
-        // a warp reads the quarter of the TMEM lanes that its index allows; warps 2..5 take tile 0, 6..9 tile 1
-        const int quarter = warp & 3, row = quarter * 32 + lane, m = warp >= 6;
+        // a warp reads the quarter of the TMEM lanes that its index allows
+        constexpr int NCH = CO / 32;  // chunks of 16 channels per warp
+        const int quarter = warp & 3, row = quarter * 32 + lane, grp = (warp - 2) >> 2, m = grp >> 1, n0 = (grp & 1) * (CO / 2);
         const int rx = row % a.bw, ry = row / a.bw;
         const bool left = rx > 0, right = rx < a.bw - 1;
-        float *const mine = xch + m * 256 + quarter * 32;
-        int it = 0;
+        float *const mine = xch + grp * 256 + quarter * 32;
         unsigned chunk = 0;
-        for (int p = blockIdx.x; p < g.pairs; p += gridDim.x, ++it) {
+        for (int it = 0; it < walk.n; ++it) {
             const int buf = it % NBUF;
-            // the four warps of a tile share barriers: they go on, or give up, together
-            if (!all_of_128(1 + m, mbar_wait(&accfull[buf], (it / NBUF) & 1, deadline))) break;
-            fence_after_sync();
-            const uint32_t acc0 = tmem + buf * (2 * BN) + m * BN + ((uint32_t)(quarter * 32) << 16);
-            const int z = p / a.ty, y = (p - z * a.ty) * 2 * a.bh + m * a.bh + ry;
+            int yp, z;
+            walk.at(it, yp, z);
+            const int y = (yp * 2 + m) * a.bh + ry;
             const bool valid = ry < a.bh && y < a.ny;
             const int64_t v = ((int64_t)z * a.ny + y) * a.nx + rx;
-#pragma unroll 1
-            for (int n = 0; n < CO; n += 16, ++chunk) {
+            uint4 mv[NCH][2];
+            if (a.mask && valid)  // under the MMAs
+#pragma unroll
+                for (int u = 0; u < NCH; ++u) load_mask16(a, v, n0 + 16 * u, mv[u]);
+            // the four warps of a group share barriers: they go on, or give up, together
+            if (!all_of_128(1 + grp, mbar_wait(&accfull[buf], (it / NBUF) & 1, deadline))) break;
+            fence_after_sync();
+            const uint32_t acc0 = tmem + buf * (2 * BN) + m * BN + ((uint32_t)(quarter * 32) << 16);
+#pragma unroll
+            for (int u = 0; u < NCH; ++u, ++chunk) {
+                const int n = n0 + 16 * u;
                 uint32_t pm[16], pc[16], pp[16];
                 tmem_ld16_start(acc0 + n, pm);
                 tmem_ld16_start(acc0 + CO + n, pc);
@@ -460,22 +554,22 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
 #pragma unroll
                     for (int i = 0; i < 16; i += 4)
                         *(uint4 *)(slot + 16 + i) = make_uint4(pp[i], pp[i + 1], pp[i + 2], pp[i + 3]);
-                if (n + 16 >= CO) {  // the accumulators are in registers: the next pair may overwrite them
+                if (u == NCH - 1) {  // the accumulators are in registers: the next pair may overwrite them
                     fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&accempty[buf]);
                 }
-                asm volatile("bar.sync %0, 128;" ::"r"(1 + m) : "memory");
+                asm volatile("bar.sync %0, 128;" ::"r"(1 + grp) : "memory");
                 float acc[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
-                    float u = __uint_as_float(__shfl_up_sync(0xffffffffu, pm[i], 1));
-                    float d = __uint_as_float(__shfl_down_sync(0xffffffffu, pp[i], 1));
-                    if (lane == 0 && quarter > 0) u = slot[i - 32];
-                    if (lane == 31 && quarter < 3) d = slot[i + 48];
-                    acc[i] = ((left ? u : 0.0f) + __uint_as_float(pc[i])) + (right ? d : 0.0f);
+                    float before = __uint_as_float(__shfl_up_sync(0xffffffffu, pm[i], 1));
+                    float after = __uint_as_float(__shfl_down_sync(0xffffffffu, pp[i], 1));
+                    if (lane == 0 && quarter > 0) before = slot[i - 32];
+                    if (lane == 31 && quarter < 3) after = slot[i + 48];
+                    acc[i] = ((left ? before : 0.0f) + __uint_as_float(pc[i])) + (right ? after : 0.0f);
                 }
-                if (valid) store16(a, v, n, acc);
+                if (valid) store16(a, v, n, acc, a.bias ? sbias + n : nullptr, mv[u]);
             }
         }
     }
@@ -488,6 +582,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         // let copies still in flight land before the shared memory is released
         for (int kk = max(0, flags[1] - g.S); kk < flags[1]; ++kk)
             mbar_wait(&full[kk % g.S], (kk / g.S) & 1, now_ns() + a.timeout_ns);
+        const int SB = max(g.SB, 1);
+        for (int kk = max(0, flags[2] - SB); kk < flags[2]; ++kk)
+            mbar_wait(&bfull[kk % SB], (kk / SB) & 1, now_ns() + a.timeout_ns);
     }
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, 512);
@@ -824,7 +921,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t *tmem_slot = (uint32_t *)(done + 1);
     int *flags = (int *)(tmem_slot + 1);  // a wait ran out; steps issued; steps consumed
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int vg = blockIdx.x / a.nmb, mb = blockIdx.x % a.nmb;
     const int q0 = blockIdx.z * a.cps;
     const int nk = max(0, min(a.nchunks, q0 + a.cps) - q0);
@@ -876,7 +973,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         }
         flags[1] = kk;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {  // in step; one lane issues
+        const uint32_t lead = elect_one();
         constexpr uint32_t idesc = idesc_bf16(128, N, true, true);
         const uint64_t a0 = mnmajor_desc(smem_u32(sm), colA == 64 ? 128 : 64, boxA, 8 * rowA);
         const uint64_t b0 = mnmajor_desc(smem_u32(sm + a.offN), CN == 64 ? 128 : 64, a.nx * rowB, 8 * rowB);
@@ -884,26 +982,26 @@ __global__ void __launch_bounds__(kThreads, 1)
         int kk = 0, s = 0;
         unsigned parity = 0;
         for (; kk < nk; ++kk) {
-            if (!mbar_wait(&full[s], parity, deadline)) {
-                flags[0] = 1;
+            if (!warp_wait(&full[s], parity, deadline)) {
+                if (lane == 0) flags[0] = 1;
                 break;
             }
             fence_after_sync();
             uint32_t da = (uint32_t)a0 + s * (a.stride >> 4), db = (uint32_t)b0 + s * (a.stride >> 4);
 #pragma unroll 4
             for (int k = 0; k < K; k += 16) {  // 16 voxels on: 16 rows of the operand's bytes
-                mma_bf16(tmem, da, ahi, db, bhi, idesc, (kk > 0 || k > 0) ? 1u : 0u);
+                mma_bf16(lead, tmem, da, ahi, db, bhi, idesc, (kk > 0 || k > 0) ? 1u : 0u);
                 da += rowA;
                 db += rowB;
             }
-            mma_commit(&empty[s]);
+            mma_commit(lead, &empty[s]);
             if (++s == a.S) {
                 s = 0;
                 parity ^= 1u;
             }
         }
-        flags[2] = kk;
-        mma_commit(done);
+        if (lane == 0) flags[2] = kk;
+        mma_commit(lead, done);
     }
     __syncwarp();
 
@@ -1294,27 +1392,44 @@ size_t fold_plan(ConvVol v, int taps, int ci, int co, FoldArgs *g) {
     if (taps != 27 || (co != 32 && co != 64) || v.nx % 8 || v.nx > 128) return 0;
     const int bh = std::min(v.ny, 128 / v.nx);
     if (bh * v.nx < 64 || v.ny <= bh) return 0;
-    const uint32_t bst = 9u * co * 64, nk = 3 * (ci / 32);
-    g->boxA = (uint32_t)v.nx * (2 * bh + 2) * 64;
-    g->strideA = (g->boxA + (uint32_t)(128 - bh * v.nx) * 64 + 1023u) & ~1023u;
-    const uint32_t room = 227 * 1024 - 1024 - 3072;  // less alignment, barriers and the epilogue's exchange
-    g->resident = nk * bst + 3 * g->strideA <= room;
-    const uint32_t stride = g->strideA + (g->resident ? 0u : bst), base = g->resident ? nk * bst : 0u;
-    g->S = (int)std::min<uint32_t>(kFoldMaxStages, (room - base) / stride);
-    if (g->S < 2) return 0;
-    g->offA = base;
-    g->offBar = base + g->S * stride;
+    const int BK = ci % 64 == 0 ? 64 : 32, rb = 2 * BK, nkb = ci / BK;
+    const int dys = fold_dys(co, BK);
+    const uint32_t slot = 3u * co * rb * dys, all = 9u * nkb / dys * slot;
+    g->boxA = (uint32_t)v.nx * (2 * bh + 2) * rb;
+    g->strideA = (g->boxA + (uint32_t)(128 - bh * v.nx) * rb + 1023u) & ~1023u;
+    const uint32_t room = 227 * 1024 - 1024 - kFoldTail;  // less alignment
+    // weight slots that cover a load's latency: a slot's MMAs take 410 (co = 64, BK = 32) to 820 cycles
+    const int least = dys == 3 ? 2 : co == 64 && BK == 64 ? 3 : 4;
+    g->S = 0;
+    for (int march = nkb == 1; march >= 0 && !g->S; --march) {
+        // boxes: three planes; else two, or as many as there is room for with their weights
+        const int least_boxes = march ? 3 : 2;
+        const int boxes = march ? 3 : std::max(2, std::min<int>(kFoldMaxStages, room / (g->strideA + 3 / dys * slot)));
+        if (all + least_boxes * g->strideA <= room) {
+            g->SB = 0;
+            g->S = (int)std::min<uint32_t>(kFoldMaxStages, (room - all) / g->strideA);
+            g->offA = all;
+        } else if (boxes * g->strideA + least * slot <= room) {
+            g->SB = (int)std::min<uint32_t>(kFoldMaxWeights, (room - boxes * g->strideA) / slot);
+            g->S = (int)std::min<uint32_t>(kFoldMaxStages, (room - g->SB * slot) / g->strideA);
+            g->offA = g->SB * slot;
+        }
+        g->march = march;
+    }
+    if (!g->S) return 0;
+    g->offBar = g->offA + g->S * g->strideA;
     g->f.bh = bh;
     g->f.ty = (v.ny + 2 * bh - 1) / (2 * bh);
+    g->nz = v.nz;
     g->pairs = g->f.ty * v.nz;
-    return g->offBar + 3072 + 1024;
+    return g->offBar + kFoldTail + 1024;
 }
 
-template <int CO>
+template <int CO, int BK>
 cudaError_t launch_fold(cudaStream_t st, size_t smem, const CUtensorMap &ma, const CUtensorMap &mb, const FoldArgs &g) {
-    static cudaError_t attr = set_smem(conv_fold_tc<CO>, 227 * 1024);
+    static cudaError_t attr = set_smem(conv_fold_tc<CO, BK>, 227 * 1024);
     if (attr != cudaSuccess) return attr;
-    conv_fold_tc<CO><<<std::min(g.pairs, 152), kFoldThreads, smem, st>>>(ma, mb, g);
+    conv_fold_tc<CO, BK><<<std::min(g.pairs, 152), kFoldThreads, smem, st>>>(ma, mb, g);
     return cudaGetLastError();
 }
 
@@ -1365,16 +1480,17 @@ rsv_status conv_fwd(cudaStream_t st, ConvVol v, int taps, int ci, int co, const 
         g.f.bh = bh;
         g.f.bd = 1;
         g.f.ty = ty;
-        g.f.nkb = ci / 32;
+        g.f.nkb = ci / BK;
         const uint64_t dims[4] = {(uint64_t)ci, (uint64_t)v.nx, (uint64_t)v.ny, (uint64_t)v.nz};
         const uint64_t strides[3] = {(uint64_t)ldx * 2, (uint64_t)v.nx * ldx * 2, (uint64_t)v.nx * v.ny * ldx * 2};
-        const uint32_t box[4] = {32u, (uint32_t)v.nx, (uint32_t)(2 * bh + 2), 1u};
-        RSV_TRY(make_map(&ma, x, 4, dims, strides, box, 64));
-        const uint64_t wdims[2] = {(uint64_t)taps * ci, (uint64_t)co};
-        const uint64_t wstrides[1] = {(uint64_t)taps * ci * 2};
-        const uint32_t wbox[2] = {32u, (uint32_t)co};
-        RSV_TRY(make_map(&mb, w, 2, wdims, wstrides, wbox, 64));
-        RSV_CUDA_TRY(co == 32 ? launch_fold<32>(st, smem, ma, mb, g) : launch_fold<64>(st, smem, ma, mb, g));
+        const uint32_t box[4] = {(uint32_t)BK, (uint32_t)v.nx, (uint32_t)(2 * bh + 2), 1u};
+        RSV_TRY(make_map(&ma, x, 4, dims, strides, box, BK * 2));
+        const uint64_t wdims[3] = {(uint64_t)ci, (uint64_t)co, (uint64_t)taps};
+        const uint64_t wstrides[2] = {(uint64_t)taps * ci * 2, (uint64_t)ci * 2};
+        const uint32_t wbox[3] = {(uint32_t)BK, (uint32_t)co, 3u * fold_dys(co, BK)};  // the x taps of one or three (dz, dy)
+        RSV_TRY(make_map(&mb, w, 3, wdims, wstrides, wbox, BK * 2));
+        RSV_CUDA_TRY(co == 32 ? (BK == 32 ? launch_fold<32, 32>(st, smem, ma, mb, g) : launch_fold<32, 64>(st, smem, ma, mb, g))
+                              : (BK == 32 ? launch_fold<64, 32>(st, smem, ma, mb, g) : launch_fold<64, 64>(st, smem, ma, mb, g)));
         count_launches(1);
         return RSV_OK;
     }

@@ -142,15 +142,33 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64
 }
 // The same with the descriptors' words apart: operands of one layout differ in the low word only, by their distance
 // in 16-byte units.  One thread issues all MMAs, so the instructions between two of them count: rebuilding
-// descriptors per MMA took 140 cycles; the MMAs themselves take 46, 53, 61, 69, 102 and 133 cycles for N = 32, 64, 96,
-// 128, 192 and 256 (M = 128, either major order, either swizzle).
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+// descriptors per MMA took 140 cycles, one addition each in a lone lane 118, in a warp in step 75; the MMAs themselves
+// take 46, 53, 61, 69, 102 and 133 cycles for N = 32, 64, 96, 128, 192 and 256 (M = 128, either major order, either
+// swizzle).
+// For a whole warp in step: `lead` is set in the one lane that issues (elect_one).  The addresses are the same in all
+// lanes, so that the compiler can keep them in uniform registers, where the instruction takes its operands from.
+__device__ __forceinline__ uint32_t elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void mma_bf16(uint32_t lead, uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                          uint32_t idesc, uint32_t accumulate) {
     asm volatile(
-        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}" ::"r"(tmem_d),
-        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate)
+        "{\n .reg .pred p, l;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n setp.ne.b32 l, %7, 0;\n mov.b64 a, {%1, %2};\n"
+        " mov.b64 b, {%3, %4};\n @l tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}" ::"r"(tmem_d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate), "r"(lead)
         : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t lead, uint64_t *bar) {
+    asm volatile(
+        "{\n .reg .pred l;\n setp.ne.b32 l, %1, 0;\n"
+        " @l tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)), "r"(lead)
+        : "memory");
+}
+// The wait of a whole warp in step: the same answer in all lanes.
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, unsigned parity, uint64_t deadline) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, deadline));
 }
 // The mbarrier receives one arrival once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t *bar) {

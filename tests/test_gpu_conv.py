@@ -185,6 +185,19 @@ def test_conv_narrow_layers_match_oracle(rsv, case):
     assert np.all(np.abs(got - ref) <= 2 * (27 * ci + 1) * U32 * absref)
 
 
+# More pairs of tiles than CTAs, so that a CTA walks along z and over the end of a column: boxes of three planes kept
+# (weights resident: 32 channels; through a ring: 64), one box at a time (rows of 128 voxels, several channel blocks).
+WALK_CASES = [
+    (32, 40, 40, 32, 32), (40, 21, 50, 32, 64), (16, 66, 40, 64, 64), (64, 10, 60, 64, 32), (128, 4, 90, 64, 64),
+    (128, 3, 90, 64, 32), (32, 33, 40, 128, 64), (64, 7, 80, 96, 32),
+]
+
+
+@pytest.mark.parametrize("case", WALK_CASES, ids=[f"{c[0]}x{c[1]}x{c[2]}_ci{c[3]}_co{c[4]}" for c in WALK_CASES])
+def test_conv_narrow_layers_walk(rsv, case):
+    test_conv_narrow_layers_match_oracle(rsv, case)
+
+
 # The weight gradient by whole rows of a plane: odd and single rows, rows of 8 and 128 voxels, two shared-memory stages
 # (128 x 64 channels), every block of rows (128, 64, 32 channels) in both roles, more channels than a thread block
 # has in the bias gradient; a leading dimension that 16-byte loads cannot take; rows too long for it.
