@@ -605,7 +605,8 @@ cudaError_t launch_mdot2(cudaStream_t st, int64_t n, const T *w, const T *u, con
     if (k < 1 || k > kMaxRestart + 1) return cudaErrorInvalidValue;
     rsv::count_launches(1);
     if (small(n))
-        return launch_pdl(mdot2_kernel<T, false>, dim3((unsigned)((n + kRedThreads - 1) / kRedThreads), (k + kGroup / 2 - 1) / (kGroup / 2)),
+        return launch_pdl(mdot2_kernel<T, false>,
+                          dim3((unsigned)((n + kRedThreads - 1) / kRedThreads), (k + kGroup / 2 - 1) / (kGroup / 2)),
                           dim3(kRedThreads), 0, st, n, w, u, V, ldv, k, partial, ow, ou, counter, done);
     if (vec_ok<T>(ldv, {w, u, V}))
         return launch_pdl(mdot2_kernel<T, true>, dim3(kRedBlocks), dim3(kRedThreads), 0, st, n, w, u, V, ldv, k,
