@@ -149,6 +149,7 @@ constexpr int kMaxLevels = 8;
 struct Cpr {  // CPR pressure stage: quasi-IMPES weights and the GMG hierarchy (cpr.cu)
     bool mixed = false;
     int nlev = 0, sweeps = 2, ncoarse = 0;
+    int64_t ndense = 0;           // rows that dense, minv, work and piv are allocated for
     int dims[kMaxLevels][3] = {};
     double *a7[kMaxLevels] = {};  // FP64 seven-point stencils, slot-major [7][n]
     void *a7f[kMaxLevels] = {};   // FP32 copies (mixed precision)

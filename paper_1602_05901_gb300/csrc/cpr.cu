@@ -649,8 +649,11 @@ cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_lev
         dims[nl][0] = g.nx, dims[nl][1] = g.ny, dims[nl][2] = g.nz;
         ++nl;
     }
+    const int64_t nb = A->nb;
+    const int nc = (int)g.n();
+    const int64_t ncd = coarsening == 1 ? 1 : nc;  // the algebraic hierarchy keeps its own coarsest inverse
     // a new setup of the same hierarchy (the usual case: new values, same grid) reuses the buffers
-    bool same = P->w64 && P->mixed == mixed && P->nlev == nl;
+    bool same = P->w64 && P->mixed == mixed && P->nlev == nl && P->ndense == ncd;
     for (int l = 0; same && l < nl; ++l)
         for (int d = 0; d < 3; ++d) same = same && P->dims[l][d] == dims[l][d];
     if (!same) free_cpr(P);
@@ -659,9 +662,8 @@ cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_lev
     for (int l = 0; l < nl; ++l)
         for (int d = 0; d < 3; ++d) P->dims[l][d] = dims[l][d];
     P->nlev = nl;
-    const int64_t nb = A->nb;
-    const int nc = (int)g.n();
     P->ncoarse = nc;
+    P->ndense = ncd;
     cudaError_t e = cudaSuccess;
     auto alloc = [&](void **p, size_t bytes) {
         if (e == cudaSuccess && !same) e = cudaMalloc(p, std::max<size_t>(bytes, 16));
@@ -676,7 +678,6 @@ cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_lev
         alloc(&P->x[l], es * n);
         alloc(&P->b[l], es * n);
     }
-    const int64_t ncd = coarsening == 1 ? 1 : nc;  // the algebraic hierarchy keeps its own coarsest inverse
     alloc((void **)&P->dense, sizeof(double) * ncd * ncd);
     alloc((void **)&P->minv, sizeof(double) * ncd * ncd);
     alloc((void **)&P->work, sizeof(double) * ncd * (ncd + kGjB));
