@@ -686,7 +686,10 @@ cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_lev
     alloc(&P->z, es * 3 * nb);
     alloc(&P->xp, es * 3 * nb);
     alloc(&P->apc, es * 3 * (size_t)A->nnzb + 64);  // tail room: the residual kernels stage whole 16-byte units
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        free_cpr(P);  // else the next setup would take the buffers for complete
+        return e;
+    }
     G3 g0{A->nx, A->ny, A->nz};
     count_launches(1);
     if (mixed)

@@ -902,6 +902,15 @@ template <typename T> constexpr const void *sweep_kernel(bool fwd) {
 }
 template <typename T> constexpr int kSweepThreads = sizeof(T) == 4 ? 96 : 160;
 
+// Gives back what was allocated so far unless `whole` is set: the next setup must not take it for complete.
+struct FreeUnlessWhole {
+    IluTiles *Tl;
+    bool whole = false;
+    ~FreeUnlessWhole() {
+        if (!whole) free_tiles(Tl);
+    }
+};
+
 }  // namespace
 
 template <typename T>
@@ -910,6 +919,7 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
     cudaError_t e = cudaSuccess;
     if (!Tl->Ff || Tl->elem != (int)sizeof(T)) {
         free_tiles(Tl);
+        FreeUnlessWhole guard{Tl};
         // Tiles of every grid in order of TJ J + TK K, the planes its start lies behind the grid's first cell: a
         // CTA that is free takes the tile that can start soonest, in every grid of a batch at once.  (One grid after
         // another left CTAs waiting in the far tiles of the first grids: 24 grids of 16 to 96 cells a side, 220 -> 157 us
@@ -1008,6 +1018,7 @@ cudaError_t tiles_setup(const rsv_mat *A, const double *dinv, IluTiles *Tl) {
                 cudaSuccess)
             return e;
         Tl->grid = std::max(1, std::min(nT, sms * std::min(per_f, per_b)));
+        guard.whole = true;
     }
     const dim3 g((unsigned)((Tl->maxS * 32 + 255) / 256), (unsigned)Tl->nT);
     rsv::count_launches(1);
