@@ -384,7 +384,8 @@ __device__ void fetch_edges(const SweepArgs<T> &P, const Tile &tl, T *results, C
             more = more && !(on && (unsigned)(q0 + w - off) < (unsigned)tl.nx && en[w].missing());
             n += more;
         }
-        n = min(min(__reduce_min_sync(ALL, n), room - q0), tl.Sp - q0);
+        // room, too, as the lane that saw the fewest steps: the lanes read the counter one by one
+        n = min(__reduce_min_sync(ALL, min(n, room - q0)), tl.Sp - q0);
 #pragma unroll
         for (int w = 0; w < B::WIN; ++w)
             en[w].put_if(w < n && on && (unsigned)(q0 + w - off) < (unsigned)tl.nx,
@@ -407,7 +408,8 @@ __device__ void fetch_edges(const SweepArgs<T> &P, const Tile &tl, T *results, C
 __device__ __forceinline__ int wait_step(Control *ctl, int s, uint64_t deadline) {
     unsigned spins = 0;
     for (;;) {
-        const int n = min(ld_acquire(&ctl->ready), ld_acquire(&ctl->loaded) - 1);
+        // the lanes read one by one, so the counters may move between them: the least of what they saw
+        const int n = __reduce_min_sync(0xffffffffu, min(ld_acquire(&ctl->ready), ld_acquire(&ctl->loaded) - 1));
         if (s < n) return n;
         if ((++spins & 63u) == 0 && __any_sync(0xffffffffu, ld_acquire(&ctl->abort) != 0 || global_timer() > deadline))
             return 0;

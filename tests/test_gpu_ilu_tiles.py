@@ -39,3 +39,26 @@ def test_ilu_apply_at_tile_edges(dims, precision):
     _, z = oracle.System.from_problem(p, pc="bilu0").pc_apply(r)
     ratio = report_ratio(f"ilu_tiles_{precision}_{dims}", per_entry_ratio(zd.double().cpu().numpy(), z), bound)
     assert ratio <= bound
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("dims", [(3, 17, 9), (70, 9, 8), (41, 40, 21)])
+def test_ilu_apply_repeats_bit_for_bit(precision, dims):
+    """The order of a cell's operations is fixed, so whatever the timing of the hand-offs between warps and tiles is, every
+    apply gives the same bits."""
+    torch = pytest.importorskip("torch")
+    from tests.helpers import build_library
+    build_library()
+    import paper_1602_05901_gb300 as rsv
+    p = synth.make_problem(*dims, seed=93)
+    A = rsv.Matrix(*dims)
+    A.set_values(p.vals)
+    s = rsv.Solver(A, precision=precision)
+    s.setup("bilu0")
+    r = torch.from_numpy(np.random.default_rng(94).standard_normal(p.n)).cuda()
+    r = r if precision == "fp64" else r.float()
+    first, z = torch.empty_like(r), torch.empty_like(r)
+    s.apply(r, first)
+    for _ in range(100):
+        s.apply(r, z.fill_(float("nan")))
+        assert torch.equal(z, first)
