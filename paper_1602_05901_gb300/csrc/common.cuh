@@ -157,8 +157,8 @@ struct Cpr {  // CPR pressure stage: quasi-IMPES weights and the GMG hierarchy (
     void *x[kMaxLevels] = {}, *b[kMaxLevels] = {};  // per-level solution and right-hand side (T)
     double *w64 = nullptr;        // quasi-IMPES weights [nb][3], FP64
     void *w = nullptr;            // weights in T
-    double *dense = nullptr, *minv = nullptr, *work = nullptr;  // coarsest matrix / inverse / scratch
-    int *piv = nullptr;           // coarsest inverse: row permutations
+    double *dense = nullptr, *minv = nullptr, *work = nullptr;  // coarsest matrix and LU / inverse / scratch
+    int *piv = nullptr;           // coarsest LU: row permutations
     void *r = nullptr, *z = nullptr, *xp = nullptr;  // full-stage residual and ILU correction (T)
     void *apc = nullptr;          // pressure column of every block [nnzb][3] (T): CPR-PF's stage-two residual
     void *amg = nullptr;          // algebraic hierarchy (amg.cu) when the pressure stage coarsens algebraically

@@ -15,7 +15,7 @@
 //   * smoothing is red-black Gauss-Seidel, colour (i+j+k) mod 2, red then
 //     black before the recursion and black then red after it;
 //   * the coarsest level (at most gmg_max_coarse cells) is solved with its
-//     explicit inverse, computed at setup by Gauss-Jordan elimination with partial pivoting.
+//     explicit inverse, computed at setup from a partial-pivoting LU.
 // Full stage (CPR-PF, two-stage multiplicative): x = Pi_p p; r = f - A x;
 // x = x + ILU0^{-1} r, with Pi_p p = (p_c, 0, 0)_c.
 //
@@ -155,12 +155,18 @@ __global__ void coarse_dense_kernel(G3 g, const double *__restrict__ a7, double 
     }
 }
 
-// The coarsest level's inverse by Gauss-Jordan elimination with partial pivoting, kGjB columns (a panel) at a time.
-// FP64 arithmetic bounds it: one SM adds and multiplies 1.7 values per clock, so only the panel's own n x kGjB
-// values stay in one CTA (gj_panel) and the other columns are updated by the whole chip (gj_update).
-// 8x8x4 cells (n = 256): LU and triangular solves by single CTAs took 4.06 + 0.28 ms, this form 0.5 ms.
-constexpr int kGjB = 8;
-constexpr int kGjRows = 1024;  // rows that one thread each of the panel CTA holds in registers
+// The coarsest level's inverse from an LU factorisation with partial pivoting, kLuB columns (a panel) at a time, and
+// triangular solves for the unit vectors.  Every entry sees the operations of the plain row-by-row elimination in that
+// order (a - l u as one fused operation, l a true quotient), so neither the rounding nor which matrices are found
+// singular depends on the panels.  A Gauss-Jordan inverse rounds differently, and with pivot rows scaled by rounded
+// reciprocals an exactly singular operator can pass.
+// FP64 arithmetic bounds it: one SM adds and multiplies 1.7 values per clock, so only the panel's own columns stay in
+// one CTA (lu_panel); the other columns are updated by the whole chip (lu_update), and columns of the inverse are solved
+// for side by side (lu_columns), bound by the chain of 2 n steps, n of them with a division.
+// A one-level CPR setup of 8x8x4 cells (n = 256) takes 0.86 ms and of 10x10x5 2.1 ms; with elimination and solves by
+// single CTAs 4.6 and 22.6 ms, with Gauss-Jordan 0.58 and 1.6 ms.
+constexpr int kLuB = 8;
+constexpr int kLuRows = 1024;  // rows that one thread each of the panel CTA holds in registers
 
 // The largest key of the warp and the smallest row that has it (keys: bits of |value|, which order like the
 // values; integer reductions keep the search off the FP64 pipe).
@@ -175,30 +181,29 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
 }
 
-// One panel: Gauss-Jordan steps k0 .. k0 + kGjB - 1 on its own columns of the n x n matrix A.  Thread i
-// holds row i of the panel in registers.  Q [n][kGjB]: the panel afterwards (rows of the pivot block: its inverse P; other rows:
-// -A_iK P).  perm[i]: the row of A that the panel's pivoting moved to position i.  Largest |pivot| first, the
-// smallest row on ties; |pivot| <= 1e-300 reports RSV_ESINGULAR.
-__global__ void __launch_bounds__(kGjRows) gj_panel(int n, int k0, const double *__restrict__ A, double *__restrict__ Q,
-                                                       int *__restrict__ perm, int *status) {
+// One panel: elimination steps k0 .. k0 + kLuB - 1 on those columns of the n x n matrix A, rows k0 and below (m of them).
+// Thread r holds row k0 + r of the panel in registers.  Q [m][kLuB]: the panel afterwards, L below the diagonal and U
+// on and above it.  perm[i], i >= k0: the row of A that the pivoting moved to row i.  Largest |pivot| first, the smallest row
+// on ties; |pivot| <= 1e-300 reports RSV_ESINGULAR.
+__global__ void __launch_bounds__(kLuRows) lu_panel(int n, int k0, const double *__restrict__ A, double *__restrict__ Q,
+                                                    int *__restrict__ perm, int *status) {
     pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
     pdl_trigger();
     __shared__ unsigned long long wmax[32];
-    __shared__ double prow[kGjB], krow[kGjB];
+    __shared__ double prow[kLuB], trow[kLuB];
     __shared__ int widx[32], sidx[2];
-    const int i = threadIdx.x, lane = i & 31, warp = i >> 5, nw = (int)(blockDim.x >> 5);
-    const int nk = min(kGjB, n - k0);
-    double a[kGjB];
+    const int r = threadIdx.x, lane = r & 31, warp = r >> 5, nw = (int)(blockDim.x >> 5);
+    const int m = n - k0, nk = min(kLuB, m);
+    double a[kLuB];
 #pragma unroll
-    for (int c = 0; c < kGjB; ++c) a[c] = i < n && c < nk ? A[(int64_t)i * n + k0 + c] : 0.0;
-    int src = i;
+    for (int c = 0; c < kLuB; ++c) a[c] = r < m && c < nk ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+    int src = k0 + r;
 #pragma unroll
-    for (int t = 0; t < kGjB; ++t) {
+    for (int t = 0; t < kLuB; ++t) {
         if (t >= nk) break;
-        const int k = k0 + t;
-        const bool in = i >= k && i < n;
+        const bool in = r >= t && r < m;
         unsigned long long key = in ? abs_bits(a[t]) : 0ull;
-        int at = in ? i : n;  // n: no candidate, behind every row of the same key
+        int at = in ? r : m;  // m: no candidate, behind every row of the same key
         warp_largest(key, at);
         if (lane == 0) {
             wmax[warp] = key;
@@ -206,68 +211,66 @@ __global__ void __launch_bounds__(kGjRows) gj_panel(int n, int k0, const double 
         }
         __syncthreads();
         key = lane < nw ? wmax[lane] : 0ull;
-        at = lane < nw ? widx[lane] : n;
+        at = lane < nw ? widx[lane] : m;
         warp_largest(key, at);
         const int p = at;
-        if (i == k) {
+        if (r == t) {
 #pragma unroll
-            for (int c = 0; c < kGjB; ++c) krow[c] = a[c];
+            for (int c = 0; c < kLuB; ++c) trow[c] = a[c];
             sidx[0] = src;
             if (!(__longlong_as_double((long long)key) > 1e-300)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
         }
-        if (i == p) {
-            const double ip = 1.0 / a[t];
+        if (r == p) {
 #pragma unroll
-            for (int c = 0; c < kGjB; ++c) prow[c] = c == t ? ip : a[c] * ip;
+            for (int c = 0; c < kLuB; ++c) prow[c] = a[c];
             sidx[1] = src;
         }
         __syncthreads();
-        if (i == p && p != k) {
+        if (r == p) {
 #pragma unroll
-            for (int c = 0; c < kGjB; ++c) a[c] = krow[c];
+            for (int c = 0; c < kLuB; ++c) a[c] = trow[c];
             src = sidx[0];
         }
-        if (i == k) {
+        if (r == t) {
 #pragma unroll
-            for (int c = 0; c < kGjB; ++c) a[c] = prow[c];
+            for (int c = 0; c < kLuB; ++c) a[c] = prow[c];
             src = sidx[1];
-        } else {
-            const double m = -a[t];
+        } else if (in) {
+            const double l = a[t] / prow[t];
+            a[t] = l;
 #pragma unroll
-            for (int c = 0; c < kGjB; ++c) a[c] = c == t ? m * prow[c] : fma(m, prow[c], a[c]);
+            for (int c = t + 1; c < kLuB; ++c) a[c] = fma(-l, prow[c], a[c]);
         }
     }
-    if (i < n) {
+    if (r < m) {
 #pragma unroll
-        for (int c = 0; c < kGjB; ++c) Q[i * kGjB + c] = a[c];
-        perm[i] = src;
+        for (int c = 0; c < kLuB; ++c) Q[r * kLuB + c] = a[c];
+        perm[k0 + r] = src;
     }
 }
 
 // The same for more rows than a CTA has threads (few levels on a large grid): the panel lives in Q, the row
 // order in perm.
-__global__ void __launch_bounds__(kGjRows) gj_panel_large(int n, int k0, const double *__restrict__ A, double *Q, int *perm,
+__global__ void __launch_bounds__(kLuRows) lu_panel_large(int n, int k0, const double *__restrict__ A, double *Q, int *perm,
                                                           int *status) {
     pdl_wait();
     pdl_trigger();
     __shared__ unsigned long long wmax[32];
-    __shared__ double prow[kGjB];
     __shared__ int widx[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nk = min(kGjB, n - k0);
-    for (int i = threadIdx.x; i < n; i += kGjRows) {
-        for (int c = 0; c < kGjB; ++c) Q[(int64_t)i * kGjB + c] = c < nk ? A[(int64_t)i * n + k0 + c] : 0.0;
-        perm[i] = i;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = n - k0, nk = min(kLuB, m);
+    for (int r = threadIdx.x; r < m; r += kLuRows) {
+        for (int c = 0; c < kLuB; ++c) Q[(int64_t)r * kLuB + c] = c < nk ? A[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+        perm[k0 + r] = k0 + r;
     }
     __syncthreads();
     for (int t = 0; t < nk; ++t) {
-        const int k = k0 + t;
         unsigned long long key = 0ull;
-        int at = n;
-        for (int i = k + threadIdx.x; i < n; i += kGjRows) {
-            const unsigned long long v = abs_bits(Q[(int64_t)i * kGjB + t]);
-            if (at == n || v > key) {
+        int at = m;
+        for (int r = t + threadIdx.x; r < m; r += kLuRows) {
+            const unsigned long long v = abs_bits(Q[(int64_t)r * kLuB + t]);
+            if (at == m || v > key) {
                 key = v;
-                at = i;
+                at = r;
             }
         }
         warp_largest(key, at);
@@ -281,69 +284,240 @@ __global__ void __launch_bounds__(kGjRows) gj_panel_large(int n, int k0, const d
         warp_largest(key, at);
         const int p = at;
         if (threadIdx.x == 0 && !(__longlong_as_double((long long)key) > 1e-300)) atomicCAS(status, 0, (int)RSV_ESINGULAR);
-        if (threadIdx.x < kGjB) {  // the pivot row, scaled; its place takes row k
+        if (threadIdx.x < kLuB && p != t) {
             const int c = threadIdx.x;
-            const double ip = 1.0 / Q[(int64_t)p * kGjB + t], v = Q[(int64_t)p * kGjB + c];
-            __syncwarp((1u << kGjB) - 1u);
-            if (p != k) Q[(int64_t)p * kGjB + c] = Q[(int64_t)k * kGjB + c];
-            prow[c] = c == t ? ip : v * ip;
-            if (c == 0 && p != k) {
-                const int sp = perm[p];
-                perm[p] = perm[k];
-                perm[k] = sp;
+            const double v = Q[(int64_t)p * kLuB + c];
+            Q[(int64_t)p * kLuB + c] = Q[t * kLuB + c];
+            Q[t * kLuB + c] = v;
+            if (c == 0) {
+                const int sp = perm[k0 + p];
+                perm[k0 + p] = perm[k0 + t];
+                perm[k0 + t] = sp;
             }
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < n; i += kGjRows) {
-            double *q = Q + (int64_t)i * kGjB;
-            const double m = -q[t];
-            for (int c = 0; c < kGjB; ++c) q[c] = i == k ? prow[c] : c == t ? m * prow[c] : fma(m, prow[c], q[c]);
+        for (int r = t + 1 + threadIdx.x; r < m; r += kLuRows) {
+            double *q = Q + (int64_t)r * kLuB;
+            const double l = q[t] / Q[t * kLuB + t];
+            q[t] = l;
+            for (int c = t + 1; c < nk; ++c) q[c] = fma(-l, Q[t * kLuB + c], q[c]);
         }
         __syncthreads();
     }
 }
 
-// The panel's effect on the matrix: B = the panel's columns from Q, every other column j
-// B_ij = (i in the pivot block ? 0 : A_perm(i)j) + sum_t Q_it A_perm(k0 + t)j.  Tracks the row order
-// (order_out = order_in through perm).  The last panel writes column j of B to column order_out(j) of
-// the result: the inverse of the row-permuted matrix, its columns put back.
-__global__ void __launch_bounds__(256) gj_update(int n, int k0, const double *__restrict__ A, const double *__restrict__ Q,
+// B = A with the panel's rows moved, its columns from Q, and the columns right of it updated.  A CTA takes 16 rows of 32
+// columns; one warp forms the columns' part of U (28 dependent FP64 operations), which the others' rows need.  Tracks the
+// row order (order_out = order_in through perm).  The last panel writes B transposed.
+__global__ void __launch_bounds__(256) lu_update(int n, int k0, const double *__restrict__ A, const double *__restrict__ Q,
                                                  const int *__restrict__ perm, const int *__restrict__ order_in,
                                                  int *__restrict__ order_out, double *__restrict__ B) {
     pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
     pdl_trigger();
-    const int j = blockIdx.x * 32 + (threadIdx.x & 31), i = blockIdx.y * 8 + (threadIdx.x >> 5);
-    if (i >= n || j >= n) return;
-    const int nk = min(kGjB, n - k0);
-    if (j == 0) order_out[i] = order_in ? order_in[perm[i]] : perm[i];
-    double r;
-    if (j >= k0 && j < k0 + nk) {
-        r = Q[(int64_t)i * kGjB + (j - k0)];
-    } else {
-        r = i >= k0 && i < k0 + nk ? 0.0 : A[(int64_t)perm[i] * n + j];
+    __shared__ double u[kLuB][32];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, i0 = blockIdx.y * 16, j = blockIdx.x * 32 + tx;
+    const int k1 = min(k0 + kLuB, n);
+    const bool right = j >= k1 && j < n;  // then the panel is a full one
+    double v[2];
+    int src[2];
 #pragma unroll
-        for (int t = 0; t < kGjB; ++t)
-            if (t < nk) r = fma(Q[(int64_t)i * kGjB + t], A[(int64_t)perm[k0 + t] * n + j], r);
+    for (int h = 0; h < 2; ++h) {
+        const int i = i0 + ty + 8 * h;
+        src[h] = i < k0 || i >= n ? i : perm[i];
+        v[h] = i < n && j < n ? A[(int64_t)src[h] * n + j] : 0.0;
     }
-    const bool last = k0 + nk >= n;
-    const int to = !last ? j : order_in ? order_in[perm[j]] : perm[j];
-    B[(int64_t)i * n + to] = r;
+    if (ty == 0 && right && i0 + 16 > k0) {
+        double w[kLuB];
+#pragma unroll
+        for (int t = 0; t < kLuB; ++t) w[t] = A[(int64_t)perm[k0 + t] * n + j];
+#pragma unroll
+        for (int t = 0; t < kLuB; ++t) {
+#pragma unroll
+            for (int s = 0; s < t; ++s) w[t] = fma(-Q[t * kLuB + s], w[s], w[t]);
+            u[t][tx] = w[t];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = i0 + ty + 8 * h;
+        if (i >= n || j >= n) continue;
+        if (j == 0) order_out[i] = order_in ? order_in[src[h]] : src[h];
+        double r = v[h];
+        if (i >= k0 && j >= k0) {
+            const double *l = Q + (int64_t)(i - k0) * kLuB;
+            if (j < k1) {
+                r = l[j - k0];
+            } else if (i < k1) {
+                r = u[i - k0][tx];
+            } else {
+#pragma unroll
+                for (int t = 0; t < kLuB; ++t) r = fma(-l[t], u[t][tx], r);
+            }
+        }
+        B[k1 < n ? (int64_t)i * n + j : (int64_t)j * n + i] = r;
+    }
 }
 
-// Minv = inverse of the n x n matrix in `dense` (overwritten).  work: n (n + kGjB) doubles; index: 3 n ints.
+// Columns j = C b .. C b + C - 1 of the inverse by CTA b: L U x = P e_j, T the transpose of L and U.  At most kLuRows rows, x
+// in registers (row threadIdx.x + q blockDim.x at q); a step's x_k travel through shared memory, and T is read four
+// steps ahead.  The quotients of a step are formed by one lane each: a division in one lane holds the FP64 pipe as
+// long as one in all of them.
+constexpr int kLuOwn = 4;
+template <int C>
+__global__ void __launch_bounds__(kLuRows / kLuOwn, C == 1 ? 2 : 1) lu_columns(int n, const double *__restrict__ T,
+                                                               const int *__restrict__ order, double *__restrict__ Minv) {
+    pdl_wait();  // launched with launch_pdl: the previous kernel may still be running
+    pdl_trigger();
+    __shared__ double xk[2][C];
+    __shared__ int start;  // x is zero above its unit entries: the first group of four steps that has one
+    const int j0 = blockIdx.x * C, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    double x[kLuOwn][C], now[4][kLuOwn], next[4][kLuOwn], dnow[4], dnext[4];
+    if (tid == 0) start = n;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kLuOwn; ++q) {
+        const int i = tid + q * nt, at = i < n ? order[i] - j0 : -1;
+#pragma unroll
+        for (int c = 0; c < C; ++c) x[q][c] = at == c ? 1.0 : 0.0;
+        if (at >= 0 && at < C) atomicMin(&start, i & ~3);
+    }
+    __syncthreads();
+    // columns k .. k + 3 of T, rows below (or above) the diagonal only
+    auto fetch = [&](int k, bool below, double(&l)[4][kLuOwn], double(&d)[4]) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const bool in = k >= 0 && k + s < n;
+            d[s] = in && !below ? T[(int64_t)(k + s) * n + k + s] : 1.0;
+#pragma unroll
+            for (int q = 0; q < kLuOwn; ++q) {
+                const int i = tid + q * nt;
+                l[s][q] = in && (below ? i > k + s && i < n : i < k + s) ? T[(int64_t)(k + s) * n + i] : 0.0;
+            }
+        }
+    };
+    // the unit lower triangle
+    fetch(start, true, next, dnext);
+#pragma unroll
+    for (int o = 0; o < kLuOwn; ++o)
+        for (int k = max(o * nt, start); k < min((o + 1) * nt, n); k += 4) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+#pragma unroll
+                for (int q = 0; q < kLuOwn; ++q) now[s][q] = next[s][q];
+            fetch(k + 4, true, next, dnext);
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                if (k + s >= n) break;
+                if (tid == k + s - o * nt)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) xk[s & 1][c] = x[o][c];
+                __syncthreads();
+#pragma unroll
+                for (int q = o; q < kLuOwn; ++q) {
+                    const int i = tid + q * nt;
+                    if (i > k + s && i < n)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) x[q][c] = fma(-now[s][q], xk[s & 1][c], x[q][c]);
+                }
+            }
+        }
+    __syncthreads();
+    // the upper triangle
+    const int last = (n - 1) / 4 * 4;
+    fetch(last, false, next, dnext);
+#pragma unroll
+    for (int o = kLuOwn - 1; o >= 0; --o)
+        for (int k = min((o + 1) * nt - 4, last); k >= o * nt; k -= 4) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                dnow[s] = dnext[s];
+#pragma unroll
+                for (int q = 0; q < kLuOwn; ++q) now[s][q] = next[s][q];
+            }
+            fetch(k - 4, false, next, dnext);
+#pragma unroll
+            for (int s = 3; s >= 0; --s) {
+                if (k + s >= n) continue;
+                const int at = k + s - o * nt;  // the thread that owns row k + s
+                if (C == 1) {
+                    if (tid == at) xk[s & 1][0] = x[o][0] /= dnow[s];
+                } else if (warp == at >> 5) {
+                    double v = 0.0;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const double t = __shfl_sync(0xffffffffu, x[o][c], at & 31);
+                        if (lane == c) v = t;
+                    }
+                    if (lane < C) xk[s & 1][lane] = v / dnow[s];
+                }
+                __syncthreads();
+                if (C > 1 && tid == at)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) x[o][c] = xk[s & 1][c];
+#pragma unroll
+                for (int q = 0; q <= o; ++q)
+                    if (tid + q * nt < k + s)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) x[q][c] = fma(-now[s][q], xk[s & 1][c], x[q][c]);
+            }
+        }
+#pragma unroll
+    for (int q = 0; q < kLuOwn; ++q) {
+        const int i = tid + q * nt;
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+            if (i < n && j0 + c < n) Minv[(int64_t)i * n + j0 + c] = x[q][c];
+    }
+}
+
+// The same for more rows: x in row j of `work`.
+__global__ void __launch_bounds__(256) lu_columns_large(int n, const double *__restrict__ T, const int *__restrict__ order,
+                                                        double *__restrict__ Minv, double *work) {
+    pdl_wait();
+    pdl_trigger();
+    const int j = blockIdx.x;
+    double *x = work + (int64_t)j * n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) x[i] = order[i] == j ? 1.0 : 0.0;
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        const double xk = x[k];
+        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) x[i] = fma(-T[(int64_t)k * n + i], xk, x[i]);
+        __syncthreads();
+    }
+    for (int k = n - 1; k >= 0; --k) {
+        if (threadIdx.x == 0) x[k] /= T[(int64_t)k * n + k];
+        __syncthreads();
+        const double xk = x[k];
+        for (int i = threadIdx.x; i < k; i += blockDim.x) x[i] = fma(-T[(int64_t)k * n + i], xk, x[i]);
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) Minv[(int64_t)i * n + j] = x[i];
+}
+
+// Minv = inverse of the n x n matrix in `dense` (overwritten).  work: n (n + kLuB) doubles; index: 3 n ints.
 cudaError_t coarse_inverse(cudaStream_t st, int n, double *dense, double *work, int *index, double *Minv, int *status) {
     double *X[2] = {dense, work}, *Q = work + (int64_t)n * n;
     int *perm = index, *order[2] = {index + n, index + 2 * n};
     cudaError_t e = cudaSuccess;
-    for (int k0 = 0, q = 0; k0 < n && e == cudaSuccess; k0 += kGjB, q ^= 1) {
+    int q = 0;
+    for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += kLuB, q ^= 1) {
+        const int m = n - k0;
         count_launches(2);
-        e = n <= kGjRows ? launch_pdl(gj_panel, dim3(1), dim3((n + 31) / 32 * 32), 0, st, n, k0, X[q], Q, perm, status)
-                         : launch_pdl(gj_panel_large, dim3(1), dim3(kGjRows), 0, st, n, k0, X[q], Q, perm, status);
+        e = m <= kLuRows ? launch_pdl(lu_panel, dim3(1), dim3((m + 31) / 32 * 32), 0, st, n, k0, X[q], Q, perm, status)
+                         : launch_pdl(lu_panel_large, dim3(1), dim3(kLuRows), 0, st, n, k0, X[q], Q, perm, status);
         if (e == cudaSuccess)
-            e = launch_pdl(gj_update, dim3((n + 31) / 32, (n + 7) / 8), dim3(256), 0, st, n, k0, X[q], Q, perm,
-                           k0 ? order[q] : nullptr, order[q ^ 1], k0 + kGjB >= n ? Minv : X[q ^ 1]);
+            e = launch_pdl(lu_update, dim3((n + 31) / 32, (n + 15) / 16), dim3(256), 0, st, n, k0, X[q], Q, perm,
+                           k0 ? order[q] : nullptr, order[q ^ 1], X[q ^ 1]);
     }
-    return e;
+    if (e != cudaSuccess) return e;
+    count_launches(1);
+    if (n > kLuRows)
+        return launch_pdl(lu_columns_large, dim3(n), dim3(256), 0, st, n, X[q], order[q], Minv, X[q ^ 1]);
+    // two CTAs are resident per SM with one column each, one with four: as many columns as one wave takes
+    const dim3 block(std::min((n + 31) / 32 * 32, kLuRows / kLuOwn));
+    return n <= 2 * 152 ? launch_pdl(lu_columns<1>, dim3(n), block, 0, st, n, X[q], order[q], Minv)
+                        : launch_pdl(lu_columns<4>, dim3((n + 3) / 4), block, 0, st, n, X[q], order[q], Minv);
 }
 
 // x = Minv b (one warp per row), b and x in T, arithmetic in FP64.
@@ -680,7 +854,7 @@ cudaError_t cpr_setup(const rsv_mat *A, cudaStream_t st, bool mixed, int max_lev
     }
     alloc((void **)&P->dense, sizeof(double) * ncd * ncd);
     alloc((void **)&P->minv, sizeof(double) * ncd * ncd);
-    alloc((void **)&P->work, sizeof(double) * ncd * (ncd + kGjB));
+    alloc((void **)&P->work, sizeof(double) * ncd * (ncd + kLuB));
     alloc((void **)&P->piv, sizeof(int) * 3 * ncd);
     alloc(&P->r, es * 3 * nb);
     alloc(&P->z, es * 3 * nb);
