@@ -7,8 +7,8 @@
 // with each system's own scalars (rho, alpha, omega, beta), its own
 // convergence test and iteration count.  A converged system freezes: the
 // vector updates, the sweeps and the products skip its rows.  Segmented reductions give every system its
-// own FP64-accurate dot products, deterministically (per system, partial
-// sums of fixed chunks are added in chunk order by the last CTA to finish).
+// own FP64-accurate dot products, deterministically (per system, the last CTA
+// to finish adds the partial sums of fixed chunks in a fixed pattern).
 //
 // One loop pass (two preconditioner applications, two SpMVs, four segmented
 // reductions and the scalar steps) is captured once into a CUDA graph holding
@@ -191,9 +191,10 @@ struct Scalars {
 
 // out1[s] = <x, y1> (or its sqrt) and, when y2, out2[s] = <x, y2>, per system s, then the scalar step `after`
 // of system s.  HBM should bound it; what did was one thread per system adding the items' partial sums one
-// after another, FP64 warp trees per item and scalar loads (24 systems, 7 M FP32 unknowns: 72 -> 22 us).  Now a warp
-// adds the partials (each lane a fixed strided subset, then a tree: still deterministic), items are read in 16-byte
-// groups, and FP32 sums go through the warp as double-float pairs.
+// after another, an FP64 tree in every warp and scalar loads (24 systems, 7 M FP32 unknowns: 72 -> 27 us).  Now items are
+// read in 16-byte groups, half a warp adds an item's sums (each lane a fixed strided subset, then a tree), and a warp adds
+// the items' partial sums in the same manner: FP64 throughout, and still deterministic.  (A tree of double-float pairs in
+// every warp takes 4 us less, but keeps 46 bits of the 53.)
 template <typename T>
 __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(const SegItem *__restrict__ items, int nitems,
                                                               const int *__restrict__ item_begin,
@@ -201,7 +202,7 @@ __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(const SegItem *__r
                                                               const T *__restrict__ y2, double *out1, double *out2,
                                                               int sqrt1, double *partial, unsigned *ticket,
                                                               const int *done, After after, Scalars sc) {
-    __shared__ double sm[2][kSegThreads / 32];
+    __shared__ double sm[2][kSegThreads];
     __shared__ bool last;
     const bool ok = ((((uintptr_t)x) | ((uintptr_t)y1) | ((uintptr_t)y2)) & 15) == 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -226,27 +227,24 @@ __global__ void __launch_bounds__(kSegThreads) seg_dot_kernel(const SegItem *__r
                     a1.add(x[i], y1[i]);
                     if (y2) a2.add(x[i], y2[i]);
                 });
-        Part<T> p1 = Part<T>::of(a1), p2 = Part<T>::of(a2);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            p1.add(p1.xor_shfl(o));
-            if (y2) p2.add(p2.xor_shfl(o));
-        }
-        if (lane == 0) {
-            sm[0][warp] = p1.value();
-            sm[1][warp] = y2 ? p2.value() : 0.0;
-        }
+        sm[0][threadIdx.x] = a1.value();
+        if (y2) sm[1][threadIdx.x] = a2.value();
         __syncthreads();
-        if (threadIdx.x < 2) {
+        if (warp == 0) {  // lanes 0-15 add the first product's sums, lanes 16-31 the second's
+            const int half = lane >> 4, l = lane & 15;
             double s1 = 0.0;
-            for (int q = 0; q < kSegThreads / 32; ++q) s1 += sm[threadIdx.x][q];
-            partial[(size_t)threadIdx.x * nitems + it] = s1;
-        }
-        __syncwarp();
-        if (threadIdx.x == 0) {
-            __threadfence();  // both partial sums before the ticket
-            const unsigned nit = (unsigned)(item_begin[w.sys + 1] - item_begin[w.sys]);
-            last = atomicAdd(&ticket[w.sys], 1u) == nit - 1;
+            if (half == 0 || y2)
+#pragma unroll
+                for (int q = 0; q < kSegThreads; q += 16) s1 += sm[half][q + l];
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            if (l == 0) partial[(size_t)half * nitems + it] = s1;
+            __syncwarp();
+            if (lane == 0) {
+                __threadfence();  // both partial sums before the ticket
+                const unsigned nit = (unsigned)(item_begin[w.sys + 1] - item_begin[w.sys]);
+                last = atomicAdd(&ticket[w.sys], 1u) == nit - 1;
+            }
         }
         __syncthreads();
         if (last && warp == 0) {

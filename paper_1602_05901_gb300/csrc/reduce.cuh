@@ -30,7 +30,7 @@ template <> struct Acc<float> {
         hi = s;
         lo = __fadd_rn(lo, __fadd_rn(err, pe));
     }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+    __device__ __forceinline__ double value() const { return exact_double(hi) + exact_double(lo); }
 };
 
 // A partial sum in its accumulator's form, for the warp reduction trees: an FP64

@@ -155,3 +155,29 @@ def test_batch_64_uneven_systems_full_size(rsv):
         off += p.nb
     assert max(its) < 1000, its
     print(f"BATCH64_FULL iters min/median/max {min(its)}/{int(np.median(its))}/{max(its)}")
+
+
+def test_batched_inner_sums_keep_fp64(rsv):
+    """<rh, A p> of the first FP32 pass is 1 + 2^-25 + 2^-52 - 1 - 2^-25 = 2^-52, each term exact in FP32 and in another
+    thread: FP64 holds every partial sum, whatever the order, so the step is taken.  A sum in fewer bits is zero, which ends
+    every inner solve as a breakdown before its first iteration."""
+    import torch
+    cells = 22
+    A = rsv.Matrix.batch([(cells, 1, 1)])
+    places = [0, 64, 32, 16, 8] + [4 * q for q in (1, 3, 5, 6, 7, 9, 10, 11, 12, 13, 14)]
+    assert max(places) < 3 * cells and len(set(places)) == 16
+    diag = np.zeros(3 * cells)
+    diag[places[:5]] = 16.0 * np.array([1.0, 2.0 ** -25, 2.0 ** -52, -1.0, -2.0 ** -25])
+    vals = np.zeros((len(A.col_idx), 3, 3))
+    for c in range(cells):
+        for q in range(A.row_ptr[c], A.row_ptr[c + 1]):
+            if A.col_idx[q] == c:
+                vals[q] = np.diag(diag[3 * c:3 * c + 3])
+    A.set_values(vals)
+    s = rsv.Solver(A, solver="bicgstab", precision="mixed", rtol=1e-8, btol=0.0, maxit=50)
+    s.setup("none")
+    b = np.zeros(3 * cells)
+    b[places] = 0.25
+    x = torch.zeros(3 * cells, dtype=torch.float64, device="cuda")
+    _, infos = s.solve_batched(torch.from_numpy(b).cuda(), x)
+    assert infos[0]["iters"] > 0
