@@ -578,13 +578,15 @@ bool vec_ok(int64_t ldv, std::initializer_list<const void *> ptrs) {
     return true;
 }
 
-}  // namespace
-
 // Systems of few unknowns: one row per thread and no more CTAs than that takes (at most one per SM), the multi-dot's
 // groups of basis vectors side by side.  On the full grid most CTAs sum zeros, an FP64 tree per group one after another,
 // and the last one adds 304 partial sums for each output.  12,000 unknowns, FP64, 30 basis vectors (ncu, mean of a
-// cycle): multi-dot 24.8 -> 11.9 us, update 14.9 -> 10.6 us.
-bool small(int64_t n) { return n > 0 && n <= 152 * kRedThreads; }
+// cycle): multi-dot 24.8 -> 11.9 us, update 14.9 -> 10.6 us.  A whole GMRES(30) step with block Jacobi, full grid -> this:
+// 1,500 unknowns FP64 66.4 -> 50.0 us and FP32 44.9 -> 35.7, 12,000 66.2 -> 52.3 and 46.4 -> 38.7, 24,000 67.0 -> 55.3 and
+// 46.3 -> 40.2, 38,880 68.6 -> 59.6 and 46.8 -> 42.4.  The line lies where the SMs have one CTA each.
+bool one_row_per_thread(int64_t n) { return n > 0 && n <= 152 * kRedThreads; }
+
+}  // namespace
 
 template <typename T>
 cudaError_t launch_mdot(cudaStream_t st, int64_t n, const T *w, const T *V, int64_t ldv, int k, double *partial,
@@ -604,7 +606,7 @@ cudaError_t launch_mdot2(cudaStream_t st, int64_t n, const T *w, const T *u, con
                          double *partial, double *ow, double *ou, unsigned *counter, const int *done) {
     if (k < 1 || k > kMaxRestart + 1) return cudaErrorInvalidValue;
     rsv::count_launches(1);
-    if (small(n))
+    if (one_row_per_thread(n))
         return launch_pdl(mdot2_kernel<T, false>,
                           dim3((unsigned)((n + kRedThreads - 1) / kRedThreads), (k + kGroup / 2 - 1) / (kGroup / 2)),
                           dim3(kRedThreads), 0, st, n, w, u, V, ldv, k, partial, ow, ou, counter, done);
@@ -620,7 +622,7 @@ cudaError_t launch_maxpy(cudaStream_t st, int64_t n, const T *base, const T *V, 
                          double sgn, T *out, double *partial, double *nrm, unsigned *counter, const int *done,
                          const int *skip) {
     rsv::count_launches(1);
-    if (small(n))
+    if (one_row_per_thread(n))
         maxpy_kernel<T, false><<<(unsigned)((n + kRedThreads - 1) / kRedThreads), kRedThreads, 0, st>>>(
             n, base, V, ldv, k, c, sgn, out, partial, nrm, counter, done, skip);
     else if (vec_ok<T>(ldv, {base, V, out}))
