@@ -236,3 +236,96 @@ def test_conv_wgrad_rows(rsv, case):
     assert np.all(np.abs(gw.cpu().double().numpy() - ref) <= 2 * nvox * U32 * absref + 1e-30)
     flat = gyh.reshape(-1, co)
     assert np.all(np.abs(gb.cpu().double().numpy() - flat.sum(0)) <= 2 * nvox * U32 * np.abs(flat).sum(0) + 1e-30)
+
+
+# The weight gradient's other forms at 27 taps, which the form by whole rows leaves to longer rows and unaligned leading
+# dimensions.  (The 27-tap cases of WG_CASES all take the form by whole rows now; the labels beside them name what they
+# took without it.)  Here: boxes of 64 voxels with either operand shifted, N = 192 and 256, several N tiles and channel blocks, ragged boxes; voxel-major copies with several blocks of
+# 128 and of 32 channels.
+OTHER_CASES = [
+    # (nx, ny, nz, ci, co, extra ldx)
+    (136, 5, 3, 192, 64, 8),
+    (136, 2, 2, 384, 128, 0),
+    (144, 3, 3, 128, 256, 8),
+    (136, 1, 5, 96, 32, 0),
+    (192, 3, 1, 32, 96, 0),
+    (24, 5, 3, 256, 96, 4),
+    (40, 3, 5, 160, 64, 4),
+]
+
+
+@pytest.mark.parametrize("case", OTHER_CASES, ids=["{}x{}x{}_ci{}_co{}_pad{}".format(*c) for c in OTHER_CASES])
+def test_conv_wgrad_long_rows_and_unaligned(rsv, case):
+    test_conv_wgrad_rows(rsv, case)
+
+
+# The folded form with everything a layer's call can carry: rows that leave part of a tile invalid, one and two accumulator
+# sets, resident and streamed weights, kept planes and one box at a time, a single pair and several per CTA.
+FULL_CASES = [
+    (24, 11, 3, 32, 32), (40, 7, 2, 64, 64), (128, 3, 3, 96, 32), (40, 21, 50, 32, 64), (32, 40, 40, 32, 32),
+    (16, 66, 40, 64, 64), (128, 3, 90, 64, 32), (64, 5, 3, 192, 64),
+]
+FULL_IDS = [f"{c[0]}x{c[1]}x{c[2]}_ci{c[3]}_co{c[4]}" for c in FULL_CASES]
+
+
+def _at(t, channel):
+    return ctypes.c_void_p(t.data_ptr() + 2 * channel)
+
+
+@pytest.mark.parametrize("relu,use_bias,masked", [(True, True, False), (False, False, True), (True, False, True)])
+@pytest.mark.parametrize("case", FULL_CASES, ids=FULL_IDS)
+def test_conv_narrow_layers_full_call(rsv, case, relu, use_bias, masked):
+    """Padded input, a mask and a BF16 output at a channel offset of a wider tensor.  Same bound as above; the BF16 output is the
+    round-to-nearest of the FP32 one, and the channels beside it stay as they were."""
+    torch = pytest.importorskip("torch")
+    nx, ny, nz, ci, co = case
+    rng = np.random.default_rng(700 + sum(case))
+    ldx, ldy, ldm = ci + 16, co + 48, co + 8
+    xt, xh = _bf16(torch, rng.standard_normal((nz, ny, nx, ldx)))
+    xh = xh[..., 8:8 + ci]
+    wt, wh = _bf16(torch, rng.standard_normal((co, 27, ci)) * np.sqrt(2.0 / (27 * ci)))
+    bias = rng.standard_normal(co).astype(np.float32) * 0.1
+    bt = torch.tensor(bias).cuda()
+    mt, mh = _bf16(torch, rng.standard_normal((nz, ny, nx, ldm)))
+    y32 = torch.full((nz * ny * nx, co), float("nan"), device="cuda")
+    yb = torch.full((nz * ny * nx, ldy), 3.0, dtype=torch.bfloat16, device="cuda")
+    st = rsv.rsv_conv3d_fwd(None, nx, ny, nz, 27, ci, co, _at(xt, 8), ldx, _p(wt), _p(bt) if use_bias else None, int(relu),
+                            _at(mt, 8) if masked else None, ldm if masked else 0, _at(yb, 32), ldy, _p(y32))
+    assert st == rsv.RSV_OK, rsv.status_string(st)
+    ref, absref = U.conv3(xh, wh), U.conv3(np.abs(xh), np.abs(wh))
+    if use_bias:
+        ref, absref = ref + bias, absref + np.abs(bias)
+    if relu:
+        ref = np.maximum(ref, 0)
+    if masked:
+        ref = ref * (mh[..., 8:8 + co] > 0)
+    got = y32.cpu().double().numpy().reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= 2 * (27 * ci + 1) * U32 * absref)
+    gb = yb.float().cpu().double().numpy().reshape(nz, ny, nx, ldy)
+    assert np.array_equal(gb[..., 32:32 + co], U.bf16_round(got))
+    assert np.all(gb[..., :32] == 3) and np.all(gb[..., 32 + co:] == 3)
+
+
+@pytest.mark.parametrize("case", FULL_CASES, ids=FULL_IDS)
+def test_conv_narrow_layers_input_gradient(rsv, case):
+    """The layer's output channels are the case's ci, its input channels (the gradient's) the case's co; masked by an
+    activation inside a wider tensor, BF16 at a channel offset."""
+    torch = pytest.importorskip("torch")
+    nx, ny, nz, co, ci = case
+    rng = np.random.default_rng(800 + sum(case))
+    ldm, ldgx = ci + 24, ci + 16
+    gyt, gyh = _bf16(torch, _vol(rng, nz, ny, nx, co, co + 8))
+    wt, wh = _bf16(torch, rng.standard_normal((co, 27, ci)) * 0.1)
+    mt, mh = _bf16(torch, rng.standard_normal((nz, ny, nx, ldm)))
+    mh = mh[..., 16:16 + ci]
+    gx32 = torch.full((nz * ny * nx, ci), float("nan"), device="cuda")
+    gxb = torch.full((nz * ny * nx, ldgx), 3.0, dtype=torch.bfloat16, device="cuda")
+    st = rsv.rsv_conv3d_dgrad(None, nx, ny, nz, ci, co, _p(gyt), co + 8, _p(wt), _at(mt, 16), ldm, _at(gxb, 8), ldgx, _p(gx32))
+    assert st == rsv.RSV_OK, rsv.status_string(st)
+    gyh = gyh[..., :co]
+    ref, absref = U.conv3_dgrad(gyh, wh) * (mh > 0), U.conv3_dgrad(np.abs(gyh), np.abs(wh))
+    got = gx32.cpu().double().numpy().reshape(ref.shape)
+    assert np.all(np.abs(got - ref) <= 2 * 27 * co * U32 * absref + 1e-30)
+    gb = gxb.float().cpu().double().numpy().reshape(nz, ny, nx, ldgx)
+    assert np.array_equal(gb[..., 8:8 + ci], U.bf16_round(got))
+    assert np.all(gb[..., :8] == 3) and np.all(gb[..., 8 + ci:] == 3)
