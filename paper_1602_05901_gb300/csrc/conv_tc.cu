@@ -545,6 +545,9 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
                 tmem_ld16_start(acc0 + CO + n, pc);
                 tmem_ld16_start(acc0 + 2 * CO + n, pp);
                 tmem_ld_wait();
+                tmem_landed(pm);
+                tmem_landed(pc);
+                tmem_landed(pp);
                 float *slot = mine + (chunk & 1) * 128;
                 if (lane == 31)
 #pragma unroll

@@ -177,7 +177,8 @@ __device__ __forceinline__ void mma_commit(uint64_t *bar) {
 }
 
 // 16 consecutive FP32 columns of the warp's 32 TMEM lanes: lane l of the warp gets row (lane base + l).
-// The values are there after tmem_ld_wait().
+// The values are there after tmem_ld_wait(); tmem_landed, called behind it on the registers of every such load, keeps
+// the compiler from moving their uses ahead of the wait (nothing else in the code ties the two together).
 __device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t r[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
@@ -188,10 +189,16 @@ __device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t r[16]) 
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_landed(uint32_t r[16]) {
+    asm volatile(""
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                   "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
     uint32_t r[16];
     tmem_ld16_start(taddr, r);
     tmem_ld_wait();
+    tmem_landed(r);
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
