@@ -896,8 +896,13 @@ __global__ void __launch_bounds__(kThreads, 1)
 // tensor at two (of 64 channels; four of 32; one of 128) of the nine (dz, dx) shifts.  An MMA's time does
 // not depend on N up to 192, so the wider N is free.  The column operand is unshifted in x and z: a voxel pair
 // counts where both are in the grid, and boxes read zeros outside.
-// 64x64x32, 64 -> 64 channels: 74 -> 27 us; a whole call with the bias gradient 123 -> 61 us.  128x128x64, 32 -> 32: 494
-// -> 161 us; 16x16x8, 256 -> 256: 86 -> 50 us.
+// An FP32 accumulator's error grows with the number of MMAs that it takes one after another.  So the MMAs of a K step go to
+// wgrad_sets(CN) accumulators in turn, as many as TMEM holds, which the epilogue adds; and the voxels are split until no
+// accumulator takes more of them than one of the form above would (wg_row_plan).  With one accumulator and a single wave
+// the error of 256 -> 256 channels on 16x16x8 was 2.4 times that form's, of 96 -> 32 on 128x128x64 2.9 times; now 0.6 and
+// 0.65, and 0.2 to 0.8 on every shape tried.
+// Kernel (ncu), boxes' form -> this: 64x64x32, 64 -> 64 channels 74 -> 27 us; 128x128x64, 32 -> 32 383 -> 116, 96 -> 32
+// 403 -> 348; 32x32x16, 384 -> 128 54 -> 43; 16x16x8, 256 -> 256 22.1 -> 20.4.
 struct WgRowArgs {
     int nx, R, kcy, nchunks, cps;  // rows per K step, steps per plane, steps, steps per split
     int cm, variants, nmb;         // channels per row block, shifts per MMA, channel blocks
@@ -910,11 +915,13 @@ struct WgRowArgs {
     uint64_t timeout_ns;
 };
 
+__host__ __device__ constexpr int wgrad_sets(int cn) { return cn == 64 ? 2 : 4; }
+
 template <int CN>
 __global__ void __launch_bounds__(kThreads, 1)
     conv_wgrad_rows(const __grid_constant__ CUtensorMap tmM, const __grid_constant__ CUtensorMap tmN, const WgRowArgs a) {
-    constexpr int N = 3 * CN;
-    constexpr uint32_t TCOLS = tmem_cols_for(N);
+    constexpr int N = 3 * CN, SETS = wgrad_sets(CN);
+    constexpr uint32_t TCOLS = tmem_cols_for(SETS * N);
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     uint8_t *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);
@@ -993,7 +1000,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t da = (uint32_t)a0 + s * (a.stride >> 4), db = (uint32_t)b0 + s * (a.stride >> 4);
 #pragma unroll 4
             for (int k = 0; k < K; k += 16) {  // 16 voxels on: 16 rows of the operand's bytes
-                mma_bf16(lead, tmem, da, ahi, db, bhi, idesc, (kk > 0 || k > 0) ? 1u : 0u);
+                mma_bf16(lead, tmem + (k / 16 % SETS) * N, da, ahi, db, bhi, idesc, (kk > 0 || k >= 16 * SETS) ? 1u : 0u);
                 da += rowA;
                 db += rowB;
             }
@@ -1014,10 +1021,24 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int v = row / a.cm, c = row % a.cm, sh = vg * a.variants + v;
     const bool valid = ok && v < nv && !flags[0];
     float *out = a.partial + ((int64_t)blockIdx.z * 27 * a.ca + mb * a.cm + c) * a.cb + blockIdx.y * CN;
+    const int nset = min(SETS, K / 16);
 #pragma unroll 1
     for (int c0 = 0; c0 < N; c0 += 16) {
+        uint32_t part[SETS][16];
+#pragma unroll
+        for (int q = 0; q < SETS; ++q)
+            if (q < nset) tmem_ld16_start(tmem + ((uint32_t)(warp * 32) << 16) + q * N + c0, part[q]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int q = 0; q < SETS; ++q) tmem_landed(part[q]);
         float acc[16];
-        tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + c0, acc);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            acc[i] = __uint_as_float(part[0][i]);
+#pragma unroll
+            for (int q = 1; q < SETS; ++q)
+                if (q < nset) acc[i] += __uint_as_float(part[q][i]);
+        }
         if (!valid) continue;
         if (nk == 0) {
 #pragma unroll
@@ -1373,8 +1394,14 @@ WgRowPlan wg_row_plan(ConvVol v, int taps, int ci, int co) {
     p.kcy = (v.ny + p.R - 1) / p.R;
     p.nchunks = p.kcy * v.nz;
     const int ctas = p.groups * p.nmb * p.nnb;
-    const int splits = std::max(1, std::min(p.nchunks, 152 / ctas));  // one CTA per SM
-    p.cps = (p.nchunks + splits - 1) / splits;
+    // One CTA per SM, in as few waves as keep the voxels that an accumulator takes at or below those of the boxes' form.
+    const int64_t most_voxels = (int64_t)wg_plan(v, taps, ci, co).cps * 64;
+    const int sets = wgrad_sets(p.cn), per_step = (v.nx * p.R / 16 + sets - 1) / sets * 16;
+    for (int waves = 1;; ++waves) {
+        const int splits = (int)std::max<int64_t>(1, std::min<int64_t>(p.nchunks, (int64_t)waves * 152 / ctas));
+        p.cps = (p.nchunks + splits - 1) / splits;
+        if (p.cps == 1 || (int64_t)p.cps * per_step <= most_voxels) break;
+    }
     p.splits = (p.nchunks + p.cps - 1) / p.cps;
     p.part_bytes = round256((size_t)p.splits * 27 * ci * co * 4);
     return p;

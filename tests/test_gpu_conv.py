@@ -329,3 +329,25 @@ def test_conv_narrow_layers_input_gradient(rsv, case):
     gb = gxb.float().cpu().double().numpy().reshape(nz, ny, nx, ldgx)
     assert np.array_equal(gb[..., 8:8 + ci], U.bf16_round(got))
     assert np.all(gb[..., :8] == 3) and np.all(gb[..., 8 + ci:] == 3)
+
+
+@pytest.mark.parametrize("case", [(24, 21, 30, 384, 128), (40, 24, 20, 96, 32), (24, 20, 20, 256, 256), (40, 9, 12, 64, 64)],
+                         ids=lambda c: "{}x{}x{}_ci{}_co{}".format(*c))
+def test_conv_wgrad_forms_are_equally_accurate(rsv, case):
+    """The form by whole rows and the one by voxel-major copies (a leading dimension that 16-byte loads cannot take) on the same
+    values: both sum in FP32, whose error grows with the voxels that one accumulator takes.  The rows' form may take no
+    more of them, so its error against 64 bits is no larger, but for a quarter of scatter."""
+    torch = pytest.importorskip("torch")
+    nx, ny, nz, ci, co = case
+    rng = np.random.default_rng(900 + sum(case))
+    x = np.maximum(_vol(rng, nz, ny, nx, ci, ci + 4), 0)
+    gyt, gyh = _bf16(torch, _vol(rng, nz, ny, nx, co))
+    ref = U.conv3_wgrad(gyh, _bf16(torch, x[..., :ci])[1])
+    error = []
+    for ld in (ci, ci + 4):
+        xt, _ = _bf16(torch, x[..., :ld])
+        gw = torch.full((co, 27, ci), float("nan"), device="cuda")
+        st = rsv.rsv_conv3d_wgrad(None, nx, ny, nz, 27, ci, co, _p(xt), ld, _p(gyt), co, _p(gw), None)
+        assert st == rsv.RSV_OK, rsv.status_string(st)
+        error.append(np.linalg.norm(gw.cpu().double().numpy() - ref) / np.linalg.norm(ref))
+    assert error[0] <= 1.25 * error[1], error
