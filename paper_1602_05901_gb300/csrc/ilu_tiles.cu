@@ -35,10 +35,15 @@
 //   through the array with one barrier per step.
 // Measured (one apply = gather + two sweeps; one warp per tile with 36 values per cell and every edge read and
 // wait in that warp -> this form):
-//   256x8x4 (a lone tile) FP32 155 -> 78 us; 100x100x50 FP32 363 -> 183 us; 256x256x128 FP32 1034 -> 905 us;
-//   75x61x37 FP64 865 -> 255 us; 128x128x64 FP64 1580 -> 516 us.
-// What is left of an FP32 apply on 100x100x50: 248 steps of 0.13 us and 24 hand-offs of about 1 us (store,
-// L2, poll) per sweep.  Independent FP32 tiles, 4 per SM, stream at 0.83 of the measured HBM rate.  Also measured:
+//   256x8x4 (a lone tile) FP32 155 -> 76 us; 100x100x50 FP32 360 -> 179 us; 256x256x128 FP32 1031 -> 912 us;
+//   256x8x4 FP64 958 -> 283 us; 75x61x37 FP64 864 -> 256 us; 128x128x64 FP64 1594 -> 518 us.
+// Where a sweep's 85 us go on 100x100x50 in FP32 (169 tiles, times and waits noted by each tile in a build for that;
+// noting them adds 0.02 us per step): the last tile starts after 60 us and runs for 24.  Up to there lie 12 hand-offs in j
+// and 12 in k, each 8 or 4 steps of the tile before and then 1.0 us until the next tile steps (store, L2, poll, halo); a
+// lone tile steps in 0.13 us, tiles in the thick of the wavefront in 0.16 to 0.2, for each waits about 34 times for its
+// neighbours' values, 150 to 500 cycles a time: the edge warp brings at most WIN steps per round trip.  No
+// tile waits for the factor or the input.
+// Independent FP32 tiles, 4 per SM, stream at 0.83 of the measured HBM rate.  Also measured:
 // factor rows by register loads several steps ahead instead of the ring (a lone tile's step 0.36 us instead
 // of 0.13: loads in flight share six scoreboards, and a wait on one waits for younger loads); one service warp for
 // edges and data (hand-off 3 us); edge windows of 8 and 16 steps (100x100x50: 181 and 219 us against 176) and of 2
