@@ -775,7 +775,7 @@ rsv_status rsv_precond_setup(rsv_solver *s, int pc_type, const rsv_pc_params *pa
         // The CPR hierarchy reads the matrix only, and neither chain fills the chip: the factor's planes are short
         // dependent launches, the coarse inverse a few CTAs.  The hierarchy runs on the side stream, issued
         // after a quarter of the planes so that the host keeps ahead of both (128x128x64 FP32: values, setup
-        // and one apply 3.78 -> 3.18 ms).
+        // and one apply 3.78 -> 3.18 ms; 3.35 since the coarse inverse is an LU's, which shares the FP64 pipes with the planes).
         const bool beside = cpr && A->nsys == 1;
         const int np = s->sch.nplanes, first = beside ? np / 4 : np;
         Side side(s);
